@@ -7,7 +7,8 @@
 //                  LN2+FFN1+GELU, FFN2+residual]; then the heads
 //                 (LN_f + n x V logits) and one select kernel (log-softmax,
 //                 top-k, Viterbi, acceptance, slot bookkeeping);
-//   prefill      = the same layer stack over the prompt in chunks of 8 rows.
+//   prefill      = the same layer stack over the prompt: bf16 models in passes of
+//                 up to PREFILL_PASS_ROWS positions, fp32 models 8 rows at a time.
 // Within a pass the kernels are chained with programmatic dependent launch;
 // each (n_heads, top_k) decode step is captured once into a CUDA graph.
 #include <cuda_runtime.h>
@@ -126,9 +127,9 @@ struct mtp_ctx {
     // batched path (bf16 weights; more fed rows than one fused pass takes): tensor-core
     // projections over all rows of a step, row-wise glue kernels, split-KV attention
     bool use_batched = true, batched_ok = false;
-    int bm_max = 0;  // rows of the batched buffers: max_batch * n_heads_max
+    int bm_max = 0;  // rows of the batched buffers (batched_rows)
     uint16_t* d_w2p = nullptr;  // W2 [layers][d][F] as stored in the blob (the fused kernels keep it transposed)
-    float *d_bx = nullptr, *d_bqkv = nullptr, *d_bq = nullptr, *d_bh = nullptr;
+    float *d_bx = nullptr, *d_bq = nullptr;
     float* d_bws = nullptr;  // attention split partials
     int* d_bwc = nullptr;    // attention split counters
     int battn_ws_units = 1;  // (group, split) pairs the attention workspace holds
@@ -539,18 +540,25 @@ int launch_step_pass(mtp_ctx* c, int rows, int rpg, int seq_base, cudaStream_t s
     return MTP_OK;
 }
 
+// Rows of the batched buffers: a decode step's (every slot's fed rows plus a prefill lane of up
+// to PREFILL_ROWS prompt rows), and for bf16 models a whole prefill pass: as many prompt rows as
+// the slots can hold, up to PREFILL_PASS_ROWS.
+int batched_rows(const mtp_ctx* c) {
+    const mtp_config& cf = c->cfg;
+    const long long step = (long long)cf.max_batch * cf.n_heads_max + PREFILL_ROWS;
+    if (c->wbytes != 2) return (int)step;
+    const long long prompts = ((long long)cf.max_batch * cf.max_ctx + 7) / 8 * 8;
+    return (int)std::max(step, std::min<long long>(prompts, PREFILL_PASS_ROWS));
+}
+
 // Buffers and tensor maps of the batched path (bf16 weights only).
 int setup_batched(mtp_ctx* c) {
     const mtp_config& cf = c->cfg;
     const int d = cf.d_model, F = cf.d_ffn, H = cf.n_attn_heads, P = cf.page_size;
-    // every slot's fed rows plus a prefill lane of up to PREFILL_ROWS prompt rows
-    c->bm_max = cf.max_batch * cf.n_heads_max + PREFILL_ROWS;
     if (c->wbytes != 2 || !c->d_w2p) return MTP_OK;
     const size_t M = (size_t)c->bm_max;
     MTP_TRY(c->alloc(&c->d_bx, M * d));
-    MTP_TRY(c->alloc(&c->d_bqkv, M * 3 * d));
     MTP_TRY(c->alloc(&c->d_bq, M * d));
-    MTP_TRY(c->alloc(&c->d_bh, M * F));
     uint16_t *ahi, *alo, *uhi, *ulo;
     MTP_TRY(c->alloc(&ahi, M * d));
     MTP_TRY(c->alloc(&alo, M * d));
@@ -561,10 +569,9 @@ int setup_batched(mtp_ctx* c) {
     c->d_uhi = reinterpret_cast<__nv_bfloat16*>(uhi);
     c->d_ulo = reinterpret_cast<__nv_bfloat16*>(ulo);
     {  // attention workspace for the decode groups (slots, plus the lane's groups of as few as one row)
-        // and the prefill groups (8-row runs)
+        // and the prefill groups (8-row runs; one wave of CTAs where their keys are split)
         const int gd = cf.max_batch + PREFILL_ROWS, gp = (c->bm_max + 7) / 8;
-        c->battn_ws_units = std::max(gd * attn_splits_for(gd, H, P, cf.max_ctx, c->num_sms),
-                                     gp * attn_splits_for(gp, H, P, cf.max_ctx, c->num_sms));
+        c->battn_ws_units = std::max(gd * attn_splits_for(gd, H, P, cf.max_ctx, c->num_sms), c->num_sms / H);
         MTP_TRY(c->alloc(&c->d_bws, attn_workspace_floats(c->battn_ws_units, H, 1, MAX_ROWS)));
         MTP_TRY(c->alloc(&c->d_bwc, (size_t)std::max(gd, gp) * H));
     }
@@ -1246,7 +1253,8 @@ MTP_API int mtp_create(const mtp_config* config, const void* weights_blob, size_
                              sb, sh));
     }
     const int lb = std::max(B, MAX_ROWS);
-    const int row_cap = (B * nm + PREFILL_ROWS + 7) / 8 * 8;  // rows of one pass (slots' rows + the prefill lane)
+    c->bm_max = batched_rows(c);
+    const int row_cap = (c->bm_max + 7) / 8 * 8;  // rows of one pass
     if ((r = c->alloc(&c->d_pe, (size_t)cf.max_ctx * d)) ||
         (r = c->alloc(&c->d_kv, (size_t)c->n_pages * c->page_elems)) ||
         (r = c->alloc(&c->d_block_table, (size_t)B * c->pages_per_seq)) ||
@@ -1432,9 +1440,10 @@ MTP_API int mtp_prefill(mtp_ctx* c, int slot, const int32_t* phonemes, int n_ph,
     MTP_TRY(slot_set(c, slot, 0, 0, max_new_tokens, 0, 1, 0, 0, n_ph));
     Prof* prof = nullptr;
     float* final_x = nullptr;
-    if (c->use_batched && c->batched_ok) {  // chunks of PREFILL_ROWS positions through the batched path
-        for (int p0 = 0; p0 < T; p0 += PREFILL_ROWS) {
-            const int m = (int)std::min<long long>(PREFILL_ROWS, T - p0);
+    if (c->use_batched && c->batched_ok) {  // the whole prompt (or as many positions as a pass holds) at once
+        const int pass = c->bm_max / 8 * 8;
+        for (int p0 = 0; p0 < T; p0 += pass) {
+            const int m = (int)std::min<long long>(pass, T - p0);
             const int rows = (m + 7) / 8 * 8;
             EmbedArgs e = embed_base(c);
             e.mode = 1; e.rows = m; e.slot = slot; e.p0 = p0; e.n_ph = n_ph; e.total = (int)T;
@@ -1498,9 +1507,12 @@ MTP_API int mtp_prefill_pending(mtp_ctx* c) {
     if (!lane_usable(c)) return fail(MTP_ERR_INVALID, "admitted prompts need the batched path");
     const mtp_config& cf = c->cfg;
     cudaStream_t s = c->stream;
-    const int P = c->bm_max / 8 * 8;  // prompt rows per pass, in attention groups of 8 positions
+    const int cap = c->bm_max / 8 * 8;  // prompt rows per pass at most, in attention groups of 8 positions
     int passes = 0;
     while (lane_pending(c)) {
+        long long want = 0;  // rows the admitted slots still need (whole groups): a pass has no empty tail
+        for (int left : c->h_prompt_left) want += left > 0 ? (left + 7) / 8 * 8 : 0;
+        const int P = (int)std::min<long long>(cap, want);
         MTP_TRY(enqueue_lane_plan(c, 0, P, 8, s, c->use_pdl, nullptr));
         MTP_TRY(run_layers_batched(c, P, 8, P / 8, PLAN_ROWS, s, c->use_pdl, nullptr, cf.max_ctx));
         Prof* prof = nullptr;

@@ -1,0 +1,59 @@
+"""Prefill passes (Sec. III-A: the prompt runs through the blocks as one sequence)
+against the oracle at the sizes where a pass can go wrong: fewer rows than an
+attention group, the edges of the 128-row tiles, and prompts or batches of
+prompts just below, at and past the rows one pass holds (4096)."""
+import copy
+
+import numpy as np
+import pytest
+
+import synth
+from oracle.mtp import MTPOracle
+
+from gpu_util import assert_logits_close, decoder, lib_module
+
+pytestmark = pytest.mark.gpu
+
+MODEL = synth.TINY_BF16
+
+
+@pytest.mark.parametrize("length", [1, 7, 9, 127, 129, 257, 1025, 4095, 4097])
+def test_one_prompt(length):
+    ph, ac = synth.make_prompt(300 + length, length // 3, length - length // 3, MODEL.phone_vocab)
+    dec, w = decoder(MODEL, max_batch=1, max_ctx=length + 32)
+    try:
+        dec.prefill(0, ph, ac, 8)
+        dec.decode_step(4, 4)
+        o = MTPOracle(MODEL, w)
+        o.prefill(ph, ac, 8)
+        assert_logits_close(dec.logits(4)[0][0], o.step(4, 4).logits, f"prompt of {length}")
+        assert dec.state(0)["len"] == length
+    finally:
+        dec.close()
+
+
+@pytest.mark.parametrize("lengths,passes", [
+    ([5, 130, 61], 1),
+    ([1000, 1000, 1000, 1000, 96], 1),    # exactly one pass of 4096 rows
+    ([1000, 1000, 1000, 1000, 97], 2),    # one prompt row left for the second pass
+    ([700, 1300, 900, 1100, 500, 33], 2),
+])
+def test_admitted_prompts(lengths, passes):
+    mtp = lib_module()
+    prompts = [synth.make_prompt(320 + b, t // 4, t - t // 4, MODEL.phone_vocab) for b, t in enumerate(lengths)]
+    dec, w = decoder(MODEL, max_batch=len(lengths), max_ctx=max(lengths) + 32)
+    try:
+        for b, (ph, ac) in enumerate(prompts):
+            dec.admit(b, ph, ac, 8)
+        assert mtp.mtp_prefill_pending(dec.ctx) == passes
+        dec.decode_step(4, 4)
+        lg = dec.logits(4)[0]
+        first = MTPOracle(MODEL, w)
+        for b, (ph, ac) in enumerate(prompts):
+            o = copy.copy(first)
+            o.prefill(ph, ac, 8)
+            assert_logits_close(lg[b], o.step(4, 4).logits, f"slot {b}")
+            assert dec.state(b)["len"] == lengths[b]
+    finally:
+        dec.close()
+    assert np.isfinite(lg).all()
