@@ -346,6 +346,12 @@ int tc_encode_2d(CUtensorMap* map, const void* base, uint64_t inner, uint64_t ro
                  bool pre_swizzled);
 int tc_tile_rows(int m);          // activation rows per tile for m rows: 32, 64 or 128
 cudaError_t launch_tc_gemm(const TcGemm& g, cudaStream_t s, bool pdl);
+// The same products over many rows by a persistent kernel of CTA pairs (tc_gemm_pair.cu): tiles of
+// 256 weight rows x 256 activation rows, one K split, g.nt = 128 (activation boxes of 128 rows).
+// tc_gemm_pair_fits: whether it is the faster of the two for m rows and k_chunks 64-wide chunks of K,
+// which launch_tc_gemm would cut into `splits`.
+bool tc_gemm_pair_fits(int n_w, int m, int k_chunks, int splits, int num_sms);
+cudaError_t launch_tc_gemm_pair(const TcGemm& g, int num_sms, cudaStream_t s, bool pdl);
 constexpr int TC_CLUSTER_SPLITS = 4;  // K splits one cluster sums in the batched path (clusters of 8 at one CTA per
                                       // SM: only 15 fit this GPU at once)
 

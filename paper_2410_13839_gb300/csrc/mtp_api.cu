@@ -377,6 +377,8 @@ int run_layers_batched(mtp_ctx* c, int M, int rpg, int groups, int plan, cudaStr
             } else {  // accumulated outputs: K splits added by atomics
                 g.splits = epilogue == TC_ACCUM ? gemm_splits(c, n_w, k, ntiles) : 1;
             }
+            const bool pairs = tc_gemm_pair_fits(n_w, M, k / 64, g.splits, c->num_sms);
+            if (pairs) g.splits = sc = 1;
             TcGemmArgs& ga = g.args;
             ga.cluster_reduce = sc;
             ga.out = out; ga.ldo = ldo; ga.bias = bias; ga.m = M;
@@ -388,7 +390,7 @@ int run_layers_batched(mtp_ctx* c, int M, int rpg, int groups, int plan, cudaStr
             ga.block_table = c->d_block_table; ga.bt_stride = c->pages_per_seq;
             ga.pack_hi = c->d_uhi; ga.pack_lo = c->d_ulo;
             ga.trace = tslot(c, MTP_K_GEMM);
-            LAUNCH(MTP_K_GEMM, launch_tc_gemm(g, s, pdl));
+            LAUNCH(MTP_K_GEMM, pairs ? launch_tc_gemm_pair(g, c->num_sms, s, pdl) : launch_tc_gemm(g, s, pdl));
             return MTP_OK;
         };
         // LN1 -> q|k|v: queries out, keys and values appended to the cache

@@ -475,6 +475,15 @@ extern "C" MTP_API int mtp_gemm_bf16x2(const void* w, const void* a_hi, const vo
     g.args.k_chunks = k / TC_K / splits;
     g.args.w_rows_per_kchunk = 0;
     g.args.epilogue = accumulate ? TC_ACCUM : TC_STORE;
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return gemm_fail(MTP_ERR_CUDA, "mtp_gemm_bf16x2: no usable CUDA device");
+    const bool pairs = tc_gemm_pair_fits(n_w, m, k / TC_K, splits, sms);  // many rows: tiles of CTA pairs
+    if (pairs) {  // whole-K tiles: nothing is added by another CTA
+        g.splits = 1;
+        g.args.k_chunks = k / TC_K;
+    }
     int* d_err = nullptr;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if (cudaMallocAsync(&d_err, sizeof(int), st) != cudaSuccess)
@@ -487,7 +496,7 @@ extern "C" MTP_API int mtp_gemm_bf16x2(const void* w, const void* a_hi, const vo
         tc_encode_2d(&g.a_lo, a_lo, (uint64_t)k, (uint64_t)m, (uint32_t)g.nt, false)) {
         rc = gemm_fail(MTP_ERR_INVALID, "mtp_gemm_bf16x2: tensor map encoding failed (alignment?)");
     } else {
-        const cudaError_t e = launch_tc_gemm(g, st, false);
+        const cudaError_t e = pairs ? launch_tc_gemm_pair(g, sms, st, false) : launch_tc_gemm(g, st, false);
         if (e != cudaSuccess) rc = report_error(MTP_ERR_CUDA, cudaGetErrorString(e));
     }
     int h_err = 0;

@@ -57,3 +57,19 @@ def test_tc_gemm_rejects_bad_shapes():
     w = torch.zeros(128, 64, device="cuda", dtype=torch.bfloat16)
     with pytest.raises(mtp.MTPError):
         mtp.mtp_gemm_bf16x2(w, a, a, out, 128, 64, 4, 2, 1)   # one k-chunk cannot split in two
+
+
+PAIR_CASES = [  # many rows: 256 x 256 tiles of CTA pairs, where they are enough to fill the GPU
+    (4096, 1024, 640, 1, 0),      # ragged last activation tile (half a tile)
+    (3072, 1024, 1025, 1, 0),     # one row in the last tile
+    (1024, 1024, 2500, 4, 1),     # accumulate; ragged
+    (1024, 4096, 4096, 8, 1),     # the largest row count, long K
+    (2560, 64, 2048, 1, 0),       # one k-chunk per tile
+    (4096, 192, 4000, 1, 0),      # fewer chunks than ring stages, several tiles per pair
+    (768, 256, 4096, 1, 0),       # the tiny model's q|k|v
+]
+
+
+@pytest.mark.parametrize("n_w,k,m,splits,accumulate", PAIR_CASES)
+def test_pair_gemm_matches_fp64_product(n_w, k, m, splits, accumulate):
+    test_tc_gemm_matches_fp32_product(n_w, k, m, splits, accumulate)
