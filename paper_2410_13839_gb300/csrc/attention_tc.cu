@@ -5,25 +5,34 @@
 //
 // Grid (split, head, tile).  A tile is 128 rows of the pass, the MMA's M side
 // and the 128 TMEM lanes; its rows may belong to several slots (a prefill pass
-// packs the prompts of many slots).  Each distinct slot of the tile is a
-// segment; the segment's keys 0 .. (its largest position) are cut into items
-// of 128 keys, and split s takes items s, s + S, ... of every segment.  Per
-// item, with the cached keys and values of the item's pages copied by
+// packs the prompts of many slots).  Each run of consecutive rows of one slot
+// is a segment; the segment's keys 0 .. (its largest position) are cut into
+// items of 128 keys, and split s takes items s, s + S, ... of every segment.
+// Per item, with the cached keys and values of the item's pages copied by
 // cp.async.bulk into a two-stage ring (the cache stores chunk c of key row t
 // at c ^ (t & 7): exactly the 128-byte-swizzled tile the MMA reads):
 //
 //   S  = (Q_hi + Q_lo) K^T       two MMAs per 16 dims, 128 x 128 fp32 in TMEM
-//   P  = exp(S - m_new)          one thread per row (TMEM lane), masked to the
-//                                row's own slot and keys <= its position,
-//                                written to shared memory as bf16 hi + lo
-//   O' = (P_hi + P_lo) V         two MMAs per 16 keys, 128 x 64 fp32 in TMEM
-//                                (V read as an MN-major operand)
-//   o  = o * exp(m - m_new) + O' in registers (online softmax)
+//   P  = 2^(S log2 e - m)        one thread per row (TMEM lane), masked to the
+//                                segment's rows and keys <= the row's position;
+//                                written to TMEM as bf16 hi + lo, 64 keys at a time
+//   O += (P_hi + P_lo) V         two MMAs per 16 keys with P read from TMEM,
+//                                128 x 64 fp32 accumulated in TMEM (V read as
+//                                an MN-major operand)
 //
+// m is a row's running reference, not always its maximum: it moves (and the
+// row's O and sum are rescaled) only when the maximum has grown by more than
+// 2^8, so most items leave O alone; the result does not depend on it.
+//
+// What bounds it: the softmax's instructions, about 10 per score with one warp
+// per scheduler and CTA.  S is read into registers at once, so the next item's
+// S = Q K^T runs under this one's softmax, P V of each half under the other
+// half's, and two CTAs share an SM (97 KB of shared memory, 256 TMEM columns
+// each).
 // Q and P enter as bf16 hi + lo pairs (hi + lo = x to about 2^-16 relative),
 // so the products keep fp32 accuracy; the keys and values are the cache's bf16.
 // One elected thread of the fifth warp issues the copies and the MMAs; the
-// four other warps own one row each per thread.  Splits leave (max, sum,
+// four other warps own one row each per thread.  Splits leave (reference, sum,
 // unnormalised output) per row in the workspace and the CTA that finishes
 // last merges them (an atomic counter per tile and head, reset by that CTA).
 #include <math.h>
@@ -40,46 +49,68 @@ namespace {
 
 constexpr int PA_ROWS = 128;     // query rows per tile: MMA M, TMEM lanes
 constexpr int PA_KEYS = 128;     // keys per item: N of Q K^T, K of P V
+constexpr int PA_SPLIT_ITEMS = 4;  // fewest items of a key split (a split costs its partials and their merge)
 constexpr int PA_THREADS = 160;  // four row warps + the issuing warp
 constexpr int PA_PART = 4 + HEAD_DIM;  // (max, sum, -, -, out[64]): out 16-byte aligned for float4 access
 constexpr uint32_t PA_TILE = PA_ROWS * 128;  // 128 rows of 128 bytes
-// shared memory (1024-byte aligned): Q hi | Q lo | P hi (keys 0-63, 64-127) |
-// P lo (same) | stage 0 K | stage 0 V | stage 1 K | stage 1 V
-constexpr uint32_t OFF_Q = 0, OFF_P = 2 * PA_TILE, OFF_KV = 6 * PA_TILE;
-constexpr uint32_t PA_SMEM = 10 * PA_TILE + 1024;
-constexpr uint32_t TM_S = 0, TM_O = 128, TM_COLS = 256;  // TMEM columns: S [128), O' double-buffered [64) x 2
+// shared memory (1024-byte aligned): Q hi | Q lo | stage 0 K | V | stage 1 K | V
+constexpr uint32_t OFF_Q = 0, OFF_KV = 2 * PA_TILE;
+constexpr uint32_t PA_SMEM = 6 * PA_TILE + 1024;
+constexpr int PA_HALF = PA_KEYS / 2;  // keys whose weights P holds at a time
+// TMEM columns: S [128) | P hi [32) | P lo [32) of half an item | O [64)
+constexpr uint32_t TM_S = 0, TM_P = 128, TM_PLO = TM_P + PA_HALF / 2, TM_O = 192, TM_COLS = 256;
+constexpr float LOG2E = 1.4426950408889634f;
+constexpr float RESCALE = 8.f;  // growth of a row's maximum (log2) that moves its reference
+
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// D = A B (+ D) with A (bf16, K-major) read from TMEM: lane = row, two K elements per column
+__device__ __forceinline__ void tc_mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
+                                          uint32_t acc) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(acc)
+        : "memory");
+}
+// 16 consecutive 32-bit columns of this warp's 32 TMEM lanes (thread i: lane i)
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16]) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
+        "%15, %16};" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]),
+        "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// (x0, x1) as one register of bf16 hi parts and one of bf16 lo parts (x0 in the low half)
+__device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& hi, uint32_t& lo) {
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(x0 - bf16_lo(hi), x1 - bf16_hi(hi));
+    lo = *reinterpret_cast<const uint32_t*>(&l);
+}
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
-// x0..x7 as 16 bytes of bf16 hi and 16 bytes of bf16 lo
-__device__ __forceinline__ void split8(const float* x, uint4& hi, uint4& lo) {
-    uint32_t h[4], l[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const __nv_bfloat16 h0 = __float2bfloat16_rn(x[2 * q]), h1 = __float2bfloat16_rn(x[2 * q + 1]);
-        const __nv_bfloat16 l0 = __float2bfloat16_rn(x[2 * q] - __bfloat162float(h0));
-        const __nv_bfloat16 l1 = __float2bfloat16_rn(x[2 * q + 1] - __bfloat162float(h1));
-        h[q] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-        l[q] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
-    }
-    hi = make_uint4(h[0], h[1], h[2], h[3]);
-    lo = make_uint4(l[0], l[1], l[2], l[3]);
-}
-
-__global__ void __launch_bounds__(PA_THREADS, 1) attn_tc_kernel(const AttnArgs a) {
+__global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a) {
     extern __shared__ __align__(1024) unsigned char pa_raw[];
-    __shared__ uint64_t kv_full[2], kv_empty[2], s_full, p_full, o_full[2], done;
+    __shared__ uint64_t kv_full[2], s_full, s_read, p_full[2], pv_done[2];  // p, pv: the item's halves
     __shared__ uint32_t tmem_base;
-    __shared__ int s_seq[PA_ROWS], s_pos[PA_ROWS];
-    __shared__ int seg_slot[PA_ROWS], seg_kmax[PA_ROWS];
-    __shared__ int s_nseg, s_abort, s_last;
+    __shared__ int s_seq[PA_ROWS];
+    __shared__ int seg_slot[PA_ROWS], seg_kmax[PA_ROWS];  // runs of consecutive rows of one slot
+    __shared__ int s_heads[PA_ROWS / 32];                 // run starts per warp
+    __shared__ int s_abort, s_last;
     unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(pa_raw) + 1023) & ~(uintptr_t)1023);
     TraceEnd trace_guard(a.trace);
     const int sp = blockIdx.x, h = blockIdx.y, tile = blockIdx.z;
     const int S = a.n_splits, H = a.n_heads, P = a.page_size;
-    const int tid = threadIdx.x, warp = tid >> 5;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int row0 = tile * PA_ROWS;
 
     // ---- independent of the previous kernel ----
@@ -88,20 +119,22 @@ __global__ void __launch_bounds__(PA_THREADS, 1) attn_tc_kernel(const AttnArgs a
         tmem_relinquish();
     }
     if (tid == 0) {
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&kv_full[i], 1);
-            mbar_init(&kv_empty[i], 1);
-            mbar_init(&o_full[i], 1);
-        }
+        mbar_init(&kv_full[0], 1);
+        mbar_init(&kv_full[1], 1);
         mbar_init(&s_full, 1);
-        mbar_init(&p_full, PA_ROWS);
-        mbar_init(&done, 1);
+        mbar_init(&s_read, PA_ROWS / 32);  // one arrival per row warp
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&p_full[i], PA_ROWS / 32);
+            mbar_init(&pv_done[i], 1);
+        }
         fence_barrier_init();
         s_abort = 0;
     }
-    {  // keys and values past a segment's pages are read as zeros times zero weights: keep them finite
-        uint4* kv = reinterpret_cast<uint4*>(sm + OFF_KV);
-        for (int i = tid; i < (int)(4 * PA_TILE / 16); i += PA_THREADS) kv[i] = make_uint4(0u, 0u, 0u, 0u);
+    // values past a segment's pages enter with weight zero: keep them finite (scores of such keys are
+    // masked by selection)
+    for (int st = 0; st < 2; ++st) {
+        uint4* v = reinterpret_cast<uint4*>(sm + OFF_KV + (uint32_t)(2 * st + 1) * PA_TILE);
+        for (int i = tid; i < (int)(PA_TILE / 16); i += PA_THREADS) v[i] = make_uint4(0u, 0u, 0u, 0u);
     }
     fence_proxy_async();
     tc_fence_before();
@@ -112,59 +145,38 @@ __global__ void __launch_bounds__(PA_THREADS, 1) attn_tc_kernel(const AttnArgs a
     pdl_wait();
     trace_wait(a.trace);
 
-    // ---- the tile's rows, segments and this split's items ----
+    // ---- the tile's rows and their runs ----
+    int my_seq = -1, my_pos = -1;
     if (tid < PA_ROWS) {
         const int r = row0 + tid;
-        const int rs = r < a.rows ? a.row_seq[r] : -1;
-        s_seq[tid] = rs;
-        s_pos[tid] = rs >= 0 ? a.row_pos[r] : -1;
+        if (r < a.rows) {  // one round of independent loads
+            my_seq = a.row_seq[r];
+            my_pos = a.row_pos[r];
+        }
+        s_seq[tid] = my_seq;
+        seg_kmax[tid] = 0;
     }
     __syncthreads();
-    if (tid == 0) {
-        int nseg = 0;
-        for (int r = 0; r < PA_ROWS; ++r) {
-            const int q = s_seq[r];
-            if (q < 0) continue;
-            int g = 0;
-            while (g < nseg && seg_slot[g] != q) ++g;
-            if (g == nseg) {
-                seg_slot[g] = q;
-                seg_kmax[g] = 0;
-                ++nseg;
-            }
-            seg_kmax[g] = max(seg_kmax[g], s_pos[r] + 1);
-        }
-        s_nseg = nseg;
-    }
-    // ---- Q of this head: rows pre-scaled by 1/sqrt(64), bf16 hi | lo, swizzled ----
+    bool head = false;
+    unsigned heads = 0;
     if (tid < PA_ROWS) {
-        const int r = row0 + tid;
-        const bool on = s_seq[tid] >= 0;
-        unsigned char* qhi = sm + OFF_Q + tid * 128;
-        unsigned char* qlo = qhi + PA_TILE;
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-            float x[8];
-            if (on) {
-                const float4* src = reinterpret_cast<const float4*>(a.q + (size_t)r * a.ldq + h * HEAD_DIM + c * 8);
-                const float4 u = src[0], v = src[1];
-                x[0] = u.x * 0.125f; x[1] = u.y * 0.125f; x[2] = u.z * 0.125f; x[3] = u.w * 0.125f;
-                x[4] = v.x * 0.125f; x[5] = v.y * 0.125f; x[6] = v.z * 0.125f; x[7] = v.w * 0.125f;
-            } else {
-#pragma unroll
-                for (int e = 0; e < 8; ++e) x[e] = 0.f;
-            }
-            uint4 hi, lo;
-            split8(x, hi, lo);
-            const int at = (c ^ (tid & 7)) << 4;
-            *reinterpret_cast<uint4*>(qhi + at) = hi;
-            *reinterpret_cast<uint4*>(qlo + at) = lo;
-        }
+        head = my_seq >= 0 && (tid == 0 || s_seq[tid - 1] != my_seq);
+        heads = __ballot_sync(FULL_MASK, head);
+        if (lane == 0) s_heads[warp] = __popc(heads);
     }
-    fence_proxy_async();  // Q is read by the tensor cores
+    __syncthreads();
+    int nseg = 0, my_seg = -1;
+#pragma unroll
+    for (int w = 0; w < PA_ROWS / 32; ++w) {
+        if (w == warp) my_seg = nseg + __popc(heads & (0xffffffffu >> (31 - lane))) - 1;  // run of this row
+        nseg += s_heads[w];
+    }
+    if (tid < PA_ROWS && my_seq >= 0) {
+        if (head) seg_slot[my_seg] = my_seq;
+        atomicMax(&seg_kmax[my_seg], my_pos + 1);
+    }
     __syncthreads();
     // this split's items in order: segment g, key tiles j = sp, sp + S, ... below the segment's end
-    const int nseg = s_nseg;
     auto skip_empty = [&](int2 t) {
         while (t.x < nseg && t.y * PA_KEYS >= seg_kmax[t.x]) {
             ++t.x;
@@ -178,101 +190,157 @@ __global__ void __launch_bounds__(PA_THREADS, 1) attn_tc_kernel(const AttnArgs a
     };
     const int2 first = skip_empty(make_int2(0, sp));
 
-    const long long kv_head = (long long)h * P * HEAD_DIM, v_off = (long long)H * P * HEAD_DIM;
-    // copies of item i into stage i & 1: the pages of keys [128 j, 128 j + 128) below the segment's end
-    auto stage_item = [&](int i, int2 t) {
-        const int g = t.x, j = t.y;
-        const int seq = seg_slot[g];
-        const int k0 = j * PA_KEYS, k1 = min(k0 + PA_KEYS, seg_kmax[g]);
-        const uint32_t blk = (uint32_t)P * 128;
-        unsigned char* ks = sm + OFF_KV + (uint32_t)(i & 1) * 2 * PA_TILE;
-        // pages past the slot's table row count as unreserved
-        auto page_of = [&](int p) { return p < a.bt_stride ? a.block_table[(size_t)seq * a.bt_stride + p] : -1; };
-        uint32_t bytes = 0;
-        for (int p = k0 / P; p * P < k1; ++p)
-            if (page_of(p) >= 0) bytes += 2 * blk;
-        mbar_arrive_expect_tx(&kv_full[i & 1], bytes);
-        for (int p = k0 / P; p * P < k1; ++p) {
-            const int phys = page_of(p);
-            if (phys < 0) {  // unreserved page: report, never read
-                if (a.err) atomicOr(a.err, ERR_BOUNDS);
-                continue;
-            }
-            const __nv_bfloat16* base = a.kv_pool + (long long)phys * a.page_elems + a.layer_off + kv_head;
-            const uint32_t at = (uint32_t)(p * P - k0) * 128;
-            bulk_copy_g2s(ks + at, base, blk, &kv_full[i & 1]);
-            bulk_copy_g2s(ks + PA_TILE + at, base + v_off, blk, &kv_full[i & 1]);
-        }
-    };
-
-    float m_run = -INFINITY, l_run = 0.f, o[HEAD_DIM];
-#pragma unroll
-    for (int c = 0; c < HEAD_DIM; ++c) o[c] = 0.f;
-
-    if (tid == PA_ROWS) {  // ---- the issuing thread: copies and MMAs ----
+    float m_run = -INFINITY, l_run = 0.f;  // m_run in log2 units
+    int items = 0;
+    bool fine = true;
+    if (warp == 4) {  // ---- the issuing warp: copies (a lane per page) and MMAs (lane 0) ----
         constexpr uint32_t IDESC_S = f16_idesc(PA_ROWS, PA_KEYS, false);
         constexpr uint32_t IDESC_O = f16_idesc(PA_ROWS, HEAD_DIM, true);
         const uint32_t q_hi = smem_addr(sm + OFF_Q), q_lo = q_hi + PA_TILE;
-        const uint32_t p_hi = smem_addr(sm + OFF_P), p_lo = p_hi + 2 * PA_TILE;
-        bool staged[2] = {false, false};
+        const long long kv_head = (long long)h * P * HEAD_DIM, v_off = (long long)H * P * HEAD_DIM;
+        // lane q: page q of the item (-2: none; -1: unreserved, as are pages past the slot's table row)
+        auto item_page = [&](int2 t) {
+            if (t.x >= nseg) return -2;
+            const int p = t.y * (PA_KEYS / P) + lane;
+            if (lane >= PA_KEYS / P || p * P >= seg_kmax[t.x]) return -2;
+            return p < a.bt_stride ? max(-1, a.block_table[(size_t)seg_slot[t.x] * a.bt_stride + p]) : -1;
+        };
+        // copies of item i into stage i & 1
+        auto stage_item = [&](int i, int page) {
+            const uint32_t blk = (uint32_t)P * 128;
+            uint64_t* bar = &kv_full[i & 1];
+            unsigned char* ks = sm + OFF_KV + (uint32_t)(i & 1) * 2 * PA_TILE + (uint32_t)(lane * P) * 128;
+            const unsigned have = __ballot_sync(FULL_MASK, page >= 0);
+            if (lane == 0) mbar_arrive_expect_tx(bar, 2 * blk * __popc(have));
+            __syncwarp();
+            if (page >= 0) {
+                const __nv_bfloat16* base = a.kv_pool + (long long)page * a.page_elems + a.layer_off + kv_head;
+                bulk_copy_g2s(ks, base, blk, bar);
+                bulk_copy_g2s(ks + PA_TILE, base + v_off, blk, bar);
+            } else if (page == -1 && a.err) {  // unreserved page: report, never read
+                atomicOr(a.err, ERR_BOUNDS);
+            }
+        };
+        auto wait = [&](uint64_t* bar, uint32_t parity) {  // one lane polls
+            return __all_sync(FULL_MASK, lane != 0 || mbar_wait(bar, parity, a.err)) != 0;
+        };
+        int staged = 0;  // items staged so far
+        int2 ahead = first;
+        {
+            const int p0 = item_page(ahead);
+            const bool any0 = ahead.x < nseg;
+            ahead = any0 ? next_item(ahead) : ahead;
+            const int p1 = item_page(ahead);
+            if (any0) stage_item(staged++, p0);
+            if (ahead.x < nseg) {
+                stage_item(staged++, p1);
+                ahead = next_item(ahead);
+            }
+        }
+        int ahead_page = item_page(ahead);
+        asm volatile("bar.sync 1, %0;" ::"n"(PA_THREADS) : "memory");  // Q is in shared memory
         bool ok = true;
-        if (first.x < nseg) {
-            stage_item(0, first);
-            staged[0] = true;
+        auto issue_s = [&](int i) {  // S of item i, once its keys are in
+            ok = wait(&kv_full[i & 1], (uint32_t)(i >> 1) & 1);
+            if (!ok) return;
+            tc_fence_after();
+            if (lane == 0) {
+                const uint32_t kb = smem_addr(sm + OFF_KV + (uint32_t)(i & 1) * 2 * PA_TILE);
+#pragma unroll
+                for (int kk = 0; kk < HEAD_DIM / 16; ++kk) {
+                    const uint64_t bk = sw128_desc(kb + kk * 32);
+                    tc_mma(tmem + TM_S, sw128_desc(q_hi + kk * 32), bk, IDESC_S, kk != 0);
+                    tc_mma(tmem + TM_S, sw128_desc(q_lo + kk * 32), bk, IDESC_S, 1u);
+                }
+                tc_commit(&s_full);
+            }
+            __syncwarp();
+        };
+        int i = 0, s_issued = 0, pv_issued = 0;
+        if (staged > 0) {
+            issue_s(0);
+            s_issued = ok;
         }
-        int i = 0;
-        for (int2 t = first; t.x < nseg; t = next_item(t), ++i) {
-            const int st = i & 1;
-            const int2 t1 = next_item(t);
-            if (t1.x < nseg) {  // item i - 1 held the other stage: its MMAs must be done
-                if (i >= 1) ok = mbar_wait(&kv_empty[st ^ 1], (uint32_t)((i - 1) >> 1) & 1, a.err);
+        for (int2 t = first; ok && t.x < nseg; ++i) {
+            t = next_item(t);
+            // S has been read into registers: the next item's overwrites it
+            ok = wait(&s_read, (uint32_t)i & 1);
+            if (!ok) break;
+            if (t.x < nseg) {
+                issue_s(i + 1);
                 if (!ok) break;
-                stage_item(i + 1, t1);
-                staged[st ^ 1] = true;
+                ++s_issued;
             }
-            ok = mbar_wait(&kv_full[st], (uint32_t)(i >> 1) & 1, a.err);
-            if (!ok) break;
-            staged[st] = false;
-            tc_fence_after();
-            const uint32_t kb = smem_addr(sm + OFF_KV + (uint32_t)st * 2 * PA_TILE), vb = kb + PA_TILE;
+            const uint32_t vb = smem_addr(sm + OFF_KV + (uint32_t)(2 * (i & 1) + 1) * PA_TILE);
 #pragma unroll
-            for (int kk = 0; kk < HEAD_DIM / 16; ++kk) {
-                const uint64_t bk = sw128_desc(kb + kk * 32);
-                tc_mma(tmem + TM_S, sw128_desc(q_hi + kk * 32), bk, IDESC_S, kk != 0);
-                tc_mma(tmem + TM_S, sw128_desc(q_lo + kk * 32), bk, IDESC_S, 1u);
-            }
-            tc_commit(&s_full);
-            ok = mbar_wait(&p_full, (uint32_t)i & 1, a.err);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t od = tmem + TM_O + (uint32_t)st * HEAD_DIM;
+            for (int half = 0; half < 2; ++half) {
+                ok = wait(&p_full[half], (uint32_t)i & 1);
+                if (!ok) break;
+                tc_fence_after();
+                if (lane == 0) {
 #pragma unroll
-            for (int kk = 0; kk < PA_KEYS / 16; ++kk) {
-                const uint32_t pa = (uint32_t)(kk >> 2) * PA_TILE + (uint32_t)(kk & 3) * 32;
-                const uint64_t bv = sw128_mn_desc(vb + kk * 2048);
-                tc_mma(od, sw128_desc(p_hi + pa), bv, IDESC_O, kk != 0);
-                tc_mma(od, sw128_desc(p_lo + pa), bv, IDESC_O, 1u);
+                    for (int kk = 0; kk < PA_HALF / 16; ++kk) {
+                        const uint64_t bv = sw128_mn_desc(vb + (half * (PA_HALF / 16) + kk) * 2048);
+                        tc_mma_ta(tmem + TM_O, tmem + TM_P + kk * 8, bv, IDESC_O, (i | half | kk) != 0);
+                        tc_mma_ta(tmem + TM_O, tmem + TM_PLO + kk * 8, bv, IDESC_O, 1u);
+                    }
+                    tc_commit(&pv_done[half]);
+                }
+                __syncwarp();
+                ++pv_issued;
             }
-            tc_commit(&o_full[st]);
-            tc_commit(&kv_empty[st]);
+            if (!ok) break;
+            if (ahead.x < nseg) {  // this item's stage is free once its MMAs have read it
+                ok = wait(&pv_done[1], (uint32_t)i & 1);
+                if (!ok) break;
+                stage_item(staged++, ahead_page);
+                ahead = next_item(ahead);
+                ahead_page = item_page(ahead);
+            }
         }
-        if (!ok) s_abort = 1;
-        tc_commit(&done);  // every MMA issued above has completed
-        mbar_wait(&done, 0, nullptr);
-        for (int st = 0; st < 2; ++st)  // copies still in flight land before the CTA leaves
-            if (staged[st]) mbar_wait(&kv_full[st], (uint32_t)((i + (st != (i & 1))) >> 1) & 1, nullptr);
-    } else if (tid < PA_ROWS) {  // ---- one row per thread: softmax and accumulation ----
-        const int my_seq = s_seq[tid], my_pos = s_pos[tid];
-        const uint32_t lane_base = (uint32_t)(warp * 32) << 16;
-        unsigned char* prow_hi = sm + OFF_P + tid * 128;
-        unsigned char* prow_lo = prow_hi + 2 * PA_TILE;
-        int i = 0;
-        for (int2 t = first; t.x < nseg; t = next_item(t), ++i) {
-            const bool in = my_seq >= 0 && seg_slot[t.x] == my_seq;
-            const int k0 = t.y * PA_KEYS;
-            // warp-uniform decisions: tcgen05.ld is issued by whole warps
-            if (!__all_sync(FULL_MASK, mbar_wait(&s_full, (uint32_t)i & 1, a.err))) {
+        if (!ok && lane == 0) {
+            s_abort = 1;
+            // copies still in flight land, and issued MMAs end (bounded), before the CTA leaves
+            for (int j = s_issued; j < staged; ++j) mbar_wait(&kv_full[j & 1], (uint32_t)(j >> 1) & 1, nullptr);
+            const int half = pv_issued & 1;  // the next commit to come on this barrier follows every MMA
+            tc_commit(&pv_done[half]);
+            mbar_wait(&pv_done[half], (uint32_t)(pv_issued >> 1) & 1, nullptr);
+        }
+        __syncwarp();
+    } else {  // ---- one row per thread: Q, then softmax ----
+        {
+            // Q of this head: rows pre-scaled by 1/sqrt(64), bf16 hi | lo, swizzled; 16 lanes per row, every
+            // load issued before any is used
+            constexpr int PER = PA_ROWS * (HEAD_DIM / 4) / PA_ROWS;
+            float4 x[PER];
+#pragma unroll
+            for (int u = 0; u < PER; ++u) {
+                const int q = (tid >> 4) + u * (PA_ROWS / 16), c4 = tid & 15;
+                x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (s_seq[q] >= 0)
+                    x[u] = *reinterpret_cast<const float4*>(a.q + (size_t)(row0 + q) * a.ldq + h * HEAD_DIM + c4 * 4);
+            }
+#pragma unroll
+            for (int u = 0; u < PER; ++u) {
+                const int q = (tid >> 4) + u * (PA_ROWS / 16), c4 = tid & 15;
+                uint2 hi, lo;
+                split_pair(x[u].x * 0.125f, x[u].y * 0.125f, hi.x, lo.x);
+                split_pair(x[u].z * 0.125f, x[u].w * 0.125f, hi.y, lo.y);
+                unsigned char* at = sm + OFF_Q + q * 128 + (((c4 >> 1) ^ (q & 7)) << 4) + (c4 & 1) * 8;
+                *reinterpret_cast<uint2*>(at) = hi;
+                *reinterpret_cast<uint2*>(at + PA_TILE) = lo;
+            }
+        }
+        fence_proxy_async();  // Q is read by the tensor cores
+        asm volatile("bar.sync 1, %0;" ::"n"(PA_THREADS) : "memory");
+        const uint32_t base = tmem + ((uint32_t)(warp * 32) << 16);
+        for (int2 t = first; t.x < nseg; t = next_item(t), ++items) {
+            // keys of the item this row sees: columns 0 .. lim
+            const int lim = my_seq >= 0 && t.x == my_seg ? my_pos - t.y * PA_KEYS : -1;
+            // one lane polls (a poll costs every polling thread); tcgen05.ld is issued by whole warps
+            if (!__all_sync(FULL_MASK, lane != 0 || mbar_wait(&s_full, (uint32_t)items & 1, a.err))) {
                 s_abort = 1;
+                fine = false;
                 break;
             }
             tc_fence_after();
@@ -280,48 +348,92 @@ __global__ void __launch_bounds__(PA_THREADS, 1) attn_tc_kernel(const AttnArgs a
 #pragma unroll
             for (int c0 = 0; c0 < PA_KEYS; c0 += 32) {
                 float v[32];
-                tmem_ld32(tmem + lane_base + TM_S + c0, v);
+                tmem_ld32(base + TM_S + c0, v);
 #pragma unroll
-                for (int e = 0; e < 32; ++e) sv[c0 + e] = (in && k0 + c0 + e <= my_pos) ? v[e] : -INFINITY;
+                for (int e = 0; e < 32; ++e) sv[c0 + e] = v[e];
             }
-            float tmax = -INFINITY;
+            if (!__all_sync(FULL_MASK, lim >= PA_KEYS - 1)) {
 #pragma unroll
-            for (int c = 0; c < PA_KEYS; ++c) tmax = fmaxf(tmax, sv[c]);
-            const float m_new = fmaxf(m_run, tmax);
-            const float corr = m_new == -INFINITY ? 1.f : (m_run == -INFINITY ? 0.f : expf(m_run - m_new));
-            float psum = 0.f;
-#pragma unroll
-            for (int c8 = 0; c8 < PA_KEYS / 8; ++c8) {
-                float pv[8];
-#pragma unroll
-                for (int e = 0; e < 8; ++e) {
-                    const float x = sv[c8 * 8 + e];
-                    pv[e] = x == -INFINITY ? 0.f : expf(x - m_new);
-                }
-                psum += ((pv[0] + pv[1]) + (pv[2] + pv[3])) + ((pv[4] + pv[5]) + (pv[6] + pv[7]));
-                uint4 hi, lo;
-                split8(pv, hi, lo);
-                const uint32_t at = (uint32_t)(c8 >> 3) * PA_TILE + ((uint32_t)((c8 & 7) ^ (tid & 7)) << 4);
-                *reinterpret_cast<uint4*>(prow_hi + at) = hi;
-                *reinterpret_cast<uint4*>(prow_lo + at) = lo;
+                for (int c = 0; c < PA_KEYS; ++c) sv[c] = c <= lim ? sv[c] : -INFINITY;
             }
-            l_run = l_run * corr + psum;
-            m_run = m_new;
-            fence_proxy_async();  // P is read by the tensor cores
             tc_fence_before();
-            mbar_arrive(&p_full);
-            if (!__all_sync(FULL_MASK, mbar_wait(&o_full[i & 1], (uint32_t)(i >> 1) & 1, a.err))) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&s_read);
+            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+            for (int c = 0; c < PA_KEYS; ++c) mx[c & 3] = fmaxf(mx[c & 3], sv[c]);
+            const float top = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * LOG2E;
+            // a row's first keys set its reference; later a maximum RESCALE above moves it
+            const bool fresh = m_run == -INFINITY;
+            const bool move = !fresh && top > m_run + RESCALE;
+            const float corr = move ? ex2(m_run - top) : 1.f;
+            if (fresh || move) m_run = top;
+            const float ref = m_run == -INFINITY ? 0.f : m_run;  // a row that has seen no key: every weight 0
+            l_run *= corr;
+            float sum[4] = {0.f, 0.f, 0.f, 0.f};
+            bool done = true;
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                uint32_t hi[PA_HALF / 2], lo[PA_HALF / 2];
+#pragma unroll
+                for (int e = 0; e < PA_HALF / 2; ++e) {
+                    const float p0 = ex2(fmaf(sv[half * PA_HALF + 2 * e], LOG2E, -ref));
+                    const float p1 = ex2(fmaf(sv[half * PA_HALF + 2 * e + 1], LOG2E, -ref));
+                    sum[(2 * e) & 3] += p0;
+                    sum[(2 * e + 1) & 3] += p1;
+                    split_pair(p0, p1, hi[e], lo[e]);
+                }
+                // the previous half's weights have been read (and O is complete up to them)
+                if (half || items > 0)
+                    done = __all_sync(FULL_MASK, lane != 0 || mbar_wait(&pv_done[half ^ 1],
+                                                                        (uint32_t)(half ? items : items - 1) & 1, a.err));
+                if (!done) break;
+                tc_fence_after();
+                if (half == 0 && __any_sync(FULL_MASK, move)) {
+#pragma unroll
+                    for (int c0 = 0; c0 < HEAD_DIM; c0 += 16) {
+                        float v[16];
+                        uint32_t r[16];
+                        tmem_ld16(base + TM_O + c0, v);
+#pragma unroll
+                        for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(v[e] * corr);
+                        tmem_st16(base + TM_O + c0, r);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < PA_HALF / 2; q += 16) {
+                    tmem_st16(base + TM_P + q, *reinterpret_cast<const uint32_t(*)[16]>(&hi[q]));
+                    tmem_st16(base + TM_PLO + q, *reinterpret_cast<const uint32_t(*)[16]>(&lo[q]));
+                }
+                tmem_st_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&p_full[half]);
+            }
+            if (!done) {
                 s_abort = 1;
+                fine = false;
                 break;
             }
+            l_run += (sum[0] + sum[1]) + (sum[2] + sum[3]);
+        }
+    }
+    // ---- this row's unnormalised output (registers) ----
+    float o[HEAD_DIM];
+#pragma unroll
+    for (int c = 0; c < HEAD_DIM; ++c) o[c] = 0.f;
+    if (tid < PA_ROWS && items > 0 && fine) {
+        if (__all_sync(FULL_MASK, lane != 0 || mbar_wait(&pv_done[1], (uint32_t)(items - 1) & 1, a.err))) {
             tc_fence_after();
 #pragma unroll
             for (int c0 = 0; c0 < HEAD_DIM; c0 += 32) {
                 float v[32];
-                tmem_ld32(tmem + lane_base + TM_O + (uint32_t)(i & 1) * HEAD_DIM + c0, v);
+                tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + TM_O + c0, v);
 #pragma unroll
-                for (int e = 0; e < 32; ++e) o[c0 + e] = o[c0 + e] * corr + v[e];
+                for (int e = 0; e < 32; ++e) o[c0 + e] = v[e];
             }
+        } else {
+            s_abort = 1;
         }
     }
     tc_fence_before();
@@ -329,33 +441,38 @@ __global__ void __launch_bounds__(PA_THREADS, 1) attn_tc_kernel(const AttnArgs a
     if (warp == 4) tmem_dealloc(tmem, TM_COLS);
     if (s_abort) return;  // error word set
 
-    // ---- results: rows of this tile ----
+    // ---- results: rows of this tile, through shared memory (Q's space is free), 16 lanes per row ----
     const int r = row0 + tid;
-    auto put = [&](const float* v) {  // 64 outputs of this row and head
-        if (a.out) {
-            float4* dst = reinterpret_cast<float4*>(a.out + (size_t)r * a.ldo + h * HEAD_DIM);
+    float4* ost = reinterpret_cast<float4*>(sm + OFF_Q);  // [128][16], chunk c of row q at c ^ (q & 15)
+    auto stage_row = [&](const float* v, float scale) {
 #pragma unroll
-            for (int c = 0; c < HEAD_DIM / 4; ++c) dst[c] = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
-        }
-        if (a.out_hi) {
-            uint4* dh = reinterpret_cast<uint4*>(a.out_hi + (size_t)r * a.ldb + h * HEAD_DIM);
-            uint4* dl = reinterpret_cast<uint4*>(a.out_lo + (size_t)r * a.ldb + h * HEAD_DIM);
+        for (int c = 0; c < HEAD_DIM / 4; ++c)
+            ost[tid * 16 + (c ^ (tid & 15))] =
+                make_float4(v[4 * c] * scale, v[4 * c + 1] * scale, v[4 * c + 2] * scale, v[4 * c + 3] * scale);
+    };
+    auto write_rows = [&]() {  // every warp writes the rows its own threads staged
+        __syncwarp();
 #pragma unroll
-            for (int c = 0; c < HEAD_DIM / 8; ++c) split8(v + 8 * c, dh[c], dl[c]);
+        for (int u = 0; u < 16; ++u) {
+            const int q = warp * 32 + u * 2 + (lane >> 4), c4 = lane & 15, rq = row0 + q;
+            if (rq >= a.rows) continue;
+            const bool on = s_seq[q] >= 0;
+            const float4 y = on ? ost[q * 16 + (c4 ^ (q & 15))] : make_float4(0.f, 0.f, 0.f, 0.f);
+            if (a.out && on) *reinterpret_cast<float4*>(a.out + (size_t)rq * a.ldo + h * HEAD_DIM + c4 * 4) = y;
+            if (a.out_hi) {
+                uint2 hi, lo;
+                split_pair(y.x, y.y, hi.x, lo.x);
+                split_pair(y.z, y.w, hi.y, lo.y);
+                *reinterpret_cast<uint2*>(a.out_hi + (size_t)rq * a.ldb + h * HEAD_DIM + c4 * 4) = hi;
+                *reinterpret_cast<uint2*>(a.out_lo + (size_t)rq * a.ldb + h * HEAD_DIM + c4 * 4) = lo;
+            }
         }
     };
-    const bool row_on = tid < PA_ROWS && r < a.rows;
-    const bool active = row_on && s_seq[tid] >= 0;
+    const bool active = tid < PA_ROWS && r < a.rows && my_seq >= 0;
     if (S == 1) {
-        if (active) {
-#pragma unroll
-            for (int c = 0; c < HEAD_DIM; ++c) o[c] /= l_run;
-            put(o);
-        } else if (row_on && a.out_hi) {
-#pragma unroll
-            for (int c = 0; c < HEAD_DIM; ++c) o[c] = 0.f;
-            put(o);
-        }
+        if (tid >= PA_ROWS) return;
+        if (active) stage_row(o, 1.f / l_run);
+        write_rows();
         return;
     }
     float* part = a.ws_part + (((size_t)(tile * H + h) * S + sp) * PA_ROWS) * PA_PART;
@@ -374,40 +491,33 @@ __global__ void __launch_bounds__(PA_THREADS, 1) attn_tc_kernel(const AttnArgs a
     if (!s_last) return;
     __threadfence();
     if (tid == 0) a.ws_count[tile * H + h] = 0;
-    if (!row_on) return;
-    if (!active) {
-        if (a.out_hi) {
+    if (tid >= PA_ROWS) return;
+    if (active) {
+        // merge the splits in split order: M = max m_s, L = sum 2^(m_s - M) l_s, out = sum 2^(m_s - M) o_s / L
+        const float* base = a.ws_part + ((size_t)(tile * H + h) * S * PA_ROWS + tid) * PA_PART;
+        const size_t sstride = (size_t)PA_ROWS * PA_PART;
+        float M = -INFINITY;
+        for (int s = 0; s < S; ++s) M = fmaxf(M, __ldcg(base + s * sstride));
+        float L = 0.f;
 #pragma unroll
-            for (int c = 0; c < HEAD_DIM; ++c) o[c] = 0.f;
-            put(o);
+        for (int c = 0; c < HEAD_DIM; ++c) o[c] = 0.f;
+        for (int s = 0; s < S; ++s) {
+            const float* ps = base + s * sstride;
+            const float ms = __ldcg(ps);
+            const float w = ms == -INFINITY ? 0.f : ex2(ms - M);
+            L = fmaf(w, __ldcg(ps + 1), L);
+#pragma unroll
+            for (int c = 0; c < HEAD_DIM; c += 4) {
+                const float4 v = __ldcg(reinterpret_cast<const float4*>(ps + 4 + c));
+                o[c] = fmaf(w, v.x, o[c]);
+                o[c + 1] = fmaf(w, v.y, o[c + 1]);
+                o[c + 2] = fmaf(w, v.z, o[c + 2]);
+                o[c + 3] = fmaf(w, v.w, o[c + 3]);
+            }
         }
-        return;
+        stage_row(o, 1.f / L);
     }
-    // merge the splits in split order: M = max m_s, L = sum exp(m_s - M) l_s, out = sum exp(m_s - M) o_s / L
-    const float* base = a.ws_part + ((size_t)(tile * H + h) * S * PA_ROWS + tid) * PA_PART;
-    const size_t sstride = (size_t)PA_ROWS * PA_PART;
-    float M = -INFINITY;
-    for (int s = 0; s < S; ++s) M = fmaxf(M, __ldcg(base + s * sstride));
-    float L = 0.f;
-#pragma unroll
-    for (int c = 0; c < HEAD_DIM; ++c) o[c] = 0.f;
-    for (int s = 0; s < S; ++s) {
-        const float* ps = base + s * sstride;
-        const float ms = __ldcg(ps);
-        const float w = ms == -INFINITY ? 0.f : expf(ms - M);
-        L = fmaf(w, __ldcg(ps + 1), L);
-#pragma unroll
-        for (int c = 0; c < HEAD_DIM; c += 4) {
-            const float4 v = __ldcg(reinterpret_cast<const float4*>(ps + 4 + c));
-            o[c] = fmaf(w, v.x, o[c]);
-            o[c + 1] = fmaf(w, v.y, o[c + 1]);
-            o[c + 2] = fmaf(w, v.z, o[c + 2]);
-            o[c + 3] = fmaf(w, v.w, o[c + 3]);
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < HEAD_DIM; ++c) o[c] /= L;
-    put(o);
+    write_rows();
 }
 
 }  // namespace
@@ -421,7 +531,7 @@ int attn_tc_tiles(int rows) { return (rows + PA_ROWS - 1) / PA_ROWS; }
 int attn_tc_splits_for(int tiles, int n_heads, int max_keys, int num_sms) {
     const int key_tiles = (max_keys + PA_KEYS - 1) / PA_KEYS;
     int s = num_sms / std::max(1, tiles * n_heads);
-    return std::max(1, std::min(s, key_tiles));
+    return std::max(1, std::min(s, key_tiles / PA_SPLIT_ITEMS));
 }
 
 cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t s, bool pdl) {

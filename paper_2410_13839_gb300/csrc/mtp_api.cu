@@ -115,7 +115,7 @@ struct mtp_ctx {
     int device = 0, num_sms = 0, wbytes = 2;
     int mlp_clusters = 1;  // MLP clusters co-resident in one wave
     bool use_graphs = true, use_pdl = true, use_l2_prefetch = false;
-    bool use_attn_tc = false;  // prefill passes: tensor-core attention (option; measured slower, see mtp.h)
+    bool use_attn_tc = false;  // prefill passes of any size: tcgen05 attention (option; else by the pass's rows)
     int use_heads_tc = 1;  // fused heads kernel: 0 never, 1 stand-alone heads calls, 2 also batched decode steps
     bool gemm_cluster = true;  // batched projections: one 128-row activation tile, K splits summed in clusters
     std::vector<void*> allocs;
@@ -329,8 +329,12 @@ int tile_index(int nt) { return nt == 32 ? 0 : (nt == 64 ? 1 : 2); }
 // Attention groups: `groups` runs of rpg rows, each of one slot (decode:
 // slot b's fed rows b*n.., plan PLAN_DEVICE; prefill: 8 consecutive prompt
 // positions, plan PLAN_ROWS).  prefill_keys > 0: a prefill pass whose rows see
-// at most that many keys; its attention runs on the tensor cores (tiles of 128
-// rows) unless that option is off.
+// at most that many keys; its attention runs in tiles of 128 rows (tcgen05)
+// above PREFILL_TC_ROWS rows, or always with that option.  A tile's chain of
+// 128-key items takes 5 + 3 us per item, which only many tiles pay back: per
+// launch 47 vs 143 us at 4096 serving-prompt rows, 28 vs 28 at 528, 19 vs 14 at
+// one prompt of 289.
+constexpr int PREFILL_TC_ROWS = 512;
 int run_layers_batched(mtp_ctx* c, int M, int rpg, int groups, int plan, cudaStream_t s, bool pdl, Prof* prof,
                        int prefill_keys = 0) {
     const mtp_config& cf = c->cfg;
@@ -422,7 +426,7 @@ int run_layers_batched(mtp_ctx* c, int M, int rpg, int groups, int plan, cudaStr
         }
         at.plan = plan; at.seq_len = c->d_len; at.seq_new = c->d_npend; at.seq_base = 0;
         at.err = c->d_err; at.kv_swizzled = 1;
-        if (prefill_keys > 0 && c->use_attn_tc && plan == PLAN_ROWS) {
+        if (prefill_keys > 0 && (c->use_attn_tc || M > PREFILL_TC_ROWS) && plan == PLAN_ROWS) {
             // tiles of 128 rows; splits as many as the batched attention workspace holds (S = 1 uses none)
             const int tiles = attn_tc_tiles(M);
             const size_t ws_floats = attn_workspace_floats(c->battn_ws_units, H, 1, MAX_ROWS);
