@@ -129,6 +129,60 @@ __global__ void __launch_bounds__(PK_THREADS) pack_rows_kernel(const PackArgs a)
     }
 }
 
+// LayerNorm rows of many-row passes, one warp per row: up to 8 float4 chunks per lane, the
+// statistics in registers and shuffles only (no block barrier), every load of the row in flight at
+// once.  4096 rows of d = 1024: 9.2 vs 15.9 us with a CTA per row, whose 256 threads hold one
+// chunk each and wait for one another.
+constexpr int PK_WARP_MAXQ = 8;
+constexpr int PK_WARP_ROWS = 1024;  // rows from which it is used (fewer rows: a CTA per row spreads wider)
+__global__ void __launch_bounds__(PK_THREADS) pack_ln_warp_kernel(const PackArgs a) {
+    const int lane = threadIdx.x & 31, r = blockIdx.x * (PK_THREADS / 32) + (threadIdx.x >> 5);
+    const int K = a.k, nq = K / 4;
+    TraceEnd trace_guard(a.trace);
+    pdl_launch_dependents();
+    pdl_wait();
+    trace_wait(a.trace);
+    if (r >= a.m) return;
+    const bool on = a.row_seq[r] >= 0;
+    const float4* xr = reinterpret_cast<const float4*>(a.x + (size_t)r * a.ldx);
+    float4 v[PK_WARP_MAXQ];
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < PK_WARP_MAXQ; ++i) {
+        const int q = lane + i * 32;
+        v[i] = on && q < nq ? xr[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll
+    for (int i = 0; i < PK_WARP_MAXQ; ++i) s += (v[i].x + v[i].y) + (v[i].z + v[i].w);
+    const float mean = warp_sum(s) / (float)K;
+    float q2 = 0.f;
+#pragma unroll
+    for (int i = 0; i < PK_WARP_MAXQ; ++i)
+        if (lane + i * 32 < nq) {
+            const float d0 = v[i].x - mean, d1 = v[i].y - mean, d2 = v[i].z - mean, d3 = v[i].w - mean;
+            q2 += (d0 * d0 + d1 * d1) + (d2 * d2 + d3 * d3);
+        }
+    const float rstd = 1.0f / sqrtf(warp_sum(q2) / (float)K + a.eps);
+#pragma unroll
+    for (int i = 0; i < PK_WARP_MAXQ; ++i) {
+        const int q = lane + i * 32;
+        if (q >= nq) continue;
+        const float4 g = __ldg(reinterpret_cast<const float4*>(a.gamma) + q);
+        const float4 b = __ldg(reinterpret_cast<const float4*>(a.beta) + q);
+        float4 y = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (on)
+            y = make_float4((v[i].x - mean) * rstd * g.x + b.x, (v[i].y - mean) * rstd * g.y + b.y,
+                            (v[i].z - mean) * rstd * g.z + b.z, (v[i].w - mean) * rstd * g.w + b.w);
+        const __nv_bfloat162 h0 = __floats2bfloat162_rn(y.x, y.y), h1 = __floats2bfloat162_rn(y.z, y.w);
+        const uint2 hi = make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1));
+        const __nv_bfloat162 l0 = __floats2bfloat162_rn(y.x - bf16_lo(hi.x), y.y - bf16_hi(hi.x));
+        const __nv_bfloat162 l1 = __floats2bfloat162_rn(y.z - bf16_lo(hi.y), y.w - bf16_hi(hi.y));
+        reinterpret_cast<uint2*>(a.hi + (size_t)r * K)[q] = hi;
+        reinterpret_cast<uint2*>(a.lo + (size_t)r * K)[q] =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&l0), *reinterpret_cast<const uint32_t*>(&l1));
+    }
+}
+
 template <typename K, typename A>
 cudaError_t launch_rows(K kern, const A& args, int rows, cudaStream_t s, bool pdl) {
     cudaLaunchConfig_t cfg = {};
@@ -158,6 +212,8 @@ cudaError_t launch_pack_rows(const PackArgs& a, cudaStream_t s, bool pdl) {
         return launch_rows(pack_rows_kernel<true, 4>, a, a.m, s, pdl);
     }
     if (a.zero_buf) return cudaErrorInvalidValue;  // zeroing comes with the every-row variant
+    if (a.mode == PACK_LN && a.m >= PK_WARP_ROWS && a.k <= 4 * 32 * PK_WARP_MAXQ)
+        return launch_rows(pack_ln_warp_kernel, a, (a.m + PK_THREADS / 32 - 1) / (PK_THREADS / 32), s, pdl);
     if (chunks <= 1) return launch_rows(pack_rows_kernel<false, 1>, a, a.m, s, pdl);
     return launch_rows(pack_rows_kernel<false, 4>, a, a.m, s, pdl);
 }
