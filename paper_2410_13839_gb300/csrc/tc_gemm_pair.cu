@@ -14,7 +14,7 @@
 // from the peer, so the same 48 KB feed 1024 cycles.  Two accumulators of 256
 // TMEM columns let the epilogue warps write one tile out while the next
 // one is multiplied.  4096 rows, d = 1024, device time against 128 x 128
-// tiles: q|k|v 40 vs 74 us (1.29 PFLOP/s of MMA), W1 with GELU 71 vs 101,
+// tiles: q|k|v 40 vs 74 us (1.29 PFLOP/s of MMA), W1 with GELU 59 vs 101,
 // W_o 22 vs 24, W2 52 vs 81.
 //
 // Per CTA, 12 or 20 warps: warp 0 copies (one lane, TMA into a four-stage ring; both
@@ -113,7 +113,8 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
 __device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(32 * TP_EPI_WARPS) : "memory"); }
 
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    return (uint32_t)f32_to_bf16_bits(lo) | ((uint32_t)f32_to_bf16_bits(hi) << 16);
+    const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t*>(&p);
 }
 
 template <int EPI>
@@ -299,20 +300,28 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
             } else if (EPI == TC_GELU_PACK) {
                 // lanes 2i, 2i + 1 exchange one value: the even lane writes features (f, f + 1) of row
                 // e, the odd lane of row e + 1
-                const int odd = lane & 1, fe = f - odd;
+                const int odd = lane & 1;
+                // rows of a sequence (the others are written as zeros)
+                const uint32_t act[2] = {__ballot_sync(FULL_MASK, s_rowt[fb][j0 + lane]),
+                                         __ballot_sync(FULL_MASK, s_rowt[fb][j0 + 32 + lane])};
+                const size_t at = (size_t)(n0 + odd) * a.ldo + (f - odd);
+                __nv_bfloat16 *ph = a.pack_hi + at, *pl = a.pack_lo + at;
+                const int mine = rows - odd;  // this lane writes rows e + odd < rows
 #pragma unroll
                 for (int e = 0; e < TP_COLS; e += 2) {
-                    const float g0 = s_rowt[fb][j0 + e] ? gelu_erf(sum[e] + bias) : 0.f;
-                    const float g1 = s_rowt[fb][j0 + e + 1] ? gelu_erf(sum[e + 1] + bias) : 0.f;
+                    const float u0 = gelu_erf(sum[e] + bias), u1 = gelu_erf(sum[e + 1] + bias);
+                    const float g0 = act[e >> 5] >> (e & 31) & 1 ? u0 : 0.f;
+                    const float g1 = act[e >> 5] >> ((e & 31) + 1) & 1 ? u1 : 0.f;
                     const float got = __shfl_xor_sync(FULL_MASK, odd ? g0 : g1, 1);
                     const float y0 = odd ? got : g0, y1 = odd ? g1 : got;
                     const uint32_t hi = pack_bf16(y0, y1);
                     const uint32_t lo = pack_bf16(y0 - bf16_lo(hi), y1 - bf16_hi(hi));
-                    if (e + odd < rows) {
-                        const size_t at = (size_t)(n0 + e + odd) * a.ldo + fe;
-                        *reinterpret_cast<uint32_t*>(a.pack_hi + at) = hi;
-                        *reinterpret_cast<uint32_t*>(a.pack_lo + at) = lo;
+                    if (e < mine) {
+                        *reinterpret_cast<uint32_t*>(ph) = hi;
+                        *reinterpret_cast<uint32_t*>(pl) = lo;
                     }
+                    ph += 2 * (size_t)a.ldo;
+                    pl += 2 * (size_t)a.ldo;
                 }
             } else {  // TC_QKV: features h * 192 + {q, k, v} * 64 + dd (one head and part per warp)
                 const int h = f / (3 * HEAD_DIM), sec = (f / HEAD_DIM) % 3, dd = f % HEAD_DIM;
