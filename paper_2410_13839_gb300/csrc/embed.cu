@@ -104,15 +104,10 @@ __global__ void convert_rows_kernel(const void* src, int src_bf16, float* dst, l
 }
 
 __global__ void __launch_bounds__(1024) lane_plan_kernel(const LanePlanArgs a) {
-    __shared__ int s_scan[1024];
+    __shared__ int s_scan[1024], s_take[1024], s_len[1024], s_left[1024];
     pdl_wait();  // the previous step's selection moved the slots' state
     pdl_launch_dependents();
     const int b = threadIdx.x;
-    for (int i = threadIdx.x; i < a.capacity; i += blockDim.x) {
-        a.row_seq[a.row0 + i] = -1;
-        a.row_pos[a.row0 + i] = -1;
-        a.row_last[a.row0 + i] = 0;
-    }
     int left = 0, len = 0;
     if (b < a.slots && a.active[b] && !a.done[b]) {
         left = max(0, a.prompt_left[b]);
@@ -128,19 +123,40 @@ __global__ void __launch_bounds__(1024) lane_plan_kernel(const LanePlanArgs a) {
         __syncthreads();
     }
     const int start = s_scan[b] - demand;
-    int take = 0;
-    if (left > 0 && start < a.capacity) {
-        take = min(left, a.capacity - start);
-        for (int i = 0; i < take; ++i) {
-            const int row = a.row0 + start + i;
-            a.row_seq[row] = b;
-            a.row_pos[row] = len + i;
-            a.row_last[row] = (i == take - 1 && take == left) ? 1 : 0;
-        }
+    const int take = left > 0 && start < a.capacity ? min(left, a.capacity - start) : 0;
+    if (take > 0) {
         a.prompt_left[b] = left - take;
         a.seq_len[b] = len + take;
     }
     if (b < a.slots) a.lane_take[b] = take;
+    s_take[b] = take;
+    s_len[b] = len;
+    s_left[b] = left;
+    __syncthreads();
+    // the rows: every thread finds the slot whose padded share its row falls in (the first inclusive
+    // sum above it) by bisection
+    for (int i = b; i < a.capacity; i += blockDim.x) {
+        int lo = 0, hi = blockDim.x;
+        while (lo < hi) {
+            const int mid = (lo + hi) >> 1;
+            if (s_scan[mid] > i)
+                hi = mid;
+            else
+                lo = mid + 1;
+        }
+        int seq = -1, pos = -1, last = 0;
+        if (lo < (int)blockDim.x) {
+            const int at = i - (lo > 0 ? s_scan[lo - 1] : 0);
+            if (at < s_take[lo]) {
+                seq = lo;
+                pos = s_len[lo] + at;
+                last = at == s_take[lo] - 1 && s_take[lo] == s_left[lo];
+            }
+        }
+        a.row_seq[a.row0 + i] = seq;
+        a.row_pos[a.row0 + i] = pos;
+        a.row_last[a.row0 + i] = last;
+    }
 }
 
 __global__ void slot_set_kernel(SlotSet s) {
@@ -226,7 +242,7 @@ cudaError_t launch_lane_plan(const LanePlanArgs& a, cudaStream_t s, bool pdl) {
     if (a.slots < 1 || a.slots > 1024 || a.rpg < 1 || a.capacity < 1 || a.capacity % a.rpg) return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(1);
-    cfg.blockDim = dim3((a.slots + 31) / 32 * 32);
+    cfg.blockDim = dim3(1024);  // a thread per slot, then per row
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

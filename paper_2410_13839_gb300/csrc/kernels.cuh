@@ -18,11 +18,12 @@ namespace mtp {
 constexpr int HEAD_DIM = 64;     // attention head width (fixed by the kernels)
 constexpr int MAX_ROWS = 8;      // rows per weight-streaming pass (B * n_heads per chunk)
 constexpr int PREFILL_ROWS = 128; // prompt positions of a decode step's prefill lane
-// Most prompt positions of one prefill pass.  A pass of a few hundred rows is bound by its chain of
-// dependent launches, like a decode step (0.55 ms for 128 rows, 0.9 ms for 384); at 4096 rows every
-// launch is several waves.  Prefill of 32 serving prompts (12.8k positions): 16.4 ms in passes of
-// 4096, 29.2 ms in passes of 384; one 289-position prompt: 0.79 ms in one pass, 1.7 ms in three.
-constexpr int PREFILL_PASS_ROWS = 4096;
+// Most prompt positions of one prefill pass (28 KB of buffers each at d = 1024).  A pass of a few
+// hundred rows is bound by its chain of dependent launches, like a decode step (0.55 ms for 128 rows,
+// 0.9 ms for 384), and a short last pass costs nearly as much as a long one.  Prefill of 32 / 128
+// serving prompts (12.8k / 48.6k positions): 7.6 / 29.3 ms in passes of 16384, 9.7 / 34.2 in
+// passes of 4096, 29.2 / 68.9 in passes of 384 / 1152; one 289-position prompt: 0.79 ms in one pass, 1.7 ms in three.
+constexpr int PREFILL_PASS_ROWS = 16384;
 constexpr int MAX_TOPK = 32;     // one warp lane per candidate
 constexpr int MAX_NHEADS = 8;    // prediction heads
 constexpr int MAX_VOCAB = 1056;  // 33 logits per lane in the top-k warp
