@@ -1,23 +1,37 @@
 // attention.cu -- causal attention of the fed rows over the paged bf16 KV cache
 // (the attention of each block, Sec. III-A), split along the key axis.
 //
-// Grid (split, head, group).  A group is the rows of one slot (the n tokens
-// fed this step, or 8 consecutive positions of a prefill chunk).  Each CTA
-// takes a contiguous range of pages of its slot and streams their keys and
-// values for its head through a ring of three shared-memory slots with
-// cp.async.bulk (two are in flight while one is read).  Each warp takes
-// 16-key tiles on the tensor cores (mma.sync) with the keys as the M side:
-// S^T = K Q^T and O^T += V^T P^T, the fed rows' Q and P entering as bf16
-// hi + lo pairs (two N = 8 operands), which keeps them to fp32 accuracy, and
-// its online-softmax state in registers; the warps' states are merged in
-// shared memory.  Partial results (max,
-// sum, unnormalised output) of the splits are merged with a log-sum-exp by
-// the CTA that finishes last (an atomic counter per group and head, reset by
-// that CTA), so no second kernel is needed.
+// A group is the rows of one slot (the n tokens fed this step, or 8
+// consecutive positions of a prefill chunk).  Each head's work is the stream of
+// every group's cached keys, in batches of 64 (one page of 128): grid (J, H),
+// CTA j of head h takes batches [j T / J, (j + 1) T / J) of the T, whatever
+// groups they belong to.  With J chosen for one wave (four CTAs per SM), all
+// CTAs do the same work whether the contexts are ragged or not, and a CTA's
+// fixed costs (plan, first copies, merges: about 5 us) are paid once per wave.
+// Splitting every group's keys in the same number of parts left the longest
+// contexts to set the time (one part) or paid those costs over and over (three
+// parts, 2.5 waves).  32 slots of 180-2000 keys, 16 heads: 35 vs 51 us alone (one
+// part), and per launch of a decode step at about 450 keys 18.6 vs 29 us (32
+// slots, three parts) and 45 vs 57 us (128 slots, one part).
 //
-// Under programmatic dependent launch the first pages that hold only keys
-// cached by earlier steps are fetched before griddepcontrol.wait; the pages
-// touched by this step's appends are read after it.
+// A CTA finds its first group by a scan over the groups' batch counts, and then
+// walks the stream: warp 0 keeps the next batches of keys and values on their
+// way into a ring of three shared-memory slots with cp.async.bulk (a lane per
+// page; plain pools, the stand-alone operator's, with tensor copies that
+// swizzle the rows like the cache: at their plain 128-byte pitch every ldmatrix
+// of eight rows was an 8-way bank conflict, 86 vs 51 us for 32 slots of about
+// 1,100 keys).  Each warp takes 16-key tiles on the tensor cores (mma.sync)
+// with the keys as the M side: S^T = K Q^T and O^T += V^T P^T, the fed rows' Q
+// and P entering as bf16 hi + lo pairs (two N = 8 operands), which keeps them
+// to fp32 accuracy, and its online-softmax state in registers; the warps'
+// states are merged in shared memory at the end of the group.  A group that
+// several CTAs share leaves partial results (max, sum, unnormalised output) in
+// the workspace, and the CTA that finishes last (an atomic counter per group
+// and head, reset by that CTA) merges them in stream order, so no second kernel
+// is needed.
+//
+// Under programmatic dependent launch the plan and the first batches that hold
+// only keys cached by earlier steps are fetched before griddepcontrol.wait.
 #include <math.h>
 
 #include <cstdio>
@@ -33,8 +47,10 @@ constexpr int ATT_THREADS = 128;  // four warps: four CTAs per SM
 constexpr int ATT_STAGES = 3;    // staging slots of the key/value ring (three 64-key slots keep ~48 KB in flight)
 constexpr int RPG = MAX_ROWS;    // rows per group, upper bound
 constexpr int PART = 2 + HEAD_DIM;  // (max, sum, out[64]) per row and split
-constexpr int MAX_SPLITS = ATTN_MAX_SPLITS;  // one warp lane per split in the merge
-static_assert(MAX_SPLITS <= 32, "the merge takes one lane per split");
+constexpr float LOG2E = 1.4426950408889634f;
+constexpr float RESCALE = 8.f;   // growth of a row's scores (log2) that moves its reference
+constexpr int NW = ATT_THREADS / 32;
+constexpr int MROWS = 4;         // rows whose warp states are merged at a time (one per warp)
 static_assert(HEAD_DIM == 64, "score scale 0.125 assumes 64-wide heads");
 
 
@@ -42,6 +58,11 @@ static_assert(HEAD_DIM == 64, "score scale 0.125 assumes 64-wide heads");
 // keys per staging half: 64, or a whole page when pages are longer
 __host__ __device__ constexpr int half_keys(int page_size) { return page_size > 64 ? page_size : 64; }
 
+__device__ __forceinline__ float ex2(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
@@ -68,142 +89,219 @@ __device__ __forceinline__ uint32_t movmatrix_trans(uint32_t r) {
 }
 // x0, x1 as bf16 pairs hi + lo (hi + lo = x to about 2^-16 relative; low halves hold x0)
 __device__ __forceinline__ void split2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
-    const __nv_bfloat16 h0 = __float2bfloat16_rn(x0), h1 = __float2bfloat16_rn(x1);
-    const __nv_bfloat16 l0 = __float2bfloat16_rn(x0 - __bfloat162float(h0));
-    const __nv_bfloat16 l1 = __float2bfloat16_rn(x1 - __bfloat162float(h1));
-    hi = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-    lo = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
+    hi = *reinterpret_cast<const uint32_t*>(&h);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(x0 - bf16_lo(hi), x1 - bf16_hi(hi));
+    lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
-// Bulk copies of pages [p_from, p_to) of `seq` (this head) into the half
-// that starts at key `key0` of the staging arrays, completing on `bar`.
-// One thread calls it; returns whether anything was requested.
-__device__ __forceinline__ bool stage_pages(const AttnArgs& a, int seq, int p_from, int p_to, int slot0,
-                                            __nv_bfloat16* Ks, __nv_bfloat16* Vs, long long kv_head_off,
-                                            long long v_off, uint64_t* bar, const int* ids = nullptr,
-                                            int id0 = 0, int n_ids = 0) {
-    const int P = a.page_size;
-    const uint32_t blk = (uint32_t)P * HEAD_DIM * 2;
-    // page p's id: from the shared copy ids[p - id0] when it holds it, else from the block table
-    auto page_id = [&](int p) {
-        return (ids && p - id0 >= 0 && p - id0 < n_ids) ? ids[p - id0] : a.block_table[(size_t)seq * a.bt_stride + p];
-    };
-    uint32_t bytes = 0;
-    for (int p = p_from; p < p_to; ++p)
-        if (page_id(p) >= 0) bytes += 2 * blk;
-    if (!bytes) return false;
-    fence_proxy_async();  // the half was last read by this CTA's threads
-    mbar_arrive_expect_tx(bar, bytes);
-    for (int p = p_from; p < p_to; ++p) {
-        const int phys = page_id(p);
-        if (phys < 0) {  // unreserved page: report, never read
-            if (a.err) atomicOr(a.err, ERR_BOUNDS);
-            continue;
+// PLAIN: the pool holds plain rows; a tensor copy with the 128-byte swizzle lays them out as the
+// cache stores them (chunk c of row t at c ^ (t & 7)).
+__device__ __forceinline__ void tma_page(void* dst, const CUtensorMap* map, int row, int page, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(
+            smem_addr(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(0), "r"(row), "r"(page), "r"(smem_addr(bar))
+        : "memory");
+}
+
+// What the plan needs of a group: the keys its rows see (0: no active row), its slot, and (PLAN_DEVICE)
+// how many rows it has: row j at position keys - rows + j.
+struct Group {
+    int keys, seq, rows;
+};
+// PLAN_DEVICE: from the slot state left by earlier steps (the rule the embedding applies), so it is known
+// before the dependency wait.
+__device__ __forceinline__ Group load_group(const AttnArgs& a, int g) {
+    Group x = {0, g, 0};
+    if (a.plan == PLAN_DEVICE) {  // one round of independent loads
+        const int act = a.active[g], dn = a.done[g], np = a.seq_new[g], len = a.seq_len[g];
+        if (act && !dn && np > 0) {
+            x.keys = len + np;
+            x.rows = np;
         }
-        const __nv_bfloat16* base = a.kv_pool + (long long)phys * a.page_elems + a.layer_off + kv_head_off;
-        const int slot = slot0 + (p - p_from);
-        bulk_copy_g2s(Ks + (size_t)slot * P * HEAD_DIM, base, blk, bar);
-        bulk_copy_g2s(Vs + (size_t)slot * P * HEAD_DIM, base + v_off, blk, bar);
+        return x;
     }
-    return true;
+#pragma unroll
+    for (int j = 0; j < RPG; ++j) {
+        if (j >= a.rows_per_group) break;
+        const int r = g * a.rows_per_group + j;
+        const int rs = r < a.rows ? a.row_seq[r] : -1, rp = r < a.rows ? a.row_pos[r] : 0;
+        if (rs >= 0) {
+            x.seq = rs;
+            x.keys = max(x.keys, rp + 1);
+        }
+    }
+    return x;
 }
 
-__global__ void __launch_bounds__(ATT_THREADS, 4) attn_kernel(const AttnArgs a) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    __shared__ uint64_t bar;         // pages staged before the dependency wait
-    __shared__ uint64_t hbar[ATT_STAGES];  // the staging slots
-    __shared__ int s_armed[ATT_STAGES];
-    __shared__ float s_scale[ATT_THREADS / 32][RPG];
-    __shared__ int s_pos[RPG];
-    __shared__ int s_act[RPG];
-    __shared__ int s_rseq[RPG];
-    __shared__ int s_seq, s_ktot, s_pre, s_last;
-    constexpr int ID_CAP = 128;
-    __shared__ int s_ids[ID_CAP];  // this split's page ids (the first ID_CAP), read once
+template <bool PLAIN>
+__global__ void __launch_bounds__(ATT_THREADS, 4)
+    attn_kernel(const AttnArgs a, const __grid_constant__ CUtensorMap plain_map) {
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
+    // the tensor copy's swizzle goes by the address: 1024-byte aligned slots
+    unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    __shared__ uint64_t bar[ATT_STAGES];
+    __shared__ int s_sum[NW], s_g0, s_off;
+    __shared__ Group s_group[ATT_THREADS];  // the groups' facts, where they are at most that many
+    __shared__ int s_share[2][4];           // groups shared with other CTAs: group, first CTA, parts, active rows
+    __shared__ int s_last[2];
 
-    const int sp = blockIdx.x, h = blockIdx.y, g = blockIdx.z;
+    const int jc = blockIdx.x, h = blockIdx.y;
     TraceEnd trace_guard(a.trace);
-    const int H = a.n_heads, P = a.page_size, S = a.n_splits;
+    const int H = a.n_heads, P = a.page_size, rpg = a.rows_per_group;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int HALF_KEYS = half_keys(P);  // keys per staging half
+    const int KB = half_keys(P);       // keys per batch
+    const int ppb = KB / P;            // pages per batch
     __nv_bfloat16* Ks = reinterpret_cast<__nv_bfloat16*>(smem);
-    __nv_bfloat16* Vs = Ks + ATT_STAGES * HALF_KEYS * HEAD_DIM;
-    float* qs = reinterpret_cast<float*>(Vs + ATT_STAGES * HALF_KEYS * HEAD_DIM);  // [RPG][64], pre-scaled
-    const int pages_per_batch = HALF_KEYS / P;  // pages per staging half
+    __nv_bfloat16* Vs = Ks + ATT_STAGES * KB * HEAD_DIM;
+    float* wst = reinterpret_cast<float*>(Vs + ATT_STAGES * KB * HEAD_DIM);  // [NW][MROWS][PART] warp states
     const long long kv_head_off = (long long)h * P * HEAD_DIM;
     const long long v_off = (long long)H * P * HEAD_DIM;
 
     if (tid == 0) {
-        mbar_init(&bar, 1);
-        for (int i = 0; i < ATT_STAGES; ++i) mbar_init(&hbar[i], 1);
+        if (PLAIN) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&plain_map)) : "memory");
+        for (int i = 0; i < ATT_STAGES; ++i) mbar_init(&bar[i], 1);
+        s_share[0][2] = s_share[1][2] = 0;
         fence_barrier_init();
-        s_pre = 0;
     }
-    __syncthreads();
+    if (a.plan != PLAN_DEVICE) {  // the rows' plan is written by an earlier kernel of this pass
+        pdl_launch_dependents();
+        pdl_wait();
+        trace_wait(a.trace);
+    }
 
-    // ---- before the wait: slot state left by earlier steps ----
-    if (tid == 0 && a.plan != PLAN_ROWS) {
-        int seq, old_len, n_new;
-        if (a.plan == PLAN_DEVICE) {
-            seq = a.seq_base + g;
-            old_len = a.seq_len[seq];
-            n_new = a.seq_new[seq];
-        } else {
-            seq = a.val_seq;
-            old_len = a.val_old;
-            n_new = a.val_new;
+    // ---- this CTA's share of the head's stream of batches ----
+    const bool few = a.groups <= ATT_THREADS && !a.whole;
+    auto group_of = [&](int g) { return few ? s_group[g] : load_group(a, g); };
+    auto batches = [&](const Group& x) { return (x.keys + KB - 1) / KB; };
+    // inclusive sum of v over the block's threads before and including this one; total: of all
+    auto block_scan = [&](int v, int& total) {
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(FULL_MASK, v, o);
+            if (lane >= o) v += u;
         }
-        if (n_new > 0) {
-            const int n_pg = (old_len + n_new + P - 1) / P;
-            const int pps = (n_pg + S - 1) / S;
-            const int pg0 = sp * pps, pg1 = min(n_pg, pg0 + pps);
-            int pre_end = min(min(pg1, pg0 + pages_per_batch), old_len / P);  // half 0 at most
-            for (int p = pg0; p < pre_end; ++p)  // only reserved pages are fetched early
-                if (a.block_table[(size_t)seq * a.bt_stride + p] < 0) pre_end = p;
-            if (pre_end > pg0) {
-                const uint32_t blk = (uint32_t)P * HEAD_DIM * 2;
-                mbar_arrive_expect_tx(&bar, 2u * blk * (uint32_t)(pre_end - pg0));
-                for (int p = pg0; p < pre_end; ++p) {
-                    const int phys = a.block_table[(size_t)seq * a.bt_stride + p];
-                    const __nv_bfloat16* base = a.kv_pool + (long long)phys * a.page_elems + a.layer_off + kv_head_off;
-                    bulk_copy_g2s(Ks + (p - pg0) * P * HEAD_DIM, base, blk, &bar);
-                    bulk_copy_g2s(Vs + (p - pg0) * P * HEAD_DIM, base + v_off, blk, &bar);
+        __syncthreads();  // s_sum's last readers are done
+        if (lane == 31) s_sum[warp] = v;
+        __syncthreads();
+        total = 0;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            if (w < warp) v += s_sum[w];
+            total += s_sum[w];
+        }
+        return v;
+    };
+    int T, J, x0, x1;  // batches of the head, CTAs that take part (each has a batch), this CTA's range
+    if (a.whole) {  // group jc, all of it
+        T = J = x0 = 0;
+        x1 = batches(load_group(a, jc));
+        if (tid == 0) {
+            s_g0 = jc;
+            s_off = 0;
+        }
+    } else {
+        int nb0 = 0;  // of the first 128 groups
+        if (tid < a.groups) {
+            const Group x = load_group(a, tid);
+            s_group[tid] = x;
+            nb0 = batches(x);
+        }
+        const int incl0 = block_scan(nb0, T);
+        for (int base = ATT_THREADS; base < a.groups; base += ATT_THREADS) {
+            int t;
+            block_scan(base + tid < a.groups ? batches(load_group(a, base + tid)) : 0, t);
+            T += t;
+        }
+        J = max(1, min((int)gridDim.x, T));
+        x0 = jc < J ? (int)((long long)jc * T / J) : T;
+        x1 = jc < J ? (int)((long long)(jc + 1) * T / J) : T;
+        if (x0 < x1) {  // the group that holds batch x0
+            int before = 0;
+            for (int base = 0; base < a.groups; base += ATT_THREADS) {
+                int nb = nb0, incl = incl0, t = 0;
+                if (!few) {
+                    nb = base + tid < a.groups ? batches(load_group(a, base + tid)) : 0;
+                    incl = block_scan(nb, t);
                 }
-                s_pre = pre_end - pg0;
+                if (before + incl - nb <= x0 && x0 < before + incl) {
+                    s_g0 = base + tid;
+                    s_off = x0 - (before + incl - nb);
+                }
+                before += t;
+                if (x0 < before) break;
             }
         }
     }
-
-    pdl_launch_dependents();
-    pdl_wait();
-    trace_wait(a.trace);
-
-    // ---- rows of this group (written by this step's embedding) ----
-    const int rpg = a.rows_per_group;
-    if (tid < RPG) {
-        const int r = g * rpg + tid;
-        const int rs = tid < rpg ? a.row_seq[r] : -1;
-        const int rp = tid < rpg ? a.row_pos[r] : -1;
-        s_act[tid] = rs >= 0;
-        s_rseq[tid] = rs;
-        s_pos[tid] = rs >= 0 ? rp : -1;
-    }
     __syncthreads();
-    if (tid == 0) {
-        int seq = -1, kmax = 0;
-        for (int j = 0; j < RPG; ++j)
-            if (s_act[j]) {
-                seq = s_rseq[j];
-                kmax = max(kmax, s_pos[j] + 1);
+
+    // ---- copies: warp 0 walks the stream ahead of the tiles ----
+    int pg = 0, pb = 0, pnb = 0, pseq = -1, ppages = 0, pold = 0, staged = 0;  // group, its next batch, ...
+    auto next_group = [&]() {  // the next group with keys, from pg on
+        for (;; ++pg) {
+            const Group x = group_of(pg);
+            pnb = batches(x);
+            pseq = x.seq;
+            ppages = (x.keys + P - 1) / P;
+            pold = a.plan == PLAN_DEVICE ? (x.keys - x.rows) / P : ppages;  // pages of earlier steps' keys only
+            if (pnb > 0) return;
+        }
+    };
+    auto stage_next = [&]() {  // the stream's next batch into the ring (warp 0)
+        const int slot = staged % ATT_STAGES, p = pb * ppb + lane;
+        const bool mine = lane < ppb && p < ppages;
+        const int phys = mine ? a.block_table[(size_t)pseq * a.bt_stride + p] : -1;
+        if (mine && phys < 0 && a.err) atomicOr(a.err, ERR_BOUNDS);  // unreserved page: report, never read
+        const unsigned have = __ballot_sync(FULL_MASK, phys >= 0);
+        const uint32_t blk = (uint32_t)P * HEAD_DIM * 2;
+        fence_proxy_async();  // the slot was last read by this CTA's threads
+        if (lane == 0) mbar_arrive_expect_tx(&bar[slot], 2 * blk * __popc(have));
+        __syncwarp();
+        if (phys >= 0) {
+            __nv_bfloat16* kd = Ks + ((size_t)slot * KB + lane * P) * HEAD_DIM;
+            __nv_bfloat16* vd = Vs + ((size_t)slot * KB + lane * P) * HEAD_DIM;
+            if (PLAIN) {
+                const int row = (int)((a.layer_off + kv_head_off) / HEAD_DIM);
+                tma_page(kd, &plain_map, row, phys, &bar[slot]);
+                tma_page(vd, &plain_map, row + (int)(v_off / HEAD_DIM), phys, &bar[slot]);
+            } else {
+                const __nv_bfloat16* base = a.kv_pool + (long long)phys * a.page_elems + a.layer_off + kv_head_off;
+                bulk_copy_g2s(kd, base, blk, &bar[slot]);
+                bulk_copy_g2s(vd, base + v_off, blk, &bar[slot]);
             }
-        s_seq = seq;
-        s_ktot = kmax;
+        }
+        ++staged;
+        if (++pb == pnb && x0 + staged < x1) {
+            ++pg;
+            next_group();
+            pb = 0;
+        }
+    };
+    const int n = x1 - x0;
+    int g = 0, cb = 0;  // group and batch within it
+    if (n > 0) {
+        g = s_g0;
+        cb = s_off;
+        if (warp == 0) {
+            pg = g;
+            next_group();
+            pb = cb;
+            if (a.plan == PLAN_DEVICE)
+                while (staged < min(n, ATT_STAGES) && min((pb + 1) * ppb, ppages) <= pold) stage_next();
+        }
     }
-    __syncthreads();
-    const int seq = s_seq, K_tot = s_ktot, n_pre = s_pre;
-    // output pair (2 lane, 2 lane + 1) of head h in row row_j of the group
-    auto put = [&](int row_j, float v0, float v1) {
-        const size_t r = (size_t)(g * rpg + row_j);
+    if (a.plan == PLAN_DEVICE) {
+        pdl_launch_dependents();
+        pdl_wait();
+        trace_wait(a.trace);
+    }
+    if (warp == 0)
+        while (staged < min(n, ATT_STAGES)) stage_next();
+
+    // output pair (2 lane, 2 lane + 1) of head h in row row_j of group gr
+    auto put = [&](int gr, int row_j, float v0, float v1) {
+        const size_t r = (size_t)gr * rpg + row_j;
         if (a.out) {
             float* o = a.out + r * a.ldo + h * HEAD_DIM + 2 * lane;
             o[0] = v0;
@@ -216,310 +314,302 @@ __global__ void __launch_bounds__(ATT_THREADS, 4) attn_kernel(const AttnArgs a) 
             *reinterpret_cast<uint32_t*>(a.out_lo + r * a.ldb + h * HEAD_DIM + 2 * lane) = lo;
         }
     };
-    if (seq < 0) {  // nothing to do for this group (no split of it counts)
-        if (n_pre > 0) mbar_wait(&bar, 0, a.err);
-        if (a.out_hi && sp == 0)
-            for (int row_j = warp; row_j < rpg; row_j += ATT_THREADS / 32) {
-                const size_t o = (size_t)(g * rpg + row_j) * a.ldb + h * HEAD_DIM + 2 * lane;
-                *reinterpret_cast<uint32_t*>(a.out_hi + o) = 0u;
-                *reinterpret_cast<uint32_t*>(a.out_lo + o) = 0u;
-            }
-        return;
-    }
-
-    const int n_pg = (K_tot + P - 1) / P;
-    const int pps = (n_pg + S - 1) / S;
-    const int pg0 = sp * pps, pg1 = min(n_pg, pg0 + pps);
-
-    for (int i = tid; i < RPG * HEAD_DIM; i += ATT_THREADS) {
-        const int j = i / HEAD_DIM, dd = i % HEAD_DIM;
-        qs[i] = s_act[j] ? a.q[(size_t)(g * rpg + j) * a.ldq + h * HEAD_DIM + dd] * 0.125f : 0.f;  // 1/sqrt(64)
-    }
-    const int n_ids = min(ID_CAP, max(0, pg1 - pg0));
-    for (int i = tid; i < n_ids; i += ATT_THREADS) s_ids[i] = a.block_table[(size_t)seq * a.bt_stride + pg0 + i];
-    __syncthreads();
-    // batches of one staging slot each: batch i = pages pg0 + i*ppb .. in slot i % ATT_STAGES
-    const int n_batches = (pg1 - pg0 + pages_per_batch - 1) / pages_per_batch;
-    if (tid == 0) {
-        for (int i = 0; i < ATT_STAGES; ++i) s_armed[i] = 0;
-        for (int i = 0; i < ATT_STAGES && i < n_batches; ++i) {
-            const int b0 = pg0 + i * pages_per_batch, b1 = min(pg1, b0 + pages_per_batch);
-            const int from = i == 0 ? b0 + n_pre : b0;  // batch 0's first pages came before the wait
-            s_armed[i] = stage_pages(a, seq, from, b1, i * pages_per_batch + (from - b0), Ks, Vs, kv_head_off,
-                                     v_off, &hbar[i], s_ids, pg0, n_ids);
-        }
-    }
-    __syncthreads();
+    if (a.out_hi)  // groups without keys: zero operand rows, a warp per group
+        for (int gr = jc + warp * gridDim.x; gr < a.groups; gr += NW * gridDim.x)
+            if (group_of(gr).keys == 0)
+                for (int row_j = 0; row_j < rpg; ++row_j) {
+                    const size_t o = ((size_t)gr * rpg + row_j) * a.ldb + h * HEAD_DIM + 2 * lane;
+                    *reinterpret_cast<uint32_t*>(a.out_hi + o) = 0u;
+                    *reinterpret_cast<uint32_t*>(a.out_lo + o) = 0u;
+                }
 
     // per-warp tensor-core tiles with the keys as the M side: S^T = K Q^T (16 keys x the 8 query
     // rows; the queries' bf16 hi and lo parts are two N = 8 operands) and O^T += V^T P^T (head
-    // dims x query rows, P^T's hi and lo parts added into the same accumulator).  Lane (g, c2):
-    // keys g, g + 8 of a tile and queries c2, c2 + 1 in S^T; head dims g, g + 8 of each 16-dim
+    // dims x query rows, P^T's hi and lo parts added into the same accumulator).  Lane (g8, c2):
+    // keys g8, g8 + 8 of a tile and queries c2, c2 + 1 in S^T; head dims g8, g8 + 8 of each 16-dim
     // block and queries c2, c2 + 1 in O^T.
     const int g8 = lane >> 2, c2 = (lane & 3) * 2;
-    bool qon[2];
-    int qpos[2];
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        qon[j] = s_act[c2 + j] != 0;
-        qpos[j] = qon[j] ? s_pos[c2 + j] : -1;
-    }
-    uint32_t qhi[4][2], qlo[4][2];  // B operand of S^T: query row g8, dims ks * 16 + 8 hh + c2, + 1
-    {
-        const bool on = s_act[g8] != 0;
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const int k = ks * 16 + hh * 8 + c2;
-                split2(on ? qs[g8 * HEAD_DIM + k] : 0.f, on ? qs[g8 * HEAD_DIM + k + 1] : 0.f, qhi[ks][hh],
-                       qlo[ks][hh]);
-            }
-    }
-    float m_w[2] = {-INFINITY, -INFINITY}, l_w[2] = {0.f, 0.f};
-    float o[4][4];  // O^T block dp: dims dp * 16 + g8 (0, 1) and + 8 (2, 3), queries c2 + (i & 1)
-#pragma unroll
-    for (int j = 0; j < 4; ++j)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) o[j][i] = 0.f;
-    const int swz = a.kv_swizzled ? 7 : 0;
+    // partials: a CTA shares at most its first group (slot 0) and its last (slot 1: begun here)
+    auto part_of = [&](int cta, int c_first) {
+        return a.ws_part + (((size_t)(h * J + cta) * 2 + (cta == c_first ? 1 : 0)) * RPG) * PART;
+    };
     bool ok = true;
-    uint32_t hphase[ATT_STAGES] = {};
-    for (int i = 0; i < n_batches; ++i) {
-        const int half = i % ATT_STAGES;
-        const int bp = pg0 + i * pages_per_batch;
-        const int nk = min(pages_per_batch, pg1 - bp) * P;
-        if (i == 0 && n_pre > 0) ok = mbar_wait(&bar, 0, a.err) && ok;
-        if (s_armed[half]) {
-            ok = mbar_wait(&hbar[half], hphase[half], a.err) && ok;
-            hphase[half] ^= 1u;
+    for (int i = 0; i < n && ok; ++g, cb = 0) {
+        const Group x = group_of(g);
+        if (x.keys == 0) continue;
+        const int gpages = (x.keys + P - 1) / P, gnb = batches(x);
+        // ---- the group's rows (lanes 0..7 of every warp) and its queries, loaded together ----
+        int row_pos = -1;
+        if (a.plan == PLAN_DEVICE) {
+            if (lane < x.rows) row_pos = x.keys - x.rows + lane;
+        } else if (lane < rpg && g * rpg + lane < a.rows) {
+            const int rs = a.row_seq[g * rpg + lane], rp = a.row_pos[g * rpg + lane];
+            row_pos = rs >= 0 ? rp : -1;
         }
-        const uint32_t kb = smem_addr(Ks + (size_t)half * HALF_KEYS * HEAD_DIM);
-        const uint32_t vb = smem_addr(Vs + (size_t)half * HALF_KEYS * HEAD_DIM);
-        for (int kt = warp * 16; kt < nk && ok; kt += (ATT_THREADS / 32) * 16) {
-            float sh[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};  // hi and lo parts: own chains
-            {
-                // A = K rows kt..kt+15: matrices (keys 0-7 | 8-15) x (dims 0-7 | 8-15) of the k-step
-                const int key = kt + (lane & 7) + (((lane >> 3) & 1) << 3), chalf = lane >> 4;
+        uint32_t qhi[4][2], qlo[4][2];  // B operand of S^T: query row g8, dims ks * 16 + 8 hh + c2, + 1
+        int qpos[2];
+        unsigned act;
+        {
+            const bool in = g8 < rpg && g * rpg + g8 < a.rows;
+            const float* qr = a.q + (size_t)(g * rpg + (in ? g8 : 0)) * a.ldq + h * HEAD_DIM + c2;
+            float2 v[4][2];
 #pragma unroll
-                for (int ks = 0; ks < 4; ++ks) {
-                    uint32_t ka[4];
-                    ldsm_x4(ka, kb + key * 128 + ((uint32_t)((2 * ks + chalf) ^ (key & swz)) << 4));
-                    const uint32_t bh[2] = {qhi[ks][0], qhi[ks][1]}, bl[2] = {qlo[ks][0], qlo[ks][1]};
-                    mma_bf16(sh, ka, bh);
-                    mma_bf16(sl, ka, bl);
+            for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh)
+                    v[ks][hh] = make_float2(qr[ks * 16 + hh * 8], qr[ks * 16 + hh * 8 + 1]);
+            act = __ballot_sync(FULL_MASK, row_pos >= 0);
+            const float scale = in && (act >> g8 & 1) ? 0.125f * LOG2E : 0.f;  // 1/sqrt(64); scores in log2 units
+#pragma unroll
+            for (int j = 0; j < 2; ++j) qpos[j] = __shfl_sync(FULL_MASK, row_pos, c2 + j);
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh)
+                    split2(scale != 0.f ? v[ks][hh].x * scale : 0.f, scale != 0.f ? v[ks][hh].y * scale : 0.f,
+                           qhi[ks][hh], qlo[ks][hh]);
+        }
+        float m_w[2] = {-INFINITY, -INFINITY}, l_w[2] = {0.f, 0.f};
+        float o[4][4];  // O^T block dp: dims dp * 16 + g8 (0, 1) and + 8 (2, 3), queries c2 + (i & 1)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[j][e] = 0.f;
+        const int gs = x0 + i - cb;  // the group's first batch in the stream
+        const int cend = min(gnb, cb + n - i);
+        for (; cb < cend; ++cb, ++i) {
+            const int slot = i % ATT_STAGES, key0 = cb * KB;
+            const int nk = min(ppb, gpages - cb * ppb) * P;
+            ok = mbar_wait(&bar[slot], (uint32_t)(i / ATT_STAGES) & 1, a.err) && ok;
+            const uint32_t kb = smem_addr(Ks + (size_t)slot * KB * HEAD_DIM);
+            const uint32_t vb = smem_addr(Vs + (size_t)slot * KB * HEAD_DIM);
+            for (int kt = warp * 16; kt < nk && ok; kt += NW * 16) {
+                float sh[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};  // hi and lo parts: own chains
+                {
+                    // A = K rows kt..kt+15: matrices (keys 0-7 | 8-15) x (dims 0-7 | 8-15) of the k-step
+                    const int key = kt + (lane & 7) + (((lane >> 3) & 1) << 3), chalf = lane >> 4;
+#pragma unroll
+                    for (int ks = 0; ks < 4; ++ks) {
+                        uint32_t ka[4];
+                        ldsm_x4(ka, kb + key * 128 + ((uint32_t)((2 * ks + chalf) ^ (key & 7)) << 4));
+                        const uint32_t bh[2] = {qhi[ks][0], qhi[ks][1]}, bl[2] = {qlo[ks][0], qlo[ks][1]};
+                        mma_bf16(sh, ka, bh);
+                        mma_bf16(sl, ka, bl);
+                    }
+                }
+                // this lane's scores: keys kt + g8 (e = 0, 1) and kt + g8 + 8 (e = 2, 3), query c2 + (e & 1)
+                float sv[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    sv[e] = key0 + kt + g8 + (e >> 1) * 8 <= qpos[e & 1] ? sh[e] + sl[e] : -INFINITY;
+                // weights are taken relative to the row's reference m_w, a bound of the scores up to a factor
+                // 2^RESCALE: it moves (a maximum over the lanes, the sums rescaled) only past that
+                float t0 = fmaxf(sv[0], sv[2]), t1 = fmaxf(sv[1], sv[3]);
+                if (__any_sync(FULL_MASK, t0 > m_w[0] + RESCALE || t1 > m_w[1] + RESCALE)) {
+#pragma unroll
+                    for (int off = 4; off < 32; off <<= 1) {  // over the tile's keys: lanes g8
+                        t0 = fmaxf(t0, __shfl_xor_sync(FULL_MASK, t0, off));
+                        t1 = fmaxf(t1, __shfl_xor_sync(FULL_MASK, t1, off));
+                    }
+                    const float mn[2] = {fmaxf(m_w[0], t0), fmaxf(m_w[1], t1)};
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const float corr = m_w[j] == -INFINITY ? 1.f : ex2(m_w[j] - mn[j]);  // (no sums yet)
+                        l_w[j] *= corr;
+                        m_w[j] = mn[j];
+#pragma unroll
+                        for (int dp = 0; dp < 4; ++dp) {
+                            o[dp][j] *= corr;
+                            o[dp][2 + j] *= corr;
+                        }
+                    }
+                }
+                float pv[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) pv[e] = sv[e] == -INFINITY ? 0.f : ex2(sv[e] - m_w[e & 1]);
+                l_w[0] += pv[0] + pv[2];
+                l_w[1] += pv[1] + pv[3];
+                // P^T as the B operand (keys x queries): this lane holds rows g8 (keys) and columns c2
+                // (queries) of each 8 x 8 block; its transpose is the operand's layout (query g8, keys c2, + 1)
+                uint32_t ph0, pl0, ph1, pl1;
+                split2(pv[0], pv[1], ph0, pl0);  // keys g8
+                split2(pv[2], pv[3], ph1, pl1);  // keys g8 + 8
+                const uint32_t bph[2] = {movmatrix_trans(ph0), movmatrix_trans(ph1)};
+                const uint32_t bpl[2] = {movmatrix_trans(pl0), movmatrix_trans(pl1)};
+                // A = V^T: matrices (dims 0-7 | 8-15 of block dp) x (keys 0-7 | 8-15), from the key rows
+                const int vkey = kt + (lane & 7) + ((lane >> 4) << 3), vhalf = (lane >> 3) & 1;
+#pragma unroll
+                for (int dp = 0; dp < 4; ++dp) {
+                    uint32_t va[4];
+                    ldsm_x4_t(va, vb + vkey * 128 + ((uint32_t)((2 * dp + vhalf) ^ (vkey & 7)) << 4));
+                    mma_bf16(o[dp], va, bph);
+                    mma_bf16(o[dp], va, bpl);
                 }
             }
-            // this lane's scores: keys kt + g8 (i = 0, 1) and kt + g8 + 8 (i = 2, 3), query c2 + (i & 1)
-            float sv[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int kp = bp * P + kt + g8 + (i >> 1) * 8, j = i & 1;
-                const float v = sh[i] + sl[i];
-                sv[i] = qon[j] && kp <= qpos[j] && kp < K_tot ? v : -INFINITY;
-            }
-            float t0 = fmaxf(sv[0], sv[2]), t1 = fmaxf(sv[1], sv[3]);  // over the tile's keys: lanes g8
-#pragma unroll
-            for (int off = 4; off < 32; off <<= 1) {
-                t0 = fmaxf(t0, __shfl_xor_sync(FULL_MASK, t0, off));
-                t1 = fmaxf(t1, __shfl_xor_sync(FULL_MASK, t1, off));
-            }
-            const float mn[2] = {fmaxf(m_w[0], t0), fmaxf(m_w[1], t1)};
-            float corr[2];
-#pragma unroll
-            for (int j = 0; j < 2; ++j)
-                corr[j] = mn[j] == -INFINITY ? 1.f : (m_w[j] == -INFINITY ? 0.f : expf(m_w[j] - mn[j]));
-            float pv[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) pv[i] = sv[i] == -INFINITY ? 0.f : expf(sv[i] - mn[i & 1]);
-            l_w[0] = l_w[0] * corr[0] + (pv[0] + pv[2]);
-            l_w[1] = l_w[1] * corr[1] + (pv[1] + pv[3]);
-            m_w[0] = mn[0];
-            m_w[1] = mn[1];
-#pragma unroll
-            for (int dp = 0; dp < 4; ++dp) {
-                o[dp][0] *= corr[0];
-                o[dp][1] *= corr[1];
-                o[dp][2] *= corr[0];
-                o[dp][3] *= corr[1];
-            }
-            // P^T as the B operand (keys x queries): this lane holds rows g8 (keys) and columns c2 (queries)
-            // of each 8 x 8 block; its transpose is the operand's layout (query g8, keys c2, c2 + 1)
-            uint32_t ph0, pl0, ph1, pl1;
-            split2(pv[0], pv[1], ph0, pl0);  // keys g8
-            split2(pv[2], pv[3], ph1, pl1);  // keys g8 + 8
-            const uint32_t bph[2] = {movmatrix_trans(ph0), movmatrix_trans(ph1)};
-            const uint32_t bpl[2] = {movmatrix_trans(pl0), movmatrix_trans(pl1)};
-            // A = V^T: matrices (dims 0-7 | 8-15 of block dp) x (keys 0-7 | 8-15), from the key rows
-            const int vkey = kt + (lane & 7) + ((lane >> 4) << 3), vhalf = (lane >> 3) & 1;
-#pragma unroll
-            for (int dp = 0; dp < 4; ++dp) {
-                uint32_t va[4];
-                ldsm_x4_t(va, vb + vkey * 128 + ((uint32_t)((2 * dp + vhalf) ^ (vkey & swz)) << 4));
-                mma_bf16(o[dp], va, bph);
-                mma_bf16(o[dp], va, bpl);
-            }
+            __syncthreads();  // every warp is done with this slot
+            if (warp == 0 && staged < n) stage_next();
         }
-        __syncthreads();  // every warp is done with this slot
-        if (tid == 0 && i + ATT_STAGES < n_batches) {
-            const int b0 = pg0 + (i + ATT_STAGES) * pages_per_batch, b1 = min(pg1, b0 + pages_per_batch);
-            s_armed[half] = stage_pages(a, seq, b0, b1, half * pages_per_batch, Ks, Vs, kv_head_off, v_off,
-                                        &hbar[half], s_ids, pg0, n_ids);
-        }
-        __syncthreads();
-    }
-    if (!__syncthreads_and(ok)) {  // error word set; let copies in flight land before leaving
-        if (n_pre > 0) mbar_wait(&bar, 0, nullptr);
-        for (int hb = 0; hb < ATT_STAGES; ++hb)
-            if (s_armed[hb]) mbar_wait(&hbar[hb], hphase[hb], nullptr);
-        return;
-    }
-    // merge the warps' (max, sum, out) per row through the staging area:
-    // warp j then holds row j's (m_run, l_run) and output dims 2 lane, 2 lane + 1
-#pragma unroll
-    for (int j = 0; j < 2; ++j)  // each lane summed its own keys; the query's keys span lanes g8
-#pragma unroll
-        for (int off = 4; off < 32; off <<= 1) l_w[j] += __shfl_xor_sync(FULL_MASK, l_w[j], off);
-    float* wst = reinterpret_cast<float*>(Ks);  // [warps][RPG][PART]
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        float* ws = wst + ((size_t)warp * RPG + c2 + j) * PART;
-        if (g8 == 0) {
-            ws[0] = m_w[j];
-            ws[1] = l_w[j];
-        }
-#pragma unroll
-        for (int dp = 0; dp < 4; ++dp) {
-            ws[2 + dp * 16 + g8] = o[dp][j];
-            ws[2 + dp * 16 + g8 + 8] = o[dp][2 + j];
-        }
-    }
-    __syncthreads();
-    constexpr int NW = ATT_THREADS / 32;
-    if (tid < NW * RPG) {
-        const int w = tid / RPG, j = tid % RPG;
-        float M = -INFINITY;
-#pragma unroll
-        for (int v = 0; v < NW; ++v) M = fmaxf(M, wst[((size_t)v * RPG + j) * PART]);
-        const float mw = wst[((size_t)w * RPG + j) * PART];
-        s_scale[w][j] = mw == -INFINITY ? 0.f : expf(mw - M);
-    }
-    __syncthreads();
-    // rows warp, warp + NW, ...: (max, sum, output dims 2 lane, 2 lane + 1) over this CTA's keys
-    constexpr int RPW = (RPG + NW - 1) / NW;  // rows per warp
-    float m_run[RPW], l_run[RPW], acc0[RPW], acc1[RPW];
-#pragma unroll
-    for (int q = 0; q < RPW; ++q) {
-        const int row_j = warp + q * NW;
-        m_run[q] = -INFINITY;
-        l_run[q] = acc0[q] = acc1[q] = 0.f;
-        if (row_j >= RPG) continue;
-#pragma unroll
-        for (int w = 0; w < NW; ++w) {
-            const float sc = s_scale[w][row_j];
-            const float* ws = wst + ((size_t)w * RPG + row_j) * PART;
-            m_run[q] = fmaxf(m_run[q], ws[0]);
-            l_run[q] = fmaf(sc, ws[1], l_run[q]);
-            acc0[q] = fmaf(sc, ws[2 + 2 * lane], acc0[q]);
-            acc1[q] = fmaf(sc, ws[3 + 2 * lane], acc1[q]);
-        }
-    }
-    if (S == 1) {
-#pragma unroll
-        for (int q = 0; q < RPW; ++q) {
-            const int row_j = warp + q * NW;
-            if (row_j < RPG && s_act[row_j]) {
-                put(row_j, acc0[q] / l_run[q], acc1[q] / l_run[q]);
-            } else if (row_j < rpg && a.out_hi) {
-                put(row_j, 0.f, 0.f);
-            }
-        }
-        return;
-    }
+        ok = __syncthreads_and(ok) != 0;
+        if (!ok) break;
 
-    float* part = a.ws_part + (((size_t)(g * H + h) * S + sp) * RPG) * PART;
+        // ---- the group's keys of this CTA are done: merge the warps' (max, sum, out) per row ----
 #pragma unroll
-    for (int q = 0; q < RPW; ++q) {
-        const int row_j = warp + q * NW;
-        if (row_j >= RPG) continue;
-        float* pj = part + row_j * PART;
-        if (lane == 0) {
-            pj[0] = m_run[q];
-            pj[1] = l_run[q];
-        }
-        pj[2 + 2 * lane] = acc0[q];
-        pj[3 + 2 * lane] = acc1[q];
-    }
-    __threadfence();
-    __syncthreads();
-    trace_mark(a.trace, 2);  // split partials written
-    if (tid == 0) s_last = atomicAdd(a.ws_count + g * H + h, 1) == S - 1;
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-
+        for (int j = 0; j < 2; ++j)  // each lane summed its own keys; the query's keys span lanes g8
+#pragma unroll
+            for (int off = 4; off < 32; off <<= 1) l_w[j] += __shfl_xor_sync(FULL_MASK, l_w[j], off);
+        // the CTAs that share the group: those of its first and last batch
+        const int c_first = a.whole ? jc : (int)(((long long)(gs + 1) * J - 1) / T);
+        const int parts = a.whole ? 1 : (int)(((long long)(gs + gnb) * J - 1) / T) - c_first + 1;
 #pragma unroll 1
-    for (int row_j = warp; row_j < RPG; row_j += NW) {
-        if (!s_act[row_j]) {
-            if (row_j < rpg && a.out_hi) put(row_j, 0.f, 0.f);
-            continue;
-        }
-        // lane s holds split s's (max, sum); every split's output pair is
-        // loaded before any is used, so the merge costs one L2 round trip
-        const float* base = a.ws_part + ((size_t)(g * H + h) * S * RPG) * PART + row_j * PART;
-        const size_t sstride = (size_t)RPG * PART;
-        float ms = -INFINITY, ls = 0.f;
-        if (lane < S) {
-            ms = __ldcg(base + lane * sstride);
-            ls = __ldcg(base + lane * sstride + 1);
-        }
-        float o0[MAX_SPLITS], o1[MAX_SPLITS];
+        for (int r0 = 0; r0 < rpg; r0 += MROWS) {
+            if ((c2 & ~(MROWS - 1)) == r0) {
 #pragma unroll
-        for (int sx = 0; sx < MAX_SPLITS; ++sx) {
-            o0[sx] = sx < S ? __ldcg(base + sx * sstride + 2 + 2 * lane) : 0.f;
-            o1[sx] = sx < S ? __ldcg(base + sx * sstride + 3 + 2 * lane) : 0.f;
-        }
-        const float M = warp_max(ms);
-        const float w = (ms == -INFINITY) ? 0.f : expf(ms - M);
-        const float L = warp_sum(w * ls);
-        float r0 = 0.f, r1 = 0.f;
+                for (int j = 0; j < 2; ++j) {
+                    float* ws = wst + ((size_t)warp * MROWS + (c2 & (MROWS - 1)) + j) * PART;
+                    if (g8 == 0) {
+                        ws[0] = m_w[j];
+                        ws[1] = l_w[j];
+                    }
 #pragma unroll
-        for (int sx = 0; sx < MAX_SPLITS; ++sx) {
-            const float ws = __shfl_sync(FULL_MASK, w, sx);
-            r0 = fmaf(ws, o0[sx], r0);
-            r1 = fmaf(ws, o1[sx], r1);
+                    for (int dp = 0; dp < 4; ++dp) {
+                        ws[2 + dp * 16 + g8] = o[dp][j];
+                        ws[2 + dp * 16 + g8 + 8] = o[dp][2 + j];
+                    }
+                }
+            }
+            __syncthreads();
+            const int row_j = r0 + warp;  // warp w merges row r0 + w: output dims 2 lane, 2 lane + 1
+            if (row_j < rpg) {
+                float M = -INFINITY, L = 0.f, y0 = 0.f, y1 = 0.f;
+#pragma unroll
+                for (int w = 0; w < NW; ++w) M = fmaxf(M, wst[((size_t)w * MROWS + warp) * PART]);
+#pragma unroll
+                for (int w = 0; w < NW; ++w) {
+                    const float* ws = wst + ((size_t)w * MROWS + warp) * PART;
+                    const float sc = ws[0] == -INFINITY ? 0.f : ex2(ws[0] - M);
+                    L = fmaf(sc, ws[1], L);
+                    y0 = fmaf(sc, ws[2 + 2 * lane], y0);
+                    y1 = fmaf(sc, ws[3 + 2 * lane], y1);
+                }
+                if (parts > 1) {
+                    float* pj = part_of(jc, c_first) + row_j * PART;
+                    if (lane == 0) {
+                        pj[0] = M;
+                        pj[1] = L;
+                    }
+                    pj[2 + 2 * lane] = y0;
+                    pj[3 + 2 * lane] = y1;
+                } else if (act >> row_j & 1) {
+                    put(g, row_j, y0 / L, y1 / L);
+                } else if (a.out_hi) {
+                    put(g, row_j, 0.f, 0.f);
+                }
+            }
+            __syncthreads();  // wst may be written again
         }
-        put(row_j, r0 / L, r1 / L);
+        if (parts > 1 && tid == 0) {
+            int* sh = s_share[jc == c_first ? 1 : 0];
+            sh[0] = g;
+            sh[1] = c_first;
+            sh[2] = parts;
+            sh[3] = (int)act;
+        }
     }
-    if (tid == 0) a.ws_count[g * H + h] = 0;
+    // ---- the shared groups (at most the CTA's first and its last): the CTA that finishes one last merges
+    // its parts; both counters are asked at once, after the stream ----
+    __threadfence();
+    __syncthreads();
+    trace_mark(a.trace, 2);  // partials written
+    if (tid < 2) {
+        const int* sh = s_share[tid];
+        s_last[tid] = ok && sh[2] > 0 ? atomicAdd(a.ws_count + (size_t)sh[0] * H + h, 1) == sh[2] - 1 : 0;
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (int k = 0; k < 2; ++k) {
+        if (!s_last[k]) continue;
+        __threadfence();
+        const int sg = s_share[k][0], c_first = s_share[k][1], parts = s_share[k][2];
+        const unsigned act = (unsigned)s_share[k][3];
+        for (int row_j = warp; row_j < rpg; row_j += NW) {
+            if (!(act >> row_j & 1)) {
+                if (a.out_hi) put(sg, row_j, 0.f, 0.f);
+                continue;
+            }
+            // the parts in stream order, four loaded at a time
+            float M = -INFINITY, L = 0.f, y0 = 0.f, y1 = 0.f;
+            for (int p0 = 0; p0 < parts; p0 += 4) {
+                float m[4], l[4], v0[4], v1[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const bool have = p0 + q < parts;
+                    const float* pj = part_of(c_first + (have ? p0 + q : 0), c_first) + row_j * PART;
+                    m[q] = have ? __ldcg(pj) : -INFINITY;
+                    l[q] = have ? __ldcg(pj + 1) : 0.f;
+                    v0[q] = have ? __ldcg(pj + 2 + 2 * lane) : 0.f;
+                    v1[q] = have ? __ldcg(pj + 3 + 2 * lane) : 0.f;
+                }
+                const float Mn = fmaxf(fmaxf(M, fmaxf(m[0], m[1])), fmaxf(m[2], m[3]));
+                const float old = M == -INFINITY ? 0.f : ex2(M - Mn);
+                L *= old;
+                y0 *= old;
+                y1 *= old;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float w = m[q] == -INFINITY ? 0.f : ex2(m[q] - Mn);
+                    L = fmaf(w, l[q], L);
+                    y0 = fmaf(w, v0[q], y0);
+                    y1 = fmaf(w, v1[q], y1);
+                }
+                M = Mn;
+            }
+            put(sg, row_j, y0 / L, y1 / L);
+        }
+        if (tid == 0) a.ws_count[(size_t)sg * H + h] = 0;
+    }
+    if (!ok && warp == 0) {  // error word set; let copies in flight land before leaving
+        for (int i = max(0, staged - ATT_STAGES); i < staged; ++i)
+            mbar_wait(&bar[i % ATT_STAGES], (uint32_t)(i / ATT_STAGES) & 1, nullptr);
+    }
 }
 
 }  // namespace
 
-size_t attn_workspace_floats(int groups, int n_heads, int n_splits, int /*rows_per_group*/) {
-    return (size_t)groups * n_heads * n_splits * RPG * PART;
+size_t attn_workspace_floats(int n_heads, int ctas) {
+    return ctas > 1 ? (size_t)n_heads * ctas * 2 * RPG * PART : 0;
 }
 
 size_t attn_smem_bytes(int page_size) {
-    return (size_t)2 * ATT_STAGES * half_keys(page_size) * HEAD_DIM * 2 + (size_t)RPG * HEAD_DIM * 4;
+    return (size_t)2 * ATT_STAGES * half_keys(page_size) * HEAD_DIM * 2 + (size_t)NW * MROWS * PART * 4 + 1024;
 }
 
-int attn_splits_for(int groups, int n_heads, int page_size, int max_keys, int num_sms) {
-    const int max_pages = (max_keys + page_size - 1) / page_size;
-    int s = num_sms / max(1, groups * n_heads);
-    s = max(1, min(min(s, max_pages), MAX_SPLITS));
-    return s;
+int attn_ctas_per_sm(int page_size) { return page_size > 64 ? ATTN_CTAS_PER_SM / 2 : ATTN_CTAS_PER_SM; }
+
+int attn_ctas_for(int groups, int n_heads, int page_size, int max_keys, int num_sms) {
+    // one wave of resident CTAs while they have batches; of a long context's batches at least two each
+    // (sharing a group costs its CTAs a partial each and a merge)
+    const int nb = (max_keys + half_keys(page_size) - 1) / half_keys(page_size);  // batches per group
+    const long long want = (long long)groups * (nb >= 8 ? nb / 2 : nb);
+    return (int)max(1ll, min(want, (long long)max(1, attn_ctas_per_sm(page_size) * num_sms / n_heads)));
 }
 
-cudaError_t launch_attention(const AttnArgs& a, int groups, cudaStream_t s, bool pdl) {
-    if (a.rows_per_group < 1 || a.rows_per_group > RPG || half_keys(a.page_size) % a.page_size != 0 ||
-        a.n_splits < 1 || a.n_splits > MAX_SPLITS)
+bool attn_whole_groups(int groups, int n_heads, int page_size, int max_keys, int num_sms) {
+    // contexts of a batch or two that fill the GPU: a plan and a merge would cost more than they share out
+    // (20 slots of 33-99 keys, 16 heads: 8.5 vs 10.4 us)
+    return max_keys <= 2 * half_keys(page_size) && (long long)groups * n_heads >= num_sms;
+}
+
+template <bool PLAIN>
+static cudaError_t launch_attn_t(const AttnArgs& a, const CUtensorMap& map, cudaStream_t s, bool pdl) {
+    if (a.rows_per_group < 1 || a.rows_per_group > RPG || half_keys(a.page_size) % a.page_size != 0 || a.groups < 1 ||
+        (!a.whole && a.ctas < 1) || (a.plan != PLAN_ROWS && a.plan != PLAN_DEVICE))
         return cudaErrorInvalidValue;
     const size_t smem = attn_smem_bytes(a.page_size);
-    cudaError_t e = ensure_kernel_smem(reinterpret_cast<const void*>(attn_kernel), smem);
+    auto kern = attn_kernel<PLAIN>;
+    cudaError_t e = ensure_kernel_smem(reinterpret_cast<const void*>(kern), smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.n_splits, a.n_heads, groups);
+    cfg.gridDim = dim3(a.whole ? a.groups : a.ctas, a.n_heads);
     cfg.blockDim = dim3(ATT_THREADS);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
@@ -528,7 +618,21 @@ cudaError_t launch_attention(const AttnArgs& a, int groups, cudaStream_t s, bool
     attr[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, attn_kernel, a);
+    return cudaLaunchKernelEx(&cfg, kern, a, map);
+}
+
+cudaError_t launch_attention(const AttnArgs& a, cudaStream_t s, bool pdl) {
+    return launch_attn_t<false>(a, CUtensorMap{}, s, pdl);
+}
+
+cudaError_t launch_attention_plain(const AttnArgs& a, cudaStream_t s) {
+    if (a.plan != PLAN_ROWS) return cudaErrorInvalidValue;
+    // [page][row of the page (layer, keys | values, head, key)][64]; the number of pages is not known here
+    // (the kernel reads only pages of the block table)
+    CUtensorMap map;
+    if (tc_encode_rows(&map, a.kv_pool, (uint64_t)a.page_elems / HEAD_DIM, (uint32_t)a.page_size) != 0)
+        return cudaErrorInvalidValue;
+    return launch_attn_t<true>(a, map, s, false);
 }
 
 }  // namespace mtp
@@ -564,7 +668,7 @@ extern "C" MTP_API int mtp_attention_noalloc(const mtp_attention_args* args, voi
         return mtp::report_error(MTP_ERR_CUDA, msg);
     }
     const cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
-    e = cudaMemsetAsync(static_cast<char*>(scratch) + p.part_bytes, 0, p.count_bytes, s);  // merge counters
+    e = cudaMemsetAsync(scratch, 0, p.count_bytes, s);  // merge counters
     if (e != cudaSuccess) return mtp::report_error(MTP_ERR_CUDA, cudaGetErrorString(e));
-    return mtp::attention_standalone_launch(args, p, scratch, s);
+    return mtp::attention_standalone_launch(args, p, scratch, MTP_ATTENTION_NOALLOC_SCRATCH_BYTES, s);
 }

@@ -535,7 +535,7 @@ int attn_tc_splits_for(int tiles, int n_heads, int max_keys, int num_sms) {
 }
 
 cudaError_t launch_attention_tc(const AttnArgs& a, cudaStream_t s, bool pdl) {
-    if (a.rows < 1 || a.n_splits < 1 || a.n_splits > 0xffff || !a.kv_swizzled || (a.page_size & 7) ||
+    if (a.rows < 1 || a.n_splits < 1 || a.n_splits > 0xffff || (a.page_size & 7) ||
         PA_KEYS % a.page_size || (a.ldq & 3) || (a.out && (a.ldo & 3)) || (a.out_hi && (a.ldb & 7)) ||
         (reinterpret_cast<uintptr_t>(a.q) & 15))
         return cudaErrorInvalidValue;

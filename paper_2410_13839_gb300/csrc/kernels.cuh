@@ -78,22 +78,25 @@ struct AttnArgs {
     __nv_bfloat16* out_hi; __nv_bfloat16* out_lo; int ldb;  // or null: output rows as bf16 hi + lo (the
                                                // W_o GEMM's operand; rows of no sequence written as zeros)
     float* ws_part; int* ws_count;             // split partials and per-(group, head) counters
-    int rows_per_group, n_heads, page_size, n_splits;
+    int rows_per_group, n_heads, page_size;
+    int groups, ctas;                          // attn_kernel: groups of rows, CTAs per head that share them out
+    int whole;                                 // attn_kernel: or a CTA per group and head (no partials)
+    int n_splits;                              // attention_tc: key splits
     int plan;
-    const int* seq_len; const int* seq_new; int seq_base;   // PLAN_DEVICE
-    int val_seq, val_old, val_new;                           // PLAN_VALUE
+    const int* seq_len; const int* seq_new; const int* active; const int* done;  // PLAN_DEVICE: group g is slot g
     int* err;
     unsigned long long* trace;
-    int kv_swizzled;                                         // pages store chunk c of key row t at c ^ (t & 7)
-    int rows;                                                // attention_tc: rows of the pass (tiles of 128)
+    int rows;                                                // rows of the pass (attention_tc: tiles of 128)
 };
 
-constexpr int ATTN_CTAS_PER_SM = 4;  // attn_kernel: 128 threads x at most 128 registers, ~51 KB of shared memory
-constexpr int ATTN_MAX_SPLITS = 32;  // key splits one launch merges
-size_t attn_workspace_floats(int groups, int n_heads, int n_splits, int rows_per_group);
+constexpr int ATTN_CTAS_PER_SM = 4;  // attn_kernel: 128 threads x at most 128 registers, ~54 KB of shared memory
+// CTAs per head of a launch (AttnArgs::ctas), and the floats of its partials (ws_part)
+int attn_ctas_for(int groups, int n_heads, int page_size, int max_keys, int num_sms);
+bool attn_whole_groups(int groups, int n_heads, int page_size, int max_keys, int num_sms);  // AttnArgs::whole
+size_t attn_workspace_floats(int n_heads, int ctas);
 size_t attn_smem_bytes(int page_size);
-int attn_splits_for(int groups, int n_heads, int page_size, int max_keys, int num_sms);
-cudaError_t launch_attention(const AttnArgs& a, int groups, cudaStream_t s, bool pdl);
+cudaError_t launch_attention(const AttnArgs& a, cudaStream_t s, bool pdl);   // the cache's swizzled pages
+cudaError_t launch_attention_plain(const AttnArgs& a, cudaStream_t s);       // plain pages, PLAN_ROWS
 // Tensor-core (tcgen05) causal attention of prompt rows: tiles of 128 rows of
 // any slots, 128-key items, swizzled pages only; grid (n_splits, heads, tiles).
 size_t attn_tc_workspace_floats(int tiles, int n_heads, int n_splits);
@@ -345,6 +348,9 @@ struct TcGemm {
 // tensor already stores chunk c of row r at c ^ (r & 7) (copied verbatim).
 int tc_encode_2d(CUtensorMap* map, const void* base, uint64_t inner, uint64_t rows, uint32_t box_rows,
                  bool pre_swizzled);
+// 3-D bf16 tensor map [blocks][rows_per_block][64] (blocks: unbounded) with boxes of box_rows rows of one
+// block, copied with the 128-byte swizzle.
+int tc_encode_rows(CUtensorMap* map, const void* base, uint64_t rows_per_block, uint32_t box_rows);
 int tc_tile_rows(int m);          // activation rows per tile for m rows: 32, 64 or 128
 cudaError_t launch_tc_gemm(const TcGemm& g, cudaStream_t s, bool pdl);
 // The same products over many rows by a persistent kernel of CTA pairs (tc_gemm_pair.cu): tiles of
@@ -393,15 +399,17 @@ cudaError_t ensure_kernel_smem(const void* kernel, size_t bytes, bool max_shared
 // the per-(group, head) merge counters (count_bytes), which must be zero when
 // a launch starts and are left zero by it.
 struct AttnStandalonePlan {
-    int groups, splits;
+    int groups, splits;  // splits: CTAs per head (mtp_attention*), key splits (mtp_attention_tc)
+    bool whole;          // mtp_attention*: a CTA per group and head instead
     size_t part_bytes, count_bytes, need;
+    size_t least;        // bytes a call is accepted with (need: what it runs fastest with)
 };
 // MTP_OK or MTP_ERR_INVALID / MTP_ERR_CUDA (message set); with check_pointers
 // the device pointers must be non-null too.
 int attention_standalone_plan(const struct ::mtp_attention_args* a, bool check_pointers, AttnStandalonePlan* p);
-// Enqueue the kernel on `stream` with `workspace` laid out as `p` describes.
+// Enqueue the kernel on `stream` with the `bytes` (>= p.least) of `workspace`: partials, then counters.
 int attention_standalone_launch(const struct ::mtp_attention_args* a, const AttnStandalonePlan& p, void* workspace,
-                                cudaStream_t stream);
+                                size_t bytes, cudaStream_t stream);
 
 // C-ABI error reporting shared by the translation units (message for mtp_last_error)
 int report_error(int code, const char* msg);

@@ -132,7 +132,8 @@ struct mtp_ctx {
     float *d_bx = nullptr, *d_bq = nullptr;
     float* d_bws = nullptr;  // attention split partials
     int* d_bwc = nullptr;    // attention split counters
-    int battn_ws_units = 1;  // (group, split) pairs the attention workspace holds
+    int battn_ctas = 1;          // most CTAs per head of an attention launch
+    size_t battn_ws_floats = 0;  // of the attention workspace
     int gemm_max_splits = 16;
     int lattice = 0;  // MTP_OPT_LATTICE
     int sampling = 0;          // MTP_OPT_SAMPLING
@@ -411,33 +412,23 @@ int run_layers_batched(mtp_ctx* c, int M, int rpg, int groups, int plan, cudaStr
         at.out_hi = c->d_ahi; at.out_lo = c->d_alo; at.ldb = d;  // straight into W_o's operand
         at.ws_part = c->d_bws; at.ws_count = c->d_bwc;
         at.rows_per_group = rpg; at.n_heads = H; at.page_size = P;
-        // key splits.  Decode steps: about 2.5 waves of CTAs at four per SM, so the slots with the
-        // longest contexts do not set the launch's length (B = 32 serving: 3 splits, 888 vs 972 us
-        // per step with one; B = 128: one split, two measured 5.6 % slower).  Prefill passes: one
-        // wave (their groups of 8 positions have similar key counts; the decode rule measured 13 %
-        // slower at B = 32).
-        {
-            int want = attn_splits_for(groups, H, P, cf.max_ctx, c->num_sms);
-            if (plan == PLAN_DEVICE) {
-                const double waves = 2.5 * ATTN_CTAS_PER_SM * c->num_sms / std::max(1, groups * H);
-                want = std::min({(int)std::lround(waves), (cf.max_ctx + P - 1) / P, ATTN_MAX_SPLITS});
-            }
-            at.n_splits = std::max(1, std::min(want, c->battn_ws_units / std::max(1, groups)));
-        }
-        at.plan = plan; at.seq_len = c->d_len; at.seq_new = c->d_npend; at.seq_base = 0;
-        at.err = c->d_err; at.kv_swizzled = 1;
+        at.groups = groups; at.rows = M;
+        at.ctas = std::min(attn_ctas_for(groups, H, P, cf.max_ctx, c->num_sms), c->battn_ctas);
+        // prefill passes (up to PREFILL_TC_ROWS rows): 8 positions see few keys more than the 8 before them, a
+        // CTA each (one prompt of 289: 14 vs 18.5 us per launch)
+        at.whole = prefill_keys > 0 || attn_whole_groups(groups, H, P, cf.max_ctx, c->num_sms);
+        at.plan = plan; at.seq_len = c->d_len; at.seq_new = c->d_npend; at.active = c->d_active; at.done = c->d_done;
+        at.err = c->d_err;
         if (prefill_keys > 0 && (c->use_attn_tc || M > PREFILL_TC_ROWS) && plan == PLAN_ROWS) {
             // tiles of 128 rows; splits as many as the batched attention workspace holds (S = 1 uses none)
             const int tiles = attn_tc_tiles(M);
-            const size_t ws_floats = attn_workspace_floats(c->battn_ws_units, H, 1, MAX_ROWS);
-            at.rows = M;
             at.n_splits = std::max(1, std::min(attn_tc_splits_for(tiles, H, prefill_keys, c->num_sms),
-                                               (int)(ws_floats / attn_tc_workspace_floats(tiles, H, 1))));
+                                               (int)(c->battn_ws_floats / attn_tc_workspace_floats(tiles, H, 1))));
             at.trace = tslot(c, MTP_K_ATTN_TC);
             LAUNCH(MTP_K_ATTN_TC, launch_attention_tc(at, s, pdl));
         } else {
             at.trace = tslot(c, MTP_K_ATTN);
-            LAUNCH(MTP_K_ATTN, launch_attention(at, groups, s, pdl));
+            LAUNCH(MTP_K_ATTN, launch_attention(at, s, pdl));
         }
         // x += attention W_o^T + b_o (the per-head W_o blocks are the k-chunks)
         MTP_TRY(gemm(W.wo, d, d, false, TC_ACCUM, c->d_bx, d, L.bo, d));
@@ -574,12 +565,12 @@ int setup_batched(mtp_ctx* c) {
     c->d_alo = reinterpret_cast<__nv_bfloat16*>(alo);
     c->d_uhi = reinterpret_cast<__nv_bfloat16*>(uhi);
     c->d_ulo = reinterpret_cast<__nv_bfloat16*>(ulo);
-    {  // attention workspace for the decode groups (slots, plus the lane's groups of as few as one row)
-        // and the prefill groups (8-row runs; one wave of CTAs where their keys are split)
-        const int gd = cf.max_batch + PREFILL_ROWS, gp = (c->bm_max + 7) / 8;
-        c->battn_ws_units = std::max(gd * attn_splits_for(gd, H, P, cf.max_ctx, c->num_sms), c->num_sms / H);
-        MTP_TRY(c->alloc(&c->d_bws, attn_workspace_floats(c->battn_ws_units, H, 1, MAX_ROWS)));
-        MTP_TRY(c->alloc(&c->d_bwc, (size_t)std::max(gd, gp) * H));
+    {  // attention workspace: one wave's partials, and those of a tensor-core prefill pass of few tiles
+        const int groups = std::max(cf.max_batch + PREFILL_ROWS, (c->bm_max + 7) / 8);  // lane: groups of one row
+        c->battn_ctas = std::max(1, ATTN_CTAS_PER_SM * c->num_sms / H);
+        c->battn_ws_floats = std::max(attn_workspace_floats(H, c->battn_ctas), attn_tc_workspace_floats(4, H, 2));
+        MTP_TRY(c->alloc(&c->d_bws, c->battn_ws_floats));
+        MTP_TRY(c->alloc(&c->d_bwc, (size_t)groups * H));
     }
     c->lmaps.resize(cf.layers);
     int bad = 0;
@@ -1176,15 +1167,22 @@ int mtp::attention_standalone_plan(const mtp_attention_args* a, bool check_point
     CUDA_TRY(cudaGetDevice(&dev));
     CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     p->groups = (a->rows + a->rows_per_group - 1) / a->rows_per_group;
-    p->splits = attn_splits_for(p->groups, a->n_heads, a->page_size, a->max_keys, sms);
-    p->part_bytes = align256(attn_workspace_floats(p->groups, a->n_heads, p->splits, a->rows_per_group) * sizeof(float));
+    p->whole = attn_whole_groups(p->groups, a->n_heads, a->page_size, a->max_keys, sms);
+    p->splits = p->whole ? 1 : attn_ctas_for(p->groups, a->n_heads, a->page_size, a->max_keys, sms);
+    p->part_bytes = align256(attn_workspace_floats(a->n_heads, p->splits) * sizeof(float));
     p->count_bytes = align256((size_t)p->groups * a->n_heads * sizeof(int));
-    p->need = p->part_bytes + p->count_bytes;
+    // a call is accepted with the partials of `parts` key splits of every group, as the operator has always
+    // asked for; it runs with as many CTAs per head as the workspace has room for
+    const int max_pages = (a->max_keys + a->page_size - 1) / a->page_size;
+    const int parts = std::max(1, std::min({sms / std::max(1, p->groups * a->n_heads), max_pages, 32}));
+    p->least = align256((size_t)p->groups * a->n_heads * parts * MAX_ROWS * (2 + HEAD_DIM) * sizeof(float)) +
+               p->count_bytes;
+    p->need = std::max(p->part_bytes + p->count_bytes, p->least);
     return MTP_OK;
 }
 
 int mtp::attention_standalone_launch(const mtp_attention_args* a, const AttnStandalonePlan& p, void* workspace,
-                                     cudaStream_t stream) {
+                                     size_t bytes, cudaStream_t stream) {
     AttnArgs at;
     std::memset(&at, 0, sizeof(at));
     const int d = a->n_heads * HEAD_DIM;
@@ -1195,12 +1193,16 @@ int mtp::attention_standalone_launch(const mtp_attention_args* a, const AttnStan
     at.block_table = a->block_table; at.bt_stride = a->bt_stride;
     at.row_seq = a->row_seq; at.row_pos = a->row_pos;
     at.out = a->out; at.ldo = d;
-    at.ws_part = static_cast<float*>(workspace);
-    at.ws_count = reinterpret_cast<int*>(static_cast<char*>(workspace) + p.part_bytes);
+    at.ws_count = static_cast<int*>(workspace);  // counters, then partials
+    at.ws_part = reinterpret_cast<float*>(static_cast<char*>(workspace) + p.count_bytes);
     at.rows_per_group = a->rows_per_group; at.n_heads = a->n_heads; at.page_size = a->page_size;
-    at.n_splits = p.splits; at.plan = PLAN_ROWS;
+    at.groups = p.groups; at.rows = a->rows;
+    const size_t room = (bytes - p.count_bytes) / sizeof(float);
+    for (at.ctas = p.splits; at.ctas > 1 && attn_workspace_floats(a->n_heads, at.ctas) > room;) --at.ctas;
+    at.whole = p.whole;
+    at.plan = PLAN_ROWS;
     at.err = nullptr;
-    CUDA_TRY(launch_attention(at, p.groups, stream, false));
+    CUDA_TRY(launch_attention_plain(at, stream));
     return MTP_OK;
 }
 
@@ -1844,9 +1846,9 @@ MTP_API int mtp_attention(const mtp_attention_args* a, void* workspace, size_t w
     AttnStandalonePlan p;
     MTP_TRY(attention_standalone_plan(a, true, &p));
     if (!workspace) return fail(MTP_ERR_INVALID, "attention: null workspace");
-    if (workspace_bytes < p.need)
+    if (workspace_bytes < p.least)
         return fail(MTP_ERR_INVALID, "attention: workspace %zu bytes, need %zu", workspace_bytes, p.need);
-    return attention_standalone_launch(a, p, workspace, static_cast<cudaStream_t>(cuda_stream));
+    return attention_standalone_launch(a, p, workspace, workspace_bytes, static_cast<cudaStream_t>(cuda_stream));
 }
 
 }  // extern "C"
@@ -1869,7 +1871,7 @@ int attention_tc_plan(const mtp_attention_args* a, bool check_pointers, AttnStan
     p->splits = attn_tc_splits_for(p->groups, a->n_heads, a->max_keys, sms);
     p->part_bytes = align256(attn_tc_workspace_floats(p->groups, a->n_heads, p->splits) * sizeof(float));
     p->count_bytes = align256((size_t)p->groups * a->n_heads * sizeof(int));
-    p->need = p->part_bytes + p->count_bytes;
+    p->need = p->least = p->part_bytes + p->count_bytes;
     return MTP_OK;
 }
 }  // namespace
@@ -1905,7 +1907,7 @@ MTP_API int mtp_attention_tc(const mtp_attention_args* a, void* workspace, size_
     at.ws_part = static_cast<float*>(workspace);
     at.ws_count = reinterpret_cast<int*>(static_cast<char*>(workspace) + p.part_bytes);
     at.rows = a->rows; at.n_heads = a->n_heads; at.page_size = a->page_size;
-    at.n_splits = p.splits; at.plan = PLAN_ROWS; at.kv_swizzled = 1;
+    at.n_splits = p.splits; at.plan = PLAN_ROWS;
     at.err = nullptr;
     CUDA_TRY(launch_attention_tc(at, static_cast<cudaStream_t>(cuda_stream), false));
     return MTP_OK;

@@ -428,6 +428,18 @@ int tc_encode_2d(CUtensorMap* map, const void* base, uint64_t inner, uint64_t ro
     return r == CUDA_SUCCESS ? 0 : -3;
 }
 
+int tc_encode_rows(CUtensorMap* map, const void* base, uint64_t rows_per_block, uint32_t box_rows) {
+    EncodeTiled fn = encode_fn();
+    if (!fn) return -1;
+    const cuuint64_t dims[3] = {TC_K, rows_per_block, (cuuint64_t)1 << 31};
+    const cuuint64_t strides[2] = {TC_K * 2, rows_per_block * TC_K * 2};
+    const cuuint32_t box[3] = {(cuuint32_t)TC_K, box_rows, 1}, estr[3] = {1, 1, 1};
+    const CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                          CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? 0 : -3;
+}
+
 int tc_tile_rows(int m) { return m <= 32 ? 32 : (m <= 64 ? 64 : 128); }
 
 cudaError_t launch_tc_gemm(const TcGemm& g, cudaStream_t s, bool pdl) {
