@@ -333,9 +333,8 @@ struct TcGemmArgs {
     const int* block_table; int bt_stride;
     __nv_bfloat16* pack_hi; __nv_bfloat16* pack_lo;  // TC_GELU_PACK: [m][n_w]
     int n_valid;                  // TC_ACCUM: 0, or only features < n_valid are added (element atomics, any ldo)
-    int cluster_reduce;           // 0/1: none; c in 2..8: each c consecutive K splits of a tile are one cluster
-                                  // that sums its partials in DSMEM, each CTA finishing 1/c of the rows
-                                  // (any epilogue; more splits than c only for TC_ACCUM, added by atomics)
+    int cluster_reduce;           // 0/1: none; 2 or 4 (TC_QKV, TC_GELU_PACK): the K splits of a tile are one
+                                  // cluster that sums its partials, each CTA finishing its share of the rows
     int* err;
     unsigned long long* trace;
 };
@@ -359,8 +358,8 @@ cudaError_t launch_tc_gemm(const TcGemm& g, cudaStream_t s, bool pdl);
 // which launch_tc_gemm would cut into `splits`.
 bool tc_gemm_pair_fits(int n_w, int m, int k_chunks, int splits, int num_sms);
 cudaError_t launch_tc_gemm_pair(const TcGemm& g, int num_sms, cudaStream_t s, bool pdl);
-constexpr int TC_CLUSTER_SPLITS = 4;  // K splits one cluster sums in the batched path (clusters of 8 at one CTA per
-                                      // SM: only 15 fit this GPU at once)
+constexpr int TC_CLUSTER_SPLITS = 4;  // most K splits one cluster sums (clusters of 8 at one CTA per SM: only 15
+                                      // fit this GPU at once)
 
 // ------------------------------------ fused heads + log-softmax + top-k ----
 // The n heads over m rows of LN_f(h) given as bf16 hi + lo (heads_tc.cu): per

@@ -14,12 +14,16 @@
 // and of both activation parts into a 4-stage shared-memory ring with TMA
 // (128-byte swizzled tiles), a second elected thread issues tcgen05.mma
 // into a TMEM accumulator (128 lanes x NT fp32 columns) and releases each
-// stage with tcgen05.commit, and the eight warps read the accumulator back
-// with tcgen05.ld (warps w and w + 4 own TMEM lanes 32w..32w+31, i.e. weight
-// rows, and take alternate 32-column chunks) and
-// store or atomically add it to out.  Grid: (N_w / 128 weight tiles, K
-// splits, activation tiles).  The weight copies of the first stages are
-// issued before griddepcontrol.wait; the activation copies after it.
+// stage with tcgen05.commit.  Eight warps read the accumulator back with
+// tcgen05.ld and finish it from the registers (tc_epilogue.cuh): warps w and
+// w + 4 share TMEM lanes 32 (w % 4) .., i.e. weight rows, and take half of the
+// columns each.  Staging the tile in shared memory first, to write float4
+// pieces of rows, took 0.65 us more and left the stores as long (512 rows,
+// d = 1024: W2 12.0 -> 10.2 us); where K splits meet in a cluster it is the
+// layout of the exchange (q|k|v and W1 of 128 rows: 8.0 -> 7.3 us).  Grid:
+// (N_w / 128 weight tiles, K splits, activation tiles).  The weight copies of
+// the first stages are issued before griddepcontrol.wait; the activation copies
+// after it.
 #include <cuda.h>
 
 #include <cstdio>
@@ -29,6 +33,7 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "mtp.h"
+#include "tc_epilogue.cuh"
 #include "tcgen05.cuh"
 
 namespace mtp {
@@ -39,11 +44,9 @@ constexpr int TC_K = 64;       // k per stage: one 128-byte swizzle row of bf16
 // ring stages per activation tile size: about 190 KB of copies in flight per CTA
 __host__ __device__ constexpr int tc_stages(int nt) { return nt <= 32 ? 8 : (nt <= 64 ? 6 : 4); }
 constexpr int TC_MAX_STAGES = 8;
-// 8 warps: two elected lanes run the ring; in the epilogue warps w and w + 4 share TMEM lane
-// quarter w % 4 and take alternate 32-column chunks, and every row loop has twice the threads
-// (the epilogue is instruction-latency bound: one warp per scheduler hid nothing)
+// 8 warps: two elected lanes run the ring; the epilogue is instruction-latency bound (one warp per
+// scheduler hid nothing)
 constexpr int TC_THREADS = 256;
-constexpr int TC_MAX_CLUSTER_SPLITS = 8;  // K splits reduced in one (portable) cluster
 constexpr uint32_t TC_W_BYTES = TC_M * TC_K * 2;
 
 // ---- PTX wrappers (tcgen05, TMA) ----
@@ -61,7 +64,6 @@ __device__ __forceinline__ void bulk_copy_s2s_cluster(uint32_t dst, uint32_t src
                  "r"(src), "r"(bytes), "r"(bar)
                  : "memory");
 }
-
 // Shared-memory address `saddr` of this CTA mapped to the CTA of cluster rank `rank`.
 __device__ __forceinline__ uint32_t mapa_rank(uint32_t saddr, int rank) {
     uint32_t r;
@@ -75,7 +77,7 @@ __host__ __device__ constexpr uint32_t tc_idesc(int nt) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nt >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
 }
 
-template <int NT, bool PART>
+template <int NT, int EPI, bool CLUSTER>
 __global__ void __launch_bounds__(TC_THREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tw, const __grid_constant__ CUtensorMap tah,
                    const __grid_constant__ CUtensorMap tal, const TcGemmArgs a) {
@@ -179,14 +181,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         }
         if (c < chunks) s_ok = 0;
         tc_commit(&done);  // every MMA issued above has completed
-    } else if (warp >= 2 && (a.epilogue == TC_QKV || a.epilogue == TC_GELU_PACK)) {
+    } else if (warp >= 2 && (EPI == TC_QKV || EPI == TC_GELU_PACK)) {
         // per-row facts of the epilogue, gathered by the two idle warps while the ring runs
         for (int j = tid - 64; j < NT; j += TC_THREADS - 64) {
             const int n = arow + j;
             const int seq = n < a.m ? a.row_seq[n] : -1;
             long long base = -1;
             int t = 0;
-            if (a.epilogue == TC_QKV && seq >= 0) {
+            if (EPI == TC_QKV && seq >= 0) {
                 const int pos = a.row_pos[n];
                 t = pos % a.page_size;
                 const int page = a.block_table[(size_t)seq * a.bt_stride + pos / a.page_size];
@@ -196,7 +198,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                     base = (long long)page * a.page_elems + a.layer_off + (long long)t * HEAD_DIM;
             }
             s_rowbase[j] = seq >= 0 ? base : -2;  // -2: no sequence
-            s_rowt[j] = a.epilogue == TC_QKV ? t : (seq >= 0);
+            s_rowt[j] = EPI == TC_QKV ? t : (seq >= 0);
         }
     }
     if (warp < 2) __syncwarp();
@@ -207,148 +209,100 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     const bool fin = __syncthreads_and(tid == 0 ? mbar_wait(&done, 0, a.err) : true) != 0;
     tc_fence_after();
     trace_mark(a.trace, 0);  // accumulator complete
-    // K splits reduced in a cluster: Sc consecutive splits of this tile are one cluster; each
-    // stages its partial tile, then sums one Sc-th of the activation rows over the cluster's tiles
-    // (DSMEM) and runs the epilogue on those rows only.  Clusters of the same tile (TC_ACCUM with
-    // more splits than one cluster holds) still add their sums with atomics.
-    const int Sc = a.cluster_reduce > 1 ? a.cluster_reduce : 1;
-    const bool creduce = Sc > 1;
-    const int rank = split % Sc;
     const bool good = fin && s_ok;
-    constexpr int TP = TC_M + 4;  // row pitch of the staged tile (floats)
-    float* T = reinterpret_cast<float*>(smem);
-    if (good) {
-        // accumulator -> shared tile T[n][f] (the stages are free: every MMA has read them)
-        const int quarter = warp & 3;  // the TMEM lanes (weight rows) this warp may read
-        for (int j0 = (warp >> 2) * 32; j0 < NT; j0 += (TC_THREADS / 128) * 32) {
-            float v[32];
-            tmem_ld32(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)j0, v);
-#pragma unroll
-            for (int j = 0; j < 32; ++j) T[(j0 + j) * TP + quarter * 32 + lane] = v[j];
-        }
-    }
-    trace_mark(a.trace, 1);  // thread 0's rows staged
-    int jbeg = 0, jend = NT;  // activation rows of the tile this CTA finishes
-    if (creduce) {
-        // each CTA pushes the rows that another CTA finishes to that CTA (one bulk copy per peer,
-        // completing on the receiver's barrier), then sums the Sc partial copies of its own rows
-        jbeg = rank * NT / Sc;
-        jend = (rank + 1) * NT / Sc;
-        const uint32_t seg = (uint32_t)(NT / Sc) * TP * 4;  // bytes of one CTA's share of rows
-        float* recv = T + (size_t)NT * TP;                  // [Sc][NT / Sc][TP]: slot = sender's rank
-        if (tid == 0) mbar_arrive_expect_tx(&red_bar, seg * (uint32_t)(Sc - 1));
+    const int quarter = warp & 3, half = warp >> 2;  // the TMEM lanes (weight rows) this warp may read
+    const int f = tile * TC_M + quarter * 32 + lane;
+    const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16);
+    const int rows = min(NT, a.m - arow);  // activation rows of the tile
+    if constexpr (CLUSTER) {
+        // K splits reduced in a cluster: Sc consecutive splits of this tile are one cluster, and each
+        // finishes an Sc-th of the activation rows.  A thread reads its weight row's columns at once and
+        // leaves them in the layout in which their finishers read them, [128 weight rows][rows of a share];
+        // a peer's share goes there in one bulk copy (into the space of its ring: the cluster barrier says
+        // that everyone's MMAs are done, and is waited for behind the staging).  Then each thread adds the
+        // Sc partials of its weight row in rank order.  (16-byte st.async pushes from the registers: 4.8 us
+        // for the 48 KB of a CTA at 128 rows, the copies 1.9 us.)
+        const int Sc = a.cluster_reduce, rank = split % Sc, R = NT / Sc;  // rows of a share
+        constexpr int N = NT / 8;             // four units of N rows per thread: half of every share
+        const int pitch = R + 4;              // floats per (sender, weight row): 16-byte rows, spread banks
+        const uint32_t part_bytes = (uint32_t)(TC_M * pitch * 4);
+        float* recv = reinterpret_cast<float*>(smem);  // parts by sender, then the staged ones by receiver
+        float* staged = recv + (size_t)Sc * TC_M * pitch;
+        const int fl = quarter * 32 + lane;
+        if (tid == 0) mbar_arrive_expect_tx(&red_bar, part_bytes * (uint32_t)(Sc - 1));
         __syncthreads();
-        cluster_arrive_release();  // every split's partial tile is staged and every receiver armed
+        cluster_arrive_release();  // this CTA's ring is free and its barrier armed
+        float v[4][N];
+        // unit u: rows r0(u) .. + N of share p(u)
+        auto share = [&](int u) { return Sc == 4 ? u : u >> 1; };
+        auto first = [&](int u) { return half * (R / 2) + (Sc == 4 ? 0 : (u & 1) * N); };
+#pragma unroll
+        for (int u = 0; u < 4; ++u) tmem_ld_issue<N>(acc + (uint32_t)(share(u) * R + first(u)), v[u]);
+        tmem_ld_wait();
+#pragma unroll
+        for (int u = 0; u < 4; ++u) tmem_ld_done(v[u]);
+        if (good) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int p = share(u);
+                float* dst = (p == rank ? recv : staged) + ((size_t)p * TC_M + fl) * pitch + first(u);
+#pragma unroll
+                for (int e = 0; e < N; e += 4)
+                    *reinterpret_cast<float4*>(dst + e) = make_float4(v[u][e], v[u][e + 1], v[u][e + 2], v[u][e + 3]);
+            }
+        }
+        fence_proxy_async();  // (read by the copies)
+        trace_mark(a.trace, 1);  // thread 0's rows staged
         cluster_wait();
-        trace_mark(a.trace, 2);  // the cluster's tiles staged
-        if (tid < Sc - 1 && good) {  // one copy per issuing thread
-            fence_proxy_async();  // the tile was written by this CTA's threads
+        __syncthreads();
+        trace_mark(a.trace, 2);  // every ring free, every row staged
+        if (tid < Sc - 1 && good) {  // one copy per issuing thread, receivers in rotated order
             const int p = (rank + 1 + tid) % Sc;
-            bulk_copy_s2s_cluster(mapa_rank(smem_addr(recv + (size_t)rank * (NT / Sc) * TP), p),
-                                  smem_addr(T + (size_t)p * (NT / Sc) * TP), seg, mapa_rank(smem_addr(&red_bar), p));
+            bulk_copy_s2s_cluster(mapa_rank(smem_addr(recv + (size_t)rank * TC_M * pitch), p),
+                                  smem_addr(staged + (size_t)p * TC_M * pitch), part_bytes,
+                                  mapa_rank(smem_addr(&red_bar), p));
         }
         const bool got = __syncthreads_and(tid == 0 ? mbar_wait(&red_bar, 0, a.err) : true) != 0;
+        cluster_arrive_relaxed();  // (waited for before leaving)
         trace_mark(a.trace, 3);  // the peers' partial rows received
         if (good && got) {
-            for (int i = tid; i < (jend - jbeg) * (TC_M / 4); i += TC_THREADS) {
-                const int jl = i / (TC_M / 4), f4 = (i % (TC_M / 4)) * 4;
-                float* t = T + (size_t)(jbeg + jl) * TP + f4;
-                float4 part[TC_MAX_CLUSTER_SPLITS];
+            const float bias = a.bias ? __ldg(a.bias + f) : 0.f;
+            for (int r0 = half * (R / 2); r0 < (half + 1) * (R / 2); r0 += N) {
+                float y[N];
 #pragma unroll
-                for (int src = 0; src < TC_MAX_CLUSTER_SPLITS; ++src)  // every partial loaded before any is added
-                    if (src < Sc)
-                        part[src] = *reinterpret_cast<const float4*>(
-                            src == rank ? t : recv + ((size_t)src * (NT / Sc) + jl) * TP + f4);
-                float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+                for (int e = 0; e < N; ++e) y[e] = 0.f;
 #pragma unroll
-                for (int src = 0; src < TC_MAX_CLUSTER_SPLITS; ++src) {  // every split's partial, in rank order
-                    if (src >= Sc) continue;
-                    acc.x += part[src].x;
-                    acc.y += part[src].y;
-                    acc.z += part[src].z;
-                    acc.w += part[src].w;
-                }
-                *reinterpret_cast<float4*>(t) = acc;
-            }
-        }
-        if (!got) s_ok = 0;
-        cluster_arrive_relaxed();  // this CTA's pushes have landed (waited for before leaving)
-    }
-    __syncthreads();
-    trace_mark(a.trace, 4);  // rows to finish summed
-    if (good && s_ok) {
-        // float4 rows of T -> out, coalesced
-        const int rows = min(NT, a.m - arow);
-        const bool add_bias = a.bias && split < Sc;  // the tile's first cluster (or split 0) adds it
-        const int P = a.page_size, H = a.n_heads, d = H * HEAD_DIM;
-        const int j1 = min(jend, rows);
-        if constexpr (PART) {  // TC_ACCUM of features < n_valid only, element atomics (rows of any pitch)
-            for (int i = tid; i < (j1 - jbeg) * TC_M; i += TC_THREADS) {
-                const int j = jbeg + i / TC_M, fl = i % TC_M, f = tile * TC_M + fl;
-                if (f < a.n_valid)
-                    atomicAdd(a.out + (size_t)(arow + j) * a.ldo + f, T[j * TP + fl] + (add_bias ? a.bias[f] : 0.f));
-            }
-        } else {
-        // every item of this thread has the same 4 features (TC_THREADS is a multiple of TC_M / 4):
-        // their bias is read once, ahead of the stores
-        static_assert(TC_THREADS % (TC_M / 4) == 0, "one feature quad per thread");
-        float4 bq = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (add_bias) {
-            const int f = tile * TC_M + (tid % (TC_M / 4)) * 4;
-            bq = make_float4(__ldg(a.bias + f), __ldg(a.bias + f + 1), __ldg(a.bias + f + 2), __ldg(a.bias + f + 3));
-        }
-        for (int i = tid; i < (j1 - jbeg) * (TC_M / 4); i += TC_THREADS) {
-            const int j = jbeg + i / (TC_M / 4), f4 = (i % (TC_M / 4)) * 4;
-            const int f = tile * TC_M + f4, n = arow + j;
-            float4 y = *reinterpret_cast<const float4*>(T + j * TP + f4);
-            y.x += bq.x;
-            y.y += bq.y;
-            y.z += bq.z;
-            y.w += bq.w;
-            if (a.epilogue == TC_ACCUM) {
-                atomicAdd(reinterpret_cast<float4*>(a.out + (size_t)n * a.ldo + f), y);
-            } else if (a.epilogue == TC_STORE) {
-                *reinterpret_cast<float4*>(a.out + (size_t)n * a.ldo + f) = y;
-            } else if (a.epilogue == TC_QKV) {  // features h*192 + {q,k,v}*64 + dd
-                const long long base = s_rowbase[j];
-                if (base == -2) continue;  // no sequence
-                const int h = f / (3 * HEAD_DIM), sec = (f / HEAD_DIM) % 3, dd = f % HEAD_DIM;
-                if (sec == 0) {
-                    *reinterpret_cast<float4*>(a.out + (size_t)n * d + h * HEAD_DIM + dd) = y;
-                    continue;
-                }
-                if (base < 0) continue;  // unreserved page (reported)
-                const int t = s_rowt[j];
-                const long long idx = base + (long long)(sec - 1) * H * P * HEAD_DIM + (long long)h * P * HEAD_DIM +
-                                      ((((dd >> 3) ^ (t & 7)) << 3) | (dd & 7));
-                uint2 pk;
-                pk.x = (uint32_t)f32_to_bf16_bits(y.x) | ((uint32_t)f32_to_bf16_bits(y.y) << 16);
-                pk.y = (uint32_t)f32_to_bf16_bits(y.z) | ((uint32_t)f32_to_bf16_bits(y.w) << 16);
-                *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(a.kv_pool) + idx) = pk;
-            } else {  // TC_GELU_PACK
-                const bool on = s_rowt[j] != 0;
-                const float v[4] = {on ? gelu_erf(y.x) : 0.f, on ? gelu_erf(y.y) : 0.f, on ? gelu_erf(y.z) : 0.f,
-                                    on ? gelu_erf(y.w) : 0.f};
-                uint32_t hi[2], lo[2];
+                for (int src = 0; src < TC_CLUSTER_SPLITS; ++src) {  // every split's partial, in rank order
+                    if (src >= Sc) break;
+                    const float4* part = reinterpret_cast<const float4*>(recv + ((size_t)src * TC_M + fl) * pitch + r0);
 #pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const __nv_bfloat16 h0 = __float2bfloat16_rn(v[2 * q]), h1 = __float2bfloat16_rn(v[2 * q + 1]);
-                    const __nv_bfloat16 l0 = __float2bfloat16_rn(v[2 * q] - __bfloat162float(h0));
-                    const __nv_bfloat16 l1 = __float2bfloat16_rn(v[2 * q + 1] - __bfloat162float(h1));
-                    hi[q] = (uint32_t)__bfloat16_as_ushort(h0) | ((uint32_t)__bfloat16_as_ushort(h1) << 16);
-                    lo[q] = (uint32_t)__bfloat16_as_ushort(l0) | ((uint32_t)__bfloat16_as_ushort(l1) << 16);
+                    for (int e = 0; e < N; e += 4) {
+                        const float4 x = part[e / 4];
+                        y[e] += x.x;
+                        y[e + 1] += x.y;
+                        y[e + 2] += x.z;
+                        y[e + 3] += x.w;
+                    }
                 }
-                *reinterpret_cast<uint2*>(a.pack_hi + (size_t)n * a.ldo + f) = make_uint2(hi[0], hi[1]);
-                *reinterpret_cast<uint2*>(a.pack_lo + (size_t)n * a.ldo + f) = make_uint2(lo[0], lo[1]);
+                const int j0 = rank * R + r0;
+                tc_epilogue<EPI, false>(a, y, arow + j0, j0, rows - j0, f, bias, s_rowbase, s_rowt);
             }
+            trace_mark(a.trace, 5);  // thread 0's stores issued
         }
+    } else if (good) {
+        constexpr int N = NT / 2 < 32 ? NT / 2 : 32;
+        // the tile's first split adds the bias (heads: rows past n_valid have none)
+        const float bias = a.bias && split == 0 && (!a.n_valid || f < a.n_valid) ? __ldg(a.bias + f) : 0.f;
+        for (int j0 = half * (NT / 2); j0 < (half + 1) * (NT / 2) && j0 < rows; j0 += N) {
+            float v[N];
+            tmem_ld<N>(acc + (uint32_t)j0, v);
+            tc_epilogue<EPI, true>(a, v, arow + j0, j0, rows - j0, f, bias, s_rowbase, s_rowt);
         }
         trace_mark(a.trace, 5);  // thread 0's stores issued
-    } else if (!fin) {
-        // the MMAs may still be running: wait for them (bounded) before freeing TMEM
-        mbar_wait(&done, 0, nullptr);
     }
-    if (creduce) cluster_wait();  // the peers are done with this CTA's tile
+    // the MMAs may still be running: wait for them (bounded) before freeing TMEM
+    if (!fin) mbar_wait(&done, 0, nullptr);
+    if constexpr (CLUSTER) cluster_wait();  // no peer still pushes into this CTA
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, TMEM_COLS);
@@ -405,8 +359,18 @@ cudaError_t launch_kern(K kern, const TcGemm& g, cudaStream_t s, bool pdl) {
 
 template <int NT>
 cudaError_t launch_nt(const TcGemm& g, cudaStream_t s, bool pdl) {
-    if (g.args.n_valid) return launch_kern<NT>(tc_gemm_kernel<NT, true>, g, s, pdl);
-    return launch_kern<NT>(tc_gemm_kernel<NT, false>, g, s, pdl);
+    const bool cluster = g.args.cluster_reduce > 1;
+    switch (g.args.epilogue) {
+        case TC_STORE: return launch_kern<NT>(tc_gemm_kernel<NT, TC_STORE, false>, g, s, pdl);
+        case TC_ACCUM: return launch_kern<NT>(tc_gemm_kernel<NT, TC_ACCUM, false>, g, s, pdl);
+        case TC_QKV:
+            if (cluster) return launch_kern<NT>(tc_gemm_kernel<NT, TC_QKV, true>, g, s, pdl);
+            return launch_kern<NT>(tc_gemm_kernel<NT, TC_QKV, false>, g, s, pdl);
+        case TC_GELU_PACK:
+            if (cluster) return launch_kern<NT>(tc_gemm_kernel<NT, TC_GELU_PACK, true>, g, s, pdl);
+            return launch_kern<NT>(tc_gemm_kernel<NT, TC_GELU_PACK, false>, g, s, pdl);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 }  // namespace
@@ -445,8 +409,11 @@ int tc_tile_rows(int m) { return m <= 32 ? 32 : (m <= 64 ? 64 : 128); }
 cudaError_t launch_tc_gemm(const TcGemm& g, cudaStream_t s, bool pdl) {
     if (g.n_w % TC_M || g.args.k_chunks < 1 || g.splits < 1 || g.args.m < 1) return cudaErrorInvalidValue;
     const int sc = g.args.cluster_reduce > 1 ? g.args.cluster_reduce : 1;
-    if (sc > TC_MAX_CLUSTER_SPLITS || g.splits % sc) return cudaErrorInvalidValue;
-    if (g.args.epilogue != TC_ACCUM && g.splits != sc) return cudaErrorInvalidValue;  // one cluster finishes a tile
+    // one cluster (2 or 4 splits) finishes a tile; accumulated outputs take their splits by atomics
+    if (g.args.epilogue == TC_ACCUM ? sc != 1 : g.splits != sc) return cudaErrorInvalidValue;
+    if ((sc != 1 && sc != 2 && sc != TC_CLUSTER_SPLITS) ||
+        (sc > 1 && g.args.epilogue != TC_QKV && g.args.epilogue != TC_GELU_PACK))
+        return cudaErrorInvalidValue;
     switch (g.nt) {
         case 32: return launch_nt<32>(g, s, pdl);
         case 64: return launch_nt<64>(g, s, pdl);

@@ -35,6 +35,7 @@
 
 #include "common.cuh"
 #include "kernels.cuh"
+#include "tc_epilogue.cuh"
 #include "tcgen05.cuh"
 
 namespace mtp {
@@ -111,11 +112,6 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
     return false;
 }
 __device__ __forceinline__ void epi_barrier() { asm volatile("bar.sync 1, %0;" ::"n"(32 * TP_EPI_WARPS) : "memory"); }
-
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
-    return *reinterpret_cast<const uint32_t*>(&p);
-}
 
 template <int EPI>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
@@ -225,7 +221,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
         }
     } else if (warp >= TP_EPI_WARP) {  // ---- epilogue ----
         const int et = tid - TP_EPI_WARP * 32, quarter = warp & 3, j0 = ((warp - TP_EPI_WARP) >> 2) * TP_COLS;
-        const int H = a.n_heads, P = a.page_size, d = H * HEAD_DIM;
+        const int P = a.page_size;
         constexpr bool FACTS = EPI == TC_QKV || EPI == TC_GELU_PACK;
         float sum[TP_COLS];
         bool ok = true;
@@ -281,71 +277,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
             const int n0 = row0 + j0, rows = min(TP_COLS, a.m - n0);  // this warp's rows
             if (rows <= 0) continue;
             const float bias = a.bias ? __ldg(a.bias + f) : 0.f;
-            if (EPI == TC_STORE) {
-                float* o = a.out + (size_t)n0 * a.ldo + f;
-#pragma unroll
-                for (int e = 0; e < TP_COLS; ++e)
-                    if (e < rows) o[(size_t)e * a.ldo] = sum[e] + bias;
-            } else if (EPI == TC_ACCUM) {  // this CTA alone owns these outputs
-                float* o = a.out + (size_t)n0 * a.ldo + f;
-#pragma unroll
-                for (int e0 = 0; e0 < TP_COLS; e0 += 8) {
-                    float x[8];
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) x[e] = e0 + e < rows ? o[(size_t)(e0 + e) * a.ldo] : 0.f;
-#pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        if (e0 + e < rows) o[(size_t)(e0 + e) * a.ldo] = x[e] + (sum[e0 + e] + bias);
-                }
-            } else if (EPI == TC_GELU_PACK) {
-                // lanes 2i, 2i + 1 exchange one value: the even lane writes features (f, f + 1) of row
-                // e, the odd lane of row e + 1
-                const int odd = lane & 1;
-                // rows of a sequence (the others are written as zeros)
-                const uint32_t act[2] = {__ballot_sync(FULL_MASK, s_rowt[fb][j0 + lane]),
-                                         __ballot_sync(FULL_MASK, s_rowt[fb][j0 + 32 + lane])};
-                const size_t at = (size_t)(n0 + odd) * a.ldo + (f - odd);
-                __nv_bfloat16 *ph = a.pack_hi + at, *pl = a.pack_lo + at;
-                const int mine = rows - odd;  // this lane writes rows e + odd < rows
-#pragma unroll
-                for (int e = 0; e < TP_COLS; e += 2) {
-                    const float u0 = gelu_erf(sum[e] + bias), u1 = gelu_erf(sum[e + 1] + bias);
-                    const float g0 = act[e >> 5] >> (e & 31) & 1 ? u0 : 0.f;
-                    const float g1 = act[e >> 5] >> ((e & 31) + 1) & 1 ? u1 : 0.f;
-                    const float got = __shfl_xor_sync(FULL_MASK, odd ? g0 : g1, 1);
-                    const float y0 = odd ? got : g0, y1 = odd ? g1 : got;
-                    const uint32_t hi = pack_bf16(y0, y1);
-                    const uint32_t lo = pack_bf16(y0 - bf16_lo(hi), y1 - bf16_hi(hi));
-                    if (e < mine) {
-                        *reinterpret_cast<uint32_t*>(ph) = hi;
-                        *reinterpret_cast<uint32_t*>(pl) = lo;
-                    }
-                    ph += 2 * (size_t)a.ldo;
-                    pl += 2 * (size_t)a.ldo;
-                }
-            } else {  // TC_QKV: features h * 192 + {q, k, v} * 64 + dd (one head and part per warp)
-                const int h = f / (3 * HEAD_DIM), sec = (f / HEAD_DIM) % 3, dd = f % HEAD_DIM;
-                if (sec == 0) {
-                    float* o = a.out + (size_t)n0 * d + h * HEAD_DIM + dd;
-#pragma unroll
-                    for (int e = 0; e < TP_COLS; ++e)
-                        if (s_rowbase[fb][j0 + e] != -2) o[(size_t)e * d] = sum[e] + bias;
-                } else {
-                    const int odd = lane & 1, de = dd - odd;
-                    const long long off = (long long)(sec - 1) * H * P * HEAD_DIM + (long long)h * P * HEAD_DIM;
-#pragma unroll
-                    for (int e = 0; e < TP_COLS; e += 2) {
-                        const float g0 = sum[e] + bias, g1 = sum[e + 1] + bias;
-                        const float got = __shfl_xor_sync(FULL_MASK, odd ? g0 : g1, 1);
-                        const uint32_t pk = odd ? pack_bf16(got, g1) : pack_bf16(g0, got);
-                        const long long base = s_rowbase[fb][j0 + e + odd];
-                        const int tr = s_rowt[fb][j0 + e + odd];
-                        if (base >= 0)
-                            *reinterpret_cast<uint32_t*>(reinterpret_cast<uint16_t*>(a.kv_pool) + base + off +
-                                                         ((((de >> 3) ^ (tr & 7)) << 3) | (de & 7))) = pk;
-                    }
-                }
-            }
+            tc_epilogue<EPI, false>(a, sum, n0, j0, rows, f, bias, s_rowbase[fb], s_rowt[fb]);
         }
     }
     // nothing signals a CTA that has left, and TMEM is freed once both are done with it
