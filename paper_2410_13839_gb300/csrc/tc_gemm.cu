@@ -26,6 +26,7 @@
 // after it.
 #include <cuda.h>
 
+#include <condition_variable>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -427,6 +428,49 @@ cudaError_t launch_tc_gemm(const TcGemm& g, cudaStream_t s, bool pdl) {
 using namespace mtp;
 
 namespace {
+// Error words of mtp_gemm_bf16x2's calls in flight: pinned host memory that the kernels reach directly, so
+// a call needs no device allocation, memset or copy of its own (with them, 512 rows of W1: 39 us a call,
+// 250 when the device was idle in between and the allocator had given its pool back; without: 33).  At
+// most ERR_SLOTS calls hold one at a time, each on its own; more at once wait for one to come back.  A word
+// is zero while it is free.
+constexpr int ERR_SLOTS = 64;
+class ErrorWords {
+public:
+    int take() {  // a free slot, -1 without the memory
+        std::unique_lock<std::mutex> lock(mu_);
+        if (!words_) {
+            void* p = nullptr;
+            if (cudaHostAlloc(&p, ERR_SLOTS * sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+                cudaGetLastError();
+                return -1;
+            }
+            std::memset(p, 0, ERR_SLOTS * sizeof(int));
+            words_ = static_cast<int*>(p);
+        }
+        back_.wait(lock, [&] { return free_ != 0; });
+        const int slot = __builtin_ctzll(free_);
+        free_ &= free_ - 1;
+        return slot;
+    }
+    void give(int slot) {
+        std::lock_guard<std::mutex> lock(mu_);
+        free_ |= 1ull << slot;
+        back_.notify_one();
+    }
+    volatile int* host(int slot) { return words_ + slot; }
+    int* device(int slot) {  // the address of the word on the current device, or null
+        void* p = nullptr;
+        return cudaHostGetDevicePointer(&p, words_, 0) == cudaSuccess ? static_cast<int*>(p) + slot : nullptr;
+    }
+
+private:
+    std::mutex mu_;
+    std::condition_variable back_;
+    unsigned long long free_ = ~0ull;
+    int* words_ = nullptr;  // kept until the process exits
+};
+ErrorWords g_error_words;
+
 int gemm_fail(int code, const char* fmt, int a = 0, int b = 0, int c = 0, int d = 0, int e = 0) {
     char buf[256];
     snprintf(buf, sizeof(buf), fmt, a, b, c, d, e);
@@ -463,12 +507,12 @@ extern "C" MTP_API int mtp_gemm_bf16x2(const void* w, const void* a_hi, const vo
         g.splits = 1;
         g.args.k_chunks = k / TC_K;
     }
-    int* d_err = nullptr;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (cudaMallocAsync(&d_err, sizeof(int), st) != cudaSuccess)
+    const int slot = g_error_words.take();
+    if (slot < 0 || !(g.args.err = g_error_words.device(slot))) {
+        if (slot >= 0) g_error_words.give(slot);
         return gemm_fail(MTP_ERR_CUDA, "mtp_gemm_bf16x2: error word allocation failed");
-    cudaMemsetAsync(d_err, 0, sizeof(int), st);
-    g.args.err = d_err;
+    }
     int rc = 0;
     if (tc_encode_2d(&g.w, w, (uint64_t)k, (uint64_t)n_w, TC_M, false) ||
         tc_encode_2d(&g.a_hi, a_hi, (uint64_t)k, (uint64_t)m, (uint32_t)g.nt, false) ||
@@ -478,12 +522,12 @@ extern "C" MTP_API int mtp_gemm_bf16x2(const void* w, const void* a_hi, const vo
         const cudaError_t e = pairs ? launch_tc_gemm_pair(g, sms, st, false) : launch_tc_gemm(g, st, false);
         if (e != cudaSuccess) rc = report_error(MTP_ERR_CUDA, cudaGetErrorString(e));
     }
-    int h_err = 0;
-    cudaMemcpyAsync(&h_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, st);
     const cudaError_t es = cudaStreamSynchronize(st);
-    cudaFreeAsync(d_err, st);
+    const int err = *g_error_words.host(slot);
+    *g_error_words.host(slot) = 0;
+    g_error_words.give(slot);
     if (rc) return rc;
     if (es != cudaSuccess) return report_error(MTP_ERR_CUDA, cudaGetErrorString(es));
-    if (h_err) return gemm_fail(MTP_ERR_DEVICE, "mtp_gemm_bf16x2: device error word 0x%x", h_err);
+    if (err) return gemm_fail(MTP_ERR_DEVICE, "mtp_gemm_bf16x2: device error word 0x%x", err);
     return MTP_OK;
 }
