@@ -51,7 +51,14 @@ __global__ void __launch_bounds__(PK_THREADS) pack_rows_kernel(const PackArgs a)
 #pragma unroll
     for (int i = 0; i < MAXQ; ++i) {
         const int q = tid + i * PK_THREADS;
-        v[i] = on && q < nq ? xr[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (ALL && a.x_bf16) {
+            const uint2 u = q < nq ? reinterpret_cast<const uint2*>(reinterpret_cast<const uint16_t*>(a.x) +
+                                                                     (size_t)r * a.ldx)[q]
+                                   : make_uint2(0u, 0u);
+            v[i] = make_float4(bf16_lo(u.x), bf16_hi(u.x), bf16_lo(u.y), bf16_hi(u.y));
+        } else {
+            v[i] = on && q < nq ? xr[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
     }
     if (a.mode == PACK_LN) {
         // each warp's mean and sum of squared deviations over its own elements (two passes
@@ -201,7 +208,8 @@ cudaError_t launch_rows(K kern, const A& args, int rows, cudaStream_t s, bool pd
 
 cudaError_t launch_pack_rows(const PackArgs& a, cudaStream_t s, bool pdl) {
     if (a.k < 4 || a.k > 16 * PK_THREADS || a.k % 4 || a.ldx % 4 || a.m < 1) return cudaErrorInvalidValue;
-    if ((reinterpret_cast<uintptr_t>(a.x) | reinterpret_cast<uintptr_t>(a.hi) | reinterpret_cast<uintptr_t>(a.lo) |
+    if (a.x_bf16 && (a.row_seq || (reinterpret_cast<uintptr_t>(a.x) & 7))) return cudaErrorInvalidValue;
+    if (((a.x_bf16 ? 0 : reinterpret_cast<uintptr_t>(a.x)) | reinterpret_cast<uintptr_t>(a.hi) | reinterpret_cast<uintptr_t>(a.lo) |
          reinterpret_cast<uintptr_t>(a.zero_after) | reinterpret_cast<uintptr_t>(a.gamma) |
          reinterpret_cast<uintptr_t>(a.beta)) & 15)
         return cudaErrorInvalidValue;  // float4 rows

@@ -97,6 +97,7 @@ __global__ void pe_kernel(float* pe, int max_ctx, int d) {
 }
 
 __global__ void convert_rows_kernel(const void* src, int src_bf16, float* dst, long long n) {
+    pdl_launch_dependents();  // the next kernel's weights may come in meanwhile
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     dst[i] = src_bf16 ? __uint_as_float((uint32_t)reinterpret_cast<const uint16_t*>(src)[i] << 16)

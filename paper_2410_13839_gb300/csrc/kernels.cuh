@@ -301,6 +301,7 @@ enum PackMode : int { PACK_LN = 0, PACK_COPY = 1, PACK_GELU = 2 };
 struct PackArgs {
     int mode;                     // PackMode
     const float* x; int ldx;      // input rows [m][ldx], k columns used
+    int x_bf16;                   // x holds bf16 rows (8-byte aligned; every-row variant, row_seq null)
     float* zero_after;            // PACK_GELU: rows zeroed after reading (may be x), or null
     const float* gamma; const float* beta; float eps;   // PACK_LN
     const int* row_seq;           // rows with row_seq < 0 are packed as zeros (null: every row is packed,

@@ -620,17 +620,18 @@ EmbedArgs embed_base(mtp_ctx* c) {
 // tensor cores: LN_f rows as bf16 hi + lo (the same kernel zeroes the logits),
 // then one split-K GEMM over the first n heads' n V rows, added into
 // logits [B][n V].
-int launch_heads_batched(mtp_ctx* c, const float* x, int B, int n, float* logits, cudaStream_t s, bool pdl,
-                         Prof* prof) {
+int launch_heads_batched(mtp_ctx* c, const void* x, bool x_bf16, int B, int n, float* logits, cudaStream_t s,
+                         bool pdl_first, bool pdl, Prof* prof) {
     const mtp_config& cf = c->cfg;
     const int d = cf.d_model, V = cf.codec_vocab;
     PackArgs pa;
     std::memset(&pa, 0, sizeof(pa));
-    pa.mode = PACK_LN; pa.x = x; pa.ldx = d; pa.gamma = c->lnf_g; pa.beta = c->lnf_b;
+    pa.mode = PACK_LN; pa.x = static_cast<const float*>(x); pa.x_bf16 = x_bf16; pa.ldx = d;
+    pa.gamma = c->lnf_g; pa.beta = c->lnf_b;
     pa.eps = cf.ln_eps; pa.row_seq = nullptr; pa.hi = c->d_ahi; pa.lo = c->d_alo; pa.k = d; pa.m = B;
     pa.zero_buf = logits; pa.zero_n = (long long)B * n * V;
     pa.trace = tslot(c, MTP_K_PACK);
-    LAUNCH(MTP_K_PACK, launch_pack_rows(pa, s, pdl));
+    LAUNCH(MTP_K_PACK, launch_pack_rows(pa, s, pdl_first));
     const int nt = tc_tile_rows(B), ntiles = (B + nt - 1) / nt;
     const int n_w = (n * V + 127) / 128 * 128, tiles = n_w / 128, chunks = d / 64;
     int splits = 1;
@@ -659,16 +660,17 @@ bool heads_fused_ok(const mtp_ctx* c, int k, bool decode_step) {
 // (B <= the batched buffers' rows): LN_f rows as bf16 hi + lo, then one kernel
 // that writes the candidates (ids, logp [B][n][k]), lse [B][n] and, when
 // `logits` is not null, the logits [B][n V].
-int launch_heads_fused(mtp_ctx* c, const float* x, int B, int n, int k, int32_t* ids, float* logp, float* lse,
-                       float* logits, cudaStream_t s, bool pdl, Prof* prof) {
+int launch_heads_fused(mtp_ctx* c, const void* x, bool x_bf16, int B, int n, int k, int32_t* ids, float* logp,
+                       float* lse, float* logits, cudaStream_t s, bool pdl_first, bool pdl, Prof* prof) {
     const mtp_config& cf = c->cfg;
     const int d = cf.d_model, V = cf.codec_vocab;
     PackArgs pa;
     std::memset(&pa, 0, sizeof(pa));
-    pa.mode = PACK_LN; pa.x = x; pa.ldx = d; pa.gamma = c->lnf_g; pa.beta = c->lnf_b;
+    pa.mode = PACK_LN; pa.x = static_cast<const float*>(x); pa.x_bf16 = x_bf16; pa.ldx = d;
+    pa.gamma = c->lnf_g; pa.beta = c->lnf_b;
     pa.eps = cf.ln_eps; pa.row_seq = nullptr; pa.hi = c->d_ahi; pa.lo = c->d_alo; pa.k = d; pa.m = B;
     pa.trace = tslot(c, MTP_K_PACK);
-    LAUNCH(MTP_K_PACK, launch_pack_rows(pa, s, pdl));
+    LAUNCH(MTP_K_PACK, launch_pack_rows(pa, s, pdl_first));
     HeadsTc g;
     std::memset(&g, 0, sizeof(g));
     g.w128 = c->heads_map; g.w144 = c->heads_map144;
@@ -806,10 +808,10 @@ int enqueue_step(mtp_ctx* c, int n, int k, cudaStream_t s, bool pdl, Prof* prof,
         }
         const bool fused = heads_fused_ok(c, k, true);
         if (fused)  // candidates, lse and the logits (kept for mtp_debug_logits and the union lattice)
-            MTP_TRY(launch_heads_fused(c, c->d_h_last, B, n, k, c->d_cand_ids, c->d_cand_logp, c->d_lse, c->d_logits,
-                                       s, pdl, prof));
+            MTP_TRY(launch_heads_fused(c, c->d_h_last, false, B, n, k, c->d_cand_ids, c->d_cand_logp, c->d_lse,
+                                       c->d_logits, s, pdl, pdl, prof));
         else
-            MTP_TRY(launch_heads_batched(c, c->d_h_last, B, n, c->d_logits, s, pdl, prof));
+            MTP_TRY(launch_heads_batched(c, c->d_h_last, false, B, n, c->d_logits, s, pdl, pdl, prof));
         SelectArgs sa = select_base(c, n, k);
         sa.pre_topk = fused ? 1 : 0;
         sa.lane = lane ? 1 : 0;
@@ -1793,42 +1795,41 @@ MTP_API int mtp_heads_topk(mtp_ctx* c, int batch, const void* hidden, int hidden
     const bool fused = c->use_batched && c->batched_ok && batch > MAX_ROWS && heads_fused_ok(c, k, false);
     const bool tc = !fused && c->use_batched && c->batched_ok && batch > MAX_ROWS && tc_rows > MAX_ROWS;
     const int chunk = fused ? c->bm_max : (tc ? tc_rows : MAX_ROWS);
+    // The rows are read where they are when their alignment allows it (fp32 by every kernel, bf16 by the row
+    // pack); else, and for bf16 in the 8-row passes, they are converted first (a 256-row call with bf16 rows:
+    // 55 vs 61 us converted).  The call's first kernel waits for everything before it; the ones behind start under programmatic
+    // launch and fetch their weights meanwhile (one fp32 row, n = 4: 12.5 vs
+    // 16.4 us).
+    const bool bf = hidden_dtype == MTP_BF16, rows8 = !fused && !tc;
+    const size_t es = bf ? 2 : 4;
+    const bool direct = !(rows8 && bf) && (reinterpret_cast<uintptr_t>(hidden) & (bf ? 7 : 15)) == 0;
+    const bool pdl = c->use_pdl;
     for (int b0 = 0; b0 < batch; b0 += chunk) {
         const int m = std::min(chunk, batch - b0);
+        const void* x = static_cast<const char*>(hidden) + (size_t)b0 * d * es;
+        if (!direct) {
+            float* dst = rows8 ? xbuf(c, 0) : c->d_bx;
+            CUDA_TRY(launch_convert_rows(x, bf, dst, m, d, s));
+            x = dst;
+        }
+        const bool x_bf16 = direct && bf, pdl_first = !direct && pdl;
         if (fused) {
-            const size_t es = hidden_dtype == MTP_BF16 ? 2 : 4;
-            CUDA_TRY(launch_convert_rows(static_cast<const char*>(hidden) + (size_t)b0 * d * es,
-                                         hidden_dtype == MTP_BF16, c->d_bx, m, d, s));
-            MTP_TRY(launch_heads_fused(c, c->d_bx, m, n, k, out_ids + (size_t)b0 * n * k,
+            MTP_TRY(launch_heads_fused(c, x, x_bf16, m, n, k, out_ids + (size_t)b0 * n * k,
                                        out_logp + (size_t)b0 * n * k, out_lse ? out_lse + (size_t)b0 * n : nullptr,
-                                       out_logits ? out_logits + (size_t)b0 * n * V : nullptr, s, false, prof));
+                                       out_logits ? out_logits + (size_t)b0 * n * V : nullptr, s, pdl_first, pdl, prof));
             continue;
         }
-        if (tc) {
-            const size_t es = hidden_dtype == MTP_BF16 ? 2 : 4;
-            CUDA_TRY(launch_convert_rows(static_cast<const char*>(hidden) + (size_t)b0 * d * es,
-                                         hidden_dtype == MTP_BF16, c->d_bx, m, d, s));
-            float* logits = out_logits ? out_logits + (size_t)b0 * n * V : c->d_logits;
-            MTP_TRY(launch_heads_batched(c, c->d_bx, m, n, logits, s, false, prof));
-            SelectArgs sa = select_base(c, n, k);
-            sa.logits = logits;
-            sa.lse = out_lse ? out_lse + (size_t)b0 * n : c->d_lse;
-            sa.cand_ids = out_ids + (size_t)b0 * n * k;
-            sa.cand_logp = out_logp + (size_t)b0 * n * k;
-            CUDA_TRY(launch_select(sa, m, false, s, false));
-            continue;
-        }
-        const size_t es = hidden_dtype == MTP_BF16 ? 2 : 4;
-        CUDA_TRY(launch_convert_rows(static_cast<const char*>(hidden) + (size_t)b0 * d * es,
-                                     hidden_dtype == MTP_BF16, xbuf(c, 0), m, d, s));
         float* logits = out_logits ? out_logits + (size_t)b0 * n * V : c->d_logits;
-        MTP_TRY(launch_heads(c, xbuf(c, 0), m, n, logits, nullptr, 0, s, false, prof));
+        if (tc)
+            MTP_TRY(launch_heads_batched(c, x, x_bf16, m, n, logits, s, pdl_first, pdl, prof));
+        else
+            MTP_TRY(launch_heads(c, static_cast<const float*>(x), m, n, logits, nullptr, 0, s, pdl_first, prof));
         SelectArgs sa = select_base(c, n, k);
         sa.logits = logits;
         sa.lse = out_lse ? out_lse + (size_t)b0 * n : c->d_lse;
         sa.cand_ids = out_ids + (size_t)b0 * n * k;
         sa.cand_logp = out_logp + (size_t)b0 * n * k;
-        CUDA_TRY(launch_select(sa, m, false, s, false));
+        CUDA_TRY(launch_select(sa, m, false, s, pdl));
     }
     return MTP_OK;
 }
