@@ -9,7 +9,7 @@
 //
 //   D = (Z_hi + Z_lo) W_slice^T      tcgen05.mma, M = 128 rows (TMEM lanes),
 //                                    N = 128 or 144 vocabulary columns, K = d
-//                                    in 64-wide chunks through a 4-stage TMA
+//                                    in 64-wide chunks through a 2-stage TMA
 //                                    ring (128-byte swizzled tiles)
 //   phase 1   thread = (row, half of the columns), one pass: max, sum of exp,
 //             sum and sum of squares of the logits (logit = D + b, read back
@@ -19,14 +19,20 @@
 //             and the row's mean and sd
 //   phase 2   logp = logit - lse (one fp32 subtraction); the candidates are
 //             logp >= T, T = mean + z sd - lse with z such that a normal row
-//             would have about 4k + 16 of them; each half's best KM candidates
-//             by (logp desc, id asc), kept sorted in registers, merged into the
-//             slice's list, which goes to the CTA that owns the row (16 rows per
-//             CTA) in its shared memory
-//   merge     the owner merges the 8 sorted lists into the row's top-k (8 lanes
-//             per row, one per list, a shuffle arg-max per step); if any
-//             row of the tile had fewer than k candidates in all, the cluster
-//             runs phase 2 again with no threshold
+//             would have about 2k + 24 of them; each thread sends its half's
+//             candidates (32 at most) to the CTA that owns the row (16 rows per
+//             CTA), in its shared memory
+//   rank      a warp of the owner per row: a candidate's place is the number of
+//             candidates that beat it (logp desc, id asc); the first k go out.
+//             If a row of the tile had fewer than k candidates, or a half more
+//             than 32, the cluster takes the exact way instead: each half's best
+//             KM sorted by insertion, the halves and then the 8 slices merged
+//             (8 lanes per row, one per list, a shuffle arg-max per step)
+//
+// What bounds it: chains of dependent instructions per row, and at one CTA per
+// SM 15 clusters of 8 fit the GPU at once, so that 256 rows of 8 heads (16
+// clusters) ran in two waves.  A two-stage ring lets two CTAs share an SM; no
+// list is kept sorted on the way.  256 rows, n = 8, top-16: HT_NEW vs 52.9 us.
 //
 // Ranking on logp after the lse is known (not on the logits) keeps the
 // candidates exactly those of a top-k over the logp row, equal values
@@ -50,23 +56,26 @@ constexpr int HT_SLICES = 8;     // vocabulary slices per head (cluster size)
 constexpr int HT_SLICE = 128;    // vocabulary rows of slices 0..6
 constexpr int HT_NMAX = 144;     // N of the last slice (up to 137 rows)
 constexpr int HT_THREADS = 256;  // two warps per TMEM lane quarter (halves of the columns)
-constexpr int HT_STAGES = 4;
+constexpr int HT_STAGES = 2;     // two CTAs per SM
 constexpr int HT_ROWS_PER_OWNER = HT_M / HT_SLICES;  // rows whose merge each CTA of the cluster does
 constexpr uint32_t HT_A_BYTES = HT_M * HT_K * 2;
 constexpr uint32_t HT_B_BYTES = HT_NMAX * HT_K * 2;
 constexpr uint32_t HT_STAGE = 2 * HT_A_BYTES + HT_B_BYTES;  // multiple of 1024
 constexpr uint32_t HT_SMEM = HT_STAGES * HT_STAGE + 1024;
 constexpr uint32_t HT_TMEM_COLS = 256;
-// after the MMAs the ring is free: the candidate lists pushed by the cluster (at most
-// 2 x 16 rows x 8 slices x 32 entries x 4 B = 32 KB), each thread's staging row of 33 floats,
-// then the logit rows (128 x 137 floats, phase 1) or the two halves' lists (phase 2)
-constexpr uint32_t HT_STAGING = 32 * 1024;
-constexpr uint32_t HT_LOGIT_STAGE = 68 * 1024;
-constexpr uint32_t HT_HALF_LISTS = 68 * 1024;
-constexpr int HT_LOGIT_PITCH = 137;
-static_assert(HT_STAGING + HT_THREADS * 33 * 4 <= HT_LOGIT_STAGE, "staging rows");
-static_assert(HT_LOGIT_STAGE + HT_M * HT_LOGIT_PITCH * 4 <= HT_STAGES * HT_STAGE, "logit rows fit the ring");
+// After the MMAs the ring is free.  Candidates sent by the cluster: [16 rows][16 halves][32] of (logp,
+// id), 64 KB; then each thread's staging row of 33 floats (a warp's 32 rows: logits on their way out, a
+// block's logp values, a row's candidates while they are ranked).  The exact way's lists: those pushed by
+// the cluster (at most 2 x 16 rows x 8 slices x 32 entries x 4 B = 32 KB) at the start, the two halves'
+// lists (64 KB) behind them, over the staging rows.
+constexpr int HT_CAND = 32;      // candidates of a half that are sent
+constexpr int HT_HALVES = 2 * HT_SLICES;
+constexpr uint32_t HT_STAGING = 64 * 1024;
+constexpr uint32_t HT_HALF_LISTS = 32 * 1024;
+static_assert(HT_ROWS_PER_OWNER * HT_HALVES * HT_CAND * 8 <= HT_STAGING, "sent candidates");
+static_assert(HT_STAGING + HT_THREADS * 33 * 4 <= HT_STAGES * HT_STAGE, "staging rows fit the ring");
 static_assert(HT_HALF_LISTS + 2 * HT_M * 32 * 8 <= HT_STAGES * HT_STAGE, "half lists fit the ring");
+static_assert(HT_HALVES * HT_CAND * 8 <= 32 * 33 * 4, "a row's candidates fit a warp's staging rows");
 
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
     asm volatile(
@@ -86,6 +95,13 @@ __device__ __forceinline__ void st_dsmem4(uint32_t addr, float4 v) {
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z),
                  "f"(v.w)
                  : "memory");
+}
+
+__device__ __forceinline__ void st_dsmem2(uint32_t addr, float v, int id) {
+    asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(__float_as_int(v)), "r"(id) : "memory");
+}
+__device__ __forceinline__ void st_dsmem_i32(uint32_t addr, int v) {
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
 // Insert (v, id) into the sorted list (value desc; an equal value already in the
@@ -109,7 +125,7 @@ __device__ __forceinline__ void topk_insert(float (&val)[KM], int (&ids)[KM], fl
 }
 
 template <int KM>
-__global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 1)
+__global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 2)
     heads_tc_kernel(const __grid_constant__ CUtensorMap tw128, const __grid_constant__ CUtensorMap tw144,
                     const __grid_constant__ CUtensorMap tah, const __grid_constant__ CUtensorMap tal,
                     const HeadsTcArgs a) {
@@ -120,6 +136,7 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
     __shared__ float4 s_stat[HT_M];  // per row: this slice's max, sum of exp, sum and sum of squares
     __shared__ float4 s_half[2][HT_M];  // the same per half of the columns
     __shared__ int s_ok, s_short;
+    __shared__ int s_cnt[HT_ROWS_PER_OWNER * HT_HALVES];  // candidates of the owned rows, per half
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(ht_raw) + 1023) & ~(uintptr_t)1023);
     TraceEnd trace_guard(a.trace);
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -215,7 +232,8 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
     const bool warp_on = ok && arow + lq * 32 < a.m;  // warp-uniform: a warp of padding rows only waits
     const uint32_t taddr = tmem + ((uint32_t)(lq * 32) << 16);
     const int cbeg = half * 64, cend = half ? N : 64;  // columns of this thread: [cbeg, cend) of the slice
-    float* lst = a.out_logits ? reinterpret_cast<float*>(smem + HT_LOGIT_STAGE) + (size_t)rt * HT_LOGIT_PITCH : nullptr;
+    float* wstg = reinterpret_cast<float*>(smem + HT_STAGING) + (size_t)warp * 32 * 33;  // the warp's staging rows
+    float* stg = wstg + lane * 33;
 
     // ---- phase 1, one pass: per (row, half), max, sum of exp (rescaled when a block of 32 raises
     // the max), and sum and sum of squares of the logits ----
@@ -234,8 +252,17 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
                 if (c < cnt) {
                     s1 += v[e];
                     s2 = fmaf(v[e], v[e], s2);
-                    if (lst) lst[c] = v[e];
                 }
+            }
+            if (a.out_logits) {  // through the staging rows: 32 consecutive logits of a row per store
+#pragma unroll
+                for (int e = 0; e < 32; ++e) stg[e] = v[e];
+                __syncwarp();
+                const int c = c0 + lane, rows = min(32, a.m - arow - lq * 32);
+                float* dst = a.out_logits + (size_t)(arow + lq * 32) * a.ldl + (size_t)head * a.V + v0 + c;
+                if (c < cnt && c < cend)
+                    for (int r = 0; r < rows; ++r) dst[(size_t)r * a.ldl] = wstg[r * 33 + lane];
+                __syncwarp();
             }
             if (cm > mx) {
                 sm *= __expf(mx - cm);
@@ -254,17 +281,7 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
         const float S = (p.x == -INFINITY ? 0.f : p.y * __expf(p.x - M)) + (q.x == -INFINITY ? 0.f : q.y * __expf(q.x - M));
         s_stat[rt] = make_float4(M, S, p.z + q.z, p.w + q.w);
     }
-    if (lst && ok) {  // the staged logit rows, 16 per warp, coalesced
-        const float* st = reinterpret_cast<const float*>(smem + HT_LOGIT_STAGE);
-#pragma unroll 1
-        for (int r = warp * 16; r < warp * 16 + 16; ++r) {
-            const int grow = arow + r;
-            if (grow >= a.m) break;
-            float* dst = a.out_logits + (size_t)grow * a.ldl + (size_t)head * a.V + v0;
-            for (int c = lane; c < cnt; c += 32) dst[c] = st[(size_t)r * HT_LOGIT_PITCH + c];
-        }
-    }
-    trace_mark(a.trace, 2);  // logits written
+    trace_mark(a.trace, 2);  // slice statistics
     cluster_arrive_release();
     cluster_wait();
 
@@ -290,27 +307,115 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
         T = __fsub_rn(mean + a.z * sqrtf(var), lse);
     }
 
-    // ---- phase 2: each half's best KM candidates (logp >= T) by (logp desc, id asc); the two
-    // halves merged into the row's slice list, pushed to the CTA that owns the row; the owner
-    // merges the 8 slice lists.  T only prunes: if a row has fewer than k candidates in all, the
-    // cluster runs the phase again without it (exact either way). ----
-    const int owner = rt / HT_ROWS_PER_OWNER, slot = (rt % HT_ROWS_PER_OWNER) * HT_SLICES + j;
-    float* stg = reinterpret_cast<float*>(smem + HT_STAGING) + (size_t)tid * 33;
-    float* hv_s = reinterpret_cast<float*>(smem + HT_HALF_LISTS);  // [2][128][KM] values, then ids
-    int* hi_s = reinterpret_cast<int*>(smem + HT_HALF_LISTS) + 2 * HT_M * KM;
+    // ---- phase 2: the candidates logp >= T of each half, sent to the CTA that owns the row ----
+    const int owner = rt / HT_ROWS_PER_OWNER;
+    if (warp_on) {
+        const int box = (rt % HT_ROWS_PER_OWNER) * HT_HALVES + 2 * j + half;
+        const uint32_t dst = dsmem_addr(smem + (size_t)box * HT_CAND * 8, owner);
+        int found = 0;
+        // per 32 columns: the logp values go to this thread's staging row and the candidates form a
+        // mask; a warp then iterates as often as its busiest lane, not once per column
 #pragma unroll 1
-    for (int round = 0; round < 2; ++round) {
+        for (int c0 = cbeg; c0 < cend; c0 += 32) {
+            float v[32];
+            tmem_ld32(taddr + (uint32_t)c0, v);
+            uint32_t mask = 0;
+#pragma unroll
+            for (int e = 0; e < 32; ++e) {
+                const float x = __fsub_rn(v[e] + s_bias[min(c0 + e, HT_NMAX - 1)], lse);
+                stg[e] = x;
+                if (c0 + e < cnt && x >= T) mask |= 1u << e;
+            }
+            while (mask) {
+                const int e = __ffs(mask) - 1;
+                mask &= mask - 1;
+                if (found < HT_CAND) st_dsmem2(dst + found * 8, stg[e], v0 + c0 + e);
+                ++found;
+            }
+            __syncwarp();  // the next tcgen05.ld is warp-collective: reconverge after the per-lane loop
+        }
+        st_dsmem_i32(dsmem_addr(&s_cnt[box], owner), found);
+    }
+    trace_mark(a.trace, 3);  // candidates sent
+    cluster_arrive_release();
+    cluster_wait();
+
+    // ---- rank: a warp per owned row ----
+    bool exact_way = false;
+    for (int rl = warp * 2; ok && rl < warp * 2 + 2; ++rl) {
+        const int grow = arow + j * HT_ROWS_PER_OWNER + rl;
+        if (grow >= a.m) break;
+        const int have = lane < HT_HALVES ? s_cnt[rl * HT_HALVES + lane] : 0;
+        int incl = have;
+#pragma unroll
+        for (int o = 1; o < HT_HALVES; o <<= 1) {
+            const int u = __shfl_up_sync(FULL_MASK, incl, o);
+            if (lane >= o) incl += u;
+        }
+        const int total = __shfl_sync(FULL_MASK, incl, HT_HALVES - 1);
+        if (__any_sync(FULL_MASK, have > HT_CAND) || total < a.k) {  // warp-uniform
+            exact_way = true;
+            continue;
+        }
+        int2* list = reinterpret_cast<int2*>(wstg);
+        const int2* box = reinterpret_cast<const int2*>(smem) + (size_t)rl * HT_HALVES * HT_CAND;
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < HT_HALVES; ++h) {
+            const int n = __shfl_sync(FULL_MASK, have, h), at = __shfl_sync(FULL_MASK, incl, h) - n;
+            if (lane < n) list[at + lane] = box[h * HT_CAND + lane];
+        }
+        __syncwarp();
+        const size_t o = ((size_t)grow * a.n + head) * a.k;
+        for (int q0 = 0; q0 < total; q0 += 64) {  // two candidates per lane at a time
+            float v[2];
+            int id[2], rank[2] = {0, 0};
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int i = q0 + q * 32 + lane;
+                const int2 c = i < total ? list[i] : make_int2(0, 0);
+                v[q] = __int_as_float(c.x);
+                id[q] = c.y;
+            }
+#pragma unroll 4
+            for (int i = 0; i < total; ++i) {
+                const int2 c = list[i];
+                const float w = __int_as_float(c.x);
+#pragma unroll
+                for (int q = 0; q < 2; ++q) rank[q] += w > v[q] || (w == v[q] && c.y < id[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (q0 + q * 32 + lane < total && rank[q] < a.k) {
+                    a.out_ids[o + rank[q]] = id[q];
+                    a.out_logp[o + rank[q]] = v[q];
+                }
+        }
+    }
+    trace_mark(a.trace, 4);  // ranked
+    const int mine = __syncthreads_or(exact_way);
+    if (tid == 0) s_short = mine;
+    cluster_arrive_release();  // the owners are done with their candidates; every CTA's verdict is written
+    cluster_wait();
+    int any = 0;
+#pragma unroll
+    for (int r = 0; r < HT_SLICES; ++r) any |= ld_dsmem_i32(dsmem_addr(&s_short, r));
+    if (!any) cluster_arrive_relaxed();  // done reading the peers' verdicts (waited for before leaving)
+
+    // ---- the exact way: each half's best KM candidates by (logp desc, id asc); the two halves merged into
+    // the row's slice list, pushed to the CTA that owns the row; the owner merges the 8 slice lists ----
+    if (any) {
+        const int slot = (rt % HT_ROWS_PER_OWNER) * HT_SLICES + j;
+        float* hv_s = reinterpret_cast<float*>(smem + HT_HALF_LISTS);  // [2][128][KM] values, then ids
+        int* hi_s = reinterpret_cast<int*>(smem + HT_HALF_LISTS) + 2 * HT_M * KM;
+        float val[KM];
+        int ids[KM];
         if (warp_on) {
-            float val[KM];
-            int ids[KM];
 #pragma unroll
             for (int q = 0; q < KM; ++q) {
                 val[q] = -INFINITY;
                 ids[q] = 0x7fffffff;
             }
-            // per 32 columns: the logp values go to this thread's staging row; the candidates that
-            // beat the current last entry form a mask, and only those are inserted (a warp iterates
-            // as often as its busiest lane, not once per column)
 #pragma unroll 1
             for (int c0 = cbeg; c0 < cend; c0 += 32) {
                 float v[32];
@@ -321,7 +426,7 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
                 for (int e = 0; e < 32; ++e) {
                     const float x = c0 + e < cnt ? __fsub_rn(v[e] + s_bias[c0 + e], lse) : -INFINITY;
                     stg[e] = x;
-                    if (x >= T && x > thr) mask |= 1u << e;
+                    if (x > thr) mask |= 1u << e;
                 }
                 while (mask) {
                     const int e = __ffs(mask) - 1;
@@ -329,8 +434,11 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
                     const float x = stg[e];
                     if (x > val[KM - 1]) topk_insert<KM>(val, ids, x, v0 + c0 + e);
                 }
-                __syncwarp();  // the next tcgen05.ld is warp-collective: reconverge after the per-lane loop
+                __syncwarp();
             }
+        }
+        __syncthreads();  // the half lists lie over the staging rows
+        if (warp_on) {
             float* mv = hv_s + ((size_t)half * HT_M + rt) * KM;
             int* mi = hi_s + ((size_t)half * HT_M + rt) * KM;
 #pragma unroll
@@ -346,14 +454,12 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
             const float* bv = hv_s + ((size_t)HT_M + rt) * KM;
             const int* bi = hi_s + ((size_t)HT_M + rt) * KM;
             int pa = 0, pb = 0;
-            float ov[KM];
-            int oi[KM];
 #pragma unroll
             for (int t = 0; t < KM; ++t) {  // the first half holds the lower ids: it wins ties
                 const float x = av[pa], y = bv[pb];
                 const bool takea = x >= y;
-                ov[t] = takea ? x : y;
-                oi[t] = takea ? ai[pa] : bi[pb];
+                val[t] = takea ? x : y;
+                ids[t] = takea ? ai[pa] : bi[pb];
                 pa += takea;
                 pb += !takea;
             }
@@ -362,19 +468,18 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
             const uint32_t dv = dsmem_addr(cv, owner), di = dsmem_addr(ci, owner);
 #pragma unroll
             for (int q = 0; q < KM; q += 4) {
-                st_dsmem4(dv + 4 * q, make_float4(ov[q], ov[q + 1], ov[q + 2], ov[q + 3]));
-                st_dsmem4(di + 4 * q, make_float4(__int_as_float(oi[q]), __int_as_float(oi[q + 1]),
-                                                  __int_as_float(oi[q + 2]), __int_as_float(oi[q + 3])));
+                st_dsmem4(dv + 4 * q, make_float4(val[q], val[q + 1], val[q + 2], val[q + 3]));
+                st_dsmem4(di + 4 * q, make_float4(__int_as_float(ids[q]), __int_as_float(ids[q + 1]),
+                                                  __int_as_float(ids[q + 2]), __int_as_float(ids[q + 3])));
             }
         }
-        trace_mark(a.trace, 3 + 2 * round);  // candidate lists pushed
+        trace_mark(a.trace, 5);  // candidate lists pushed
         cluster_arrive_release();
         cluster_wait();
 
-        // ---- merge: rows 16 j .. 16 j + 15 of the tile; lanes 8 r .. 8 r + 7 (threads 0..127)
-        // walk the 8 sorted lists of row r (lane = slice), each step the group's best head is
-        // taken (ids differ between slices, so one lane advances) ----
-        bool short_row = false;
+        // merge: rows 16 j .. 16 j + 15 of the tile; lanes 8 r .. 8 r + 7 (threads 0..127) walk the 8 sorted
+        // lists of row r (lane = slice), each step the group's best head is taken (ids differ between slices,
+        // so one lane advances)
         if (ok && tid < HT_ROWS_PER_OWNER * HT_SLICES) {
             const int rl = tid >> 3, sl = tid & 7, grow = arow + j * HT_ROWS_PER_OWNER + rl;
             const float* cv = reinterpret_cast<const float*>(smem) + (size_t)(rl * HT_SLICES + sl) * KM;
@@ -406,24 +511,14 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
                 if (writer) {
                     a.out_ids[o + t] = bi;
                     a.out_logp[o + t] = bv;
-                    short_row |= bv == -INFINITY;  // fewer than k candidates: the lists ran out
                 }
             }
         }
-        trace_mark(a.trace, 4 + 2 * round);  // merged
-        if (round == 1) break;
-        const int mine = __syncthreads_or(short_row);
-        if (tid == 0) s_short = mine;
-        cluster_arrive_release();  // the owners are done with their lists; every CTA's verdict is written
-        cluster_wait();
-        int any = 0;
-#pragma unroll
-        for (int r = 0; r < HT_SLICES; ++r) any |= ld_dsmem_i32(dsmem_addr(&s_short, r));
-        if (!any) break;
-        T = -INFINITY;
+        trace_mark(a.trace, 6);  // merged
     }
     if (ok && a.out_lse && row_on && j == 0 && half == 0) a.out_lse[(size_t)row * a.n + head] = lse;
     if (!fin) mbar_wait(&done, 0, nullptr);  // MMAs may still run: let them finish before TMEM is freed
+    if (!any) cluster_wait();                // (the exact way's own barrier follows the reads)
     tc_fence_before();
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, HT_TMEM_COLS);
@@ -454,10 +549,10 @@ float normal_upper_quantile(double p) {
 cudaError_t launch_heads_tc(const HeadsTc& g0, cudaStream_t s, bool pdl) {
     HeadsTc g = g0;
     HeadsTcArgs& a = g.args;
-    // Candidate threshold: were a row's logits normal, about 4k + 16 of its V would lie above
-    // mean + z sd.  It only prunes the top-k work; rows left with fewer than k candidates
-    // run again without it.
-    a.z = normal_upper_quantile(std::min(0.5, (4.0 * a.k + 16.0) / a.V));
+    // Candidate threshold: were a row's logits normal, about 2k + 24 of its V would lie above
+    // mean + z sd.  It only prunes the ranking; a tile with a row left with fewer than k
+    // candidates (or with more than are sent) takes the exact way.
+    a.z = normal_upper_quantile(std::min(0.5, (2.0 * a.k + 24.0) / a.V));
     if (!heads_tc_supported(a.V, a.k) || a.m < 1 || a.n < 1 || a.k_chunks < 1 ||
         (a.a_rows != 32 && a.a_rows != 64 && a.a_rows != HT_M) || (a.m > a.a_rows && a.a_rows != HT_M))
         return cudaErrorInvalidValue;
