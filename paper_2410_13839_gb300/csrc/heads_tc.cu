@@ -10,7 +10,9 @@
 //   D = (Z_hi + Z_lo) W_slice^T      tcgen05.mma, M = 128 rows (TMEM lanes),
 //                                    N = 128 or 144 vocabulary columns, K = d
 //                                    in 64-wide chunks through a 2-stage TMA
-//                                    ring (128-byte swizzled tiles)
+//                                    ring (128-byte swizzled tiles); the rows of
+//                                    a whole tile are the same in the 8 CTAs, so
+//                                    each copies an eighth of them to all
 //   phase 1   thread = (row, half of the columns), one pass: max, sum of exp,
 //             sum and sum of squares of the logits (logit = D + b, read back
 //             from TMEM), the two halves combined in shared memory; the 8
@@ -19,20 +21,24 @@
 //             and the row's mean and sd
 //   phase 2   logp = logit - lse (one fp32 subtraction); the candidates are
 //             logp >= T, T = mean + z sd - lse with z such that a normal row
-//             would have about 2k + 24 of them; each thread sends its half's
-//             candidates (32 at most) to the CTA that owns the row (16 rows per
-//             CTA), in its shared memory
-//   rank      a warp of the owner per row: a candidate's place is the number of
-//             candidates that beat it (logp desc, id asc); the first k go out.
+//             would have about 2k + 24 of them; each thread lists its half's
+//             candidates (32 at most) in its CTA's shared memory
+//   rank      half a warp per row in the CTA that owns it (16 rows per CTA) reads
+//             the row's 16 lists over DSMEM, 16 loads in flight; a candidate's
+//             place is the number of candidates that beat it (logp desc, id
+//             asc); the first k go out.
 //             If a row of the tile had fewer than k candidates, or a half more
 //             than 32, the cluster takes the exact way instead: each half's best
 //             KM sorted by insertion, the halves and then the 8 slices merged
 //             (8 lanes per row, one per list, a shuffle arg-max per step)
 //
-// What bounds it: chains of dependent instructions per row, and at one CTA per
-// SM 15 clusters of 8 fit the GPU at once, so that 256 rows of 8 heads (16
-// clusters) ran in two waves.  A two-stage ring lets two CTAs share an SM; no
-// list is kept sorted on the way.  256 rows, n = 8, top-16: HT_NEW vs 52.9 us.
+// What bounds it: chains of dependent instructions per row (8 warps hold a
+// tile), then the ring's latency.  At one CTA per SM 15 clusters of 8 fit the
+// GPU at once, so that 256 rows of 8 heads (16 clusters) ran in two waves: more
+// clusters than that take a two-stage ring, which lets two CTAs share an SM.
+// No list is kept sorted on the way.  us a call, n = 8, top-16, against sorted
+// insertion in every thread and one CTA per SM: 9 rows 25 vs 35, 128 rows 27 vs
+// 37, 256 rows 32 vs 62, 500 rows 35 vs 99.
 //
 // Ranking on logp after the lse is known (not on the logits) keeps the
 // candidates exactly those of a top-k over the logp row, equal values
@@ -56,32 +62,47 @@ constexpr int HT_SLICES = 8;     // vocabulary slices per head (cluster size)
 constexpr int HT_SLICE = 128;    // vocabulary rows of slices 0..6
 constexpr int HT_NMAX = 144;     // N of the last slice (up to 137 rows)
 constexpr int HT_THREADS = 256;  // two warps per TMEM lane quarter (halves of the columns)
-constexpr int HT_STAGES = 2;     // two CTAs per SM
+constexpr int HT_MAX_STAGES = 4, HT_STAGES = 2;  // ring stages: one CTA per SM, two CTAs per SM
 constexpr int HT_ROWS_PER_OWNER = HT_M / HT_SLICES;  // rows whose merge each CTA of the cluster does
 constexpr uint32_t HT_A_BYTES = HT_M * HT_K * 2;
 constexpr uint32_t HT_B_BYTES = HT_NMAX * HT_K * 2;
 constexpr uint32_t HT_STAGE = 2 * HT_A_BYTES + HT_B_BYTES;  // multiple of 1024
-constexpr uint32_t HT_SMEM = HT_STAGES * HT_STAGE + 1024;
 constexpr uint32_t HT_TMEM_COLS = 256;
-// After the MMAs the ring is free.  Candidates sent by the cluster: [16 rows][16 halves][32] of (logp,
-// id), 64 KB; then each thread's staging row of 33 floats (a warp's 32 rows: logits on their way out, a
+// After the MMAs the ring is free.  Candidates of this slice: [128 rows][2 halves][32] of (logp, id), 64 KB; then each thread's staging row of 33 floats (a warp's 32 rows: logits on their way out, a
 // block's logp values, a row's candidates while they are ranked).  The exact way's lists: those pushed by
 // the cluster (at most 2 x 16 rows x 8 slices x 32 entries x 4 B = 32 KB) at the start, the two halves'
 // lists (64 KB) behind them, over the staging rows.
-constexpr int HT_CAND = 32;      // candidates of a half that are sent
+constexpr int HT_CAND = 32;      // candidates of a half that are listed
 constexpr int HT_HALVES = 2 * HT_SLICES;
 constexpr uint32_t HT_STAGING = 64 * 1024;
 constexpr uint32_t HT_HALF_LISTS = 32 * 1024;
-static_assert(HT_ROWS_PER_OWNER * HT_HALVES * HT_CAND * 8 <= HT_STAGING, "sent candidates");
+static_assert(HT_M * 2 * HT_CAND * 8 <= HT_STAGING, "candidate lists");
 static_assert(HT_STAGING + HT_THREADS * 33 * 4 <= HT_STAGES * HT_STAGE, "staging rows fit the ring");
 static_assert(HT_HALF_LISTS + 2 * HT_M * 32 * 8 <= HT_STAGES * HT_STAGE, "half lists fit the ring");
-static_assert(HT_HALVES * HT_CAND * 8 <= 32 * 33 * 4, "a row's candidates fit a warp's staging rows");
+constexpr int HT_ROW_CAND = 32 * 33 * 4 / 16;  // candidates of a row that are ranked (two rows in a warp's staging rows)
 
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
             smem_addr(dst)),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_addr(bar))
+        : "memory");
+}
+
+// The same box into every CTA of the cluster, at this offset, each completing on its own barrier.
+__device__ __forceinline__ void tma_load_2d_all(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, {%2, "
+        "%3}], [%4], %5;" ::"r"(smem_addr(dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_addr(bar)), "h"((uint16_t)0xff)
+        : "memory");
+}
+// Arrive on `bar` in every CTA of the cluster once the MMAs issued so far are done.
+__device__ __forceinline__ void tc_commit_all(uint64_t* bar) {
+    asm volatile(
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_addr(bar)),
+        "h"((uint16_t)0xff)
         : "memory");
 }
 
@@ -97,11 +118,10 @@ __device__ __forceinline__ void st_dsmem4(uint32_t addr, float4 v) {
                  : "memory");
 }
 
-__device__ __forceinline__ void st_dsmem2(uint32_t addr, float v, int id) {
-    asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(__float_as_int(v)), "r"(id) : "memory");
-}
-__device__ __forceinline__ void st_dsmem_i32(uint32_t addr, int v) {
-    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+__device__ __forceinline__ int2 ld_dsmem_i32x2(uint32_t addr) {
+    int2 v;
+    asm volatile("ld.shared::cluster.v2.s32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
+    return v;
 }
 
 // Insert (v, id) into the sorted list (value desc; an equal value already in the
@@ -129,14 +149,15 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
     heads_tc_kernel(const __grid_constant__ CUtensorMap tw128, const __grid_constant__ CUtensorMap tw144,
                     const __grid_constant__ CUtensorMap tah, const __grid_constant__ CUtensorMap tal,
                     const HeadsTcArgs a) {
+    const bool all = a.a_rows == HT_M;  // whole tiles: each CTA copies its 16 rows of a stage to all eight
     extern __shared__ __align__(1024) unsigned char ht_raw[];
-    __shared__ uint64_t full[HT_STAGES], empty[HT_STAGES], done;
+    __shared__ uint64_t full[HT_MAX_STAGES], empty[HT_MAX_STAGES], done;
     __shared__ uint32_t tmem_base;
     __shared__ float s_bias[HT_NMAX];
     __shared__ float4 s_stat[HT_M];  // per row: this slice's max, sum of exp, sum and sum of squares
     __shared__ float4 s_half[2][HT_M];  // the same per half of the columns
     __shared__ int s_ok, s_short;
-    __shared__ int s_cnt[HT_ROWS_PER_OWNER * HT_HALVES];  // candidates of the owned rows, per half
+    __shared__ int s_cnt[HT_M * 2];  // candidates of each row, per half
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(ht_raw) + 1023) & ~(uintptr_t)1023);
     TraceEnd trace_guard(a.trace);
     const int tid = threadIdx.x, warp = tid >> 5;
@@ -157,9 +178,9 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
         tmem_relinquish();
     }
     if (tid == 32) {
-        for (int s = 0; s < HT_STAGES; ++s) {
+        for (int s = 0; s < HT_MAX_STAGES; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
+            mbar_init(&empty[s], all ? HT_SLICES : 1);  // every CTA that a stage's copies go to has read it
         }
         mbar_init(&done, 1);
         fence_barrier_init();
@@ -168,11 +189,15 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
     for (int c = tid; c < HT_NMAX; c += HT_THREADS) s_bias[c] = c < cnt ? a.bias[wrow + c] : 0.f;
     tc_fence_before();
     __syncthreads();
+    if (all) {  // the peers' barriers are initialised before anything completes on them
+        cluster_arrive_release();
+        cluster_wait();
+    }
     tc_fence_after();
     const uint32_t tmem = tmem_base;
 
     // weight tiles of the first stages: independent of the previous kernel
-    const int pre = chunks < HT_STAGES ? chunks : HT_STAGES;
+    const int stages = a.stages, pre = min(chunks, stages);
     if (tid == 0) {
         for (int c = 0; c < pre; ++c) {
             unsigned char* st = smem + (size_t)c * HT_STAGE;
@@ -186,25 +211,31 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
 
     if (tid == 0) {  // producer
         for (int c = 0; c < chunks; ++c) {
-            const int s = c % HT_STAGES;
+            const int s = c % stages;
             unsigned char* st = smem + (size_t)s * HT_STAGE;
-            if (c >= HT_STAGES) {
-                if (!mbar_wait(&empty[s], (uint32_t)((c / HT_STAGES) - 1) & 1, a.err)) {
+            if (c >= stages) {
+                if (!mbar_wait(&empty[s], (uint32_t)((c / stages) - 1) & 1, a.err)) {
                     s_ok = 0;
                     break;
                 }
                 mbar_arrive_expect_tx(&full[s], stage_bytes);
                 tma_load_2d(st + 2 * HT_A_BYTES, wide ? &tw144 : &tw128, c * HT_K, wrow, &full[s]);
             }
-            tma_load_2d(st, &tah, c * HT_K, arow, &full[s]);
-            tma_load_2d(st + HT_A_BYTES, &tal, c * HT_K, arow, &full[s]);
+            if (all) {
+                constexpr int R = HT_M / HT_SLICES;
+                tma_load_2d_all(st + j * R * HT_K * 2, &tah, c * HT_K, arow + j * R, &full[s]);
+                tma_load_2d_all(st + HT_A_BYTES + j * R * HT_K * 2, &tal, c * HT_K, arow + j * R, &full[s]);
+            } else {
+                tma_load_2d(st, &tah, c * HT_K, arow, &full[s]);
+                tma_load_2d(st + HT_A_BYTES, &tal, c * HT_K, arow, &full[s]);
+            }
         }
     } else if (tid == 32) {  // MMA issuer
         const uint32_t idesc = f16_idesc(HT_M, N, false);
         int c = 0;
         for (; c < chunks; ++c) {
-            const int s = c % HT_STAGES;
-            if (!mbar_wait(&full[s], (uint32_t)(c / HT_STAGES) & 1, a.err)) break;
+            const int s = c % stages;
+            if (!mbar_wait(&full[s], (uint32_t)(c / stages) & 1, a.err)) break;
             tc_fence_after();
             const uint32_t hb = smem_addr(smem + (size_t)s * HT_STAGE), lb = hb + HT_A_BYTES, wb = lb + HT_A_BYTES;
 #pragma unroll
@@ -213,7 +244,10 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
                 tc_mma(tmem, sw128_desc(hb + kk * 32), dw, idesc, (c | kk) != 0);
                 tc_mma(tmem, sw128_desc(lb + kk * 32), dw, idesc, 1u);
             }
-            tc_commit(&empty[s]);
+            if (all)
+                tc_commit_all(&empty[s]);
+            else
+                tc_commit(&empty[s]);
         }
         if (c < chunks) s_ok = 0;
         tc_commit(&done);
@@ -307,11 +341,9 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
         T = __fsub_rn(mean + a.z * sqrtf(var), lse);
     }
 
-    // ---- phase 2: the candidates logp >= T of each half, sent to the CTA that owns the row ----
-    const int owner = rt / HT_ROWS_PER_OWNER;
+    // ---- phase 2: the candidates logp >= T of each half, listed ----
     if (warp_on) {
-        const int box = (rt % HT_ROWS_PER_OWNER) * HT_HALVES + 2 * j + half;
-        const uint32_t dst = dsmem_addr(smem + (size_t)box * HT_CAND * 8, owner);
+        int2* list = reinterpret_cast<int2*>(smem) + (size_t)(rt * 2 + half) * HT_CAND;
         int found = 0;
         // per 32 columns: the logp values go to this thread's staging row and the candidates form a
         // mask; a warp then iterates as often as its busiest lane, not once per column
@@ -329,66 +361,78 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
             while (mask) {
                 const int e = __ffs(mask) - 1;
                 mask &= mask - 1;
-                if (found < HT_CAND) st_dsmem2(dst + found * 8, stg[e], v0 + c0 + e);
+                if (found < HT_CAND) list[found] = make_int2(__float_as_int(stg[e]), v0 + c0 + e);
                 ++found;
             }
             __syncwarp();  // the next tcgen05.ld is warp-collective: reconverge after the per-lane loop
         }
-        st_dsmem_i32(dsmem_addr(&s_cnt[box], owner), found);
+        s_cnt[rt * 2 + half] = found;
     }
-    trace_mark(a.trace, 3);  // candidates sent
+    trace_mark(a.trace, 3);  // candidates listed
     cluster_arrive_release();
     cluster_wait();
 
-    // ---- rank: a warp per owned row ----
+    // ---- rank: half a warp per owned row ----
     bool exact_way = false;
-    for (int rl = warp * 2; ok && rl < warp * 2 + 2; ++rl) {
-        const int grow = arow + j * HT_ROWS_PER_OWNER + rl;
-        if (grow >= a.m) break;
-        const int have = lane < HT_HALVES ? s_cnt[rl * HT_HALVES + lane] : 0;
+    const int l16 = lane & 15, rl = warp * 2 + (lane >> 4), grow = arow + j * HT_ROWS_PER_OWNER + rl;
+    if (ok && arow + j * HT_ROWS_PER_OWNER + warp * 2 < a.m) {  // warp-uniform
+        const bool row_here = grow < a.m;
+        const int row_t = j * HT_ROWS_PER_OWNER + rl;  // the row within the tile; lane h of 16: half h & 1 of slice h / 2
+        const int have = row_here ? ld_dsmem_i32(dsmem_addr(&s_cnt[row_t * 2 + (l16 & 1)], l16 >> 1)) : 0;
         int incl = have;
 #pragma unroll
         for (int o = 1; o < HT_HALVES; o <<= 1) {
-            const int u = __shfl_up_sync(FULL_MASK, incl, o);
-            if (lane >= o) incl += u;
+            const int u = __shfl_up_sync(FULL_MASK, incl, o, 16);
+            if (l16 >= o) incl += u;
         }
-        const int total = __shfl_sync(FULL_MASK, incl, HT_HALVES - 1);
-        if (__any_sync(FULL_MASK, have > HT_CAND) || total < a.k) {  // warp-uniform
-            exact_way = true;
-            continue;
-        }
-        int2* list = reinterpret_cast<int2*>(wstg);
-        const int2* box = reinterpret_cast<const int2*>(smem) + (size_t)rl * HT_HALVES * HT_CAND;
+        const int total = __shfl_sync(FULL_MASK, incl, 15, 16);
+        const unsigned over = __ballot_sync(FULL_MASK, have > HT_CAND) >> (lane & 16) & 0xffffu;
+        const bool bad = row_here && (over || total < a.k || total > HT_ROW_CAND);
+        exact_way = bad;
+        const int cnt_r = row_here && !bad ? total : 0;
+        // the row's candidates as keys that order like (logp, lower id): the float's bits made monotonic
+        unsigned long long* keys = reinterpret_cast<unsigned long long*>(wstg) + (lane >> 4) * HT_ROW_CAND;
         __syncwarp();
 #pragma unroll
-        for (int h = 0; h < HT_HALVES; ++h) {
-            const int n = __shfl_sync(FULL_MASK, have, h), at = __shfl_sync(FULL_MASK, incl, h) - n;
-            if (lane < n) list[at + lane] = box[h * HT_CAND + lane];
+        for (int part = 0; part < HT_CAND; part += 16) {
+            int2 got[HT_HALVES];
+            if (part && !__any_sync(FULL_MASK, have > 16)) break;
+#pragma unroll
+            for (int h = 0; h < HT_HALVES; ++h) {
+                const int n = __shfl_sync(FULL_MASK, have, h, 16);
+                const int2* src = reinterpret_cast<const int2*>(smem) + (size_t)(row_t * 2 + (h & 1)) * HT_CAND + part + l16;
+                got[h] = cnt_r && part + l16 < n ? ld_dsmem_i32x2(dsmem_addr(src, h >> 1)) : make_int2(0, 0);
+            }
+#pragma unroll
+            for (int h = 0; h < HT_HALVES; ++h) {
+                const int n = __shfl_sync(FULL_MASK, have, h, 16), at = __shfl_sync(FULL_MASK, incl, h, 16) - n;
+                if (cnt_r && part + l16 < n) {
+                    const uint32_t f = __float_as_uint(__fadd_rn(__int_as_float(got[h].x), 0.f));  // -0 as 0
+                    const uint32_t mono = f ^ (f >> 31 ? 0xffffffffu : 0x80000000u);
+                    keys[at + part + l16] = (unsigned long long)mono << 32 | (0xffffffffu - (uint32_t)got[h].y);
+                }
+            }
         }
         __syncwarp();
         const size_t o = ((size_t)grow * a.n + head) * a.k;
-        for (int q0 = 0; q0 < total; q0 += 64) {  // two candidates per lane at a time
-            float v[2];
-            int id[2], rank[2] = {0, 0};
+        const int most = max(cnt_r, __shfl_xor_sync(FULL_MASK, cnt_r, 16));
+        for (int q0 = 0; q0 < most; q0 += 64) {  // four candidates per lane at a time
+            unsigned long long key[4];
+            int rank[4] = {0, 0, 0, 0};
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                const int i = q0 + q * 32 + lane;
-                const int2 c = i < total ? list[i] : make_int2(0, 0);
-                v[q] = __int_as_float(c.x);
-                id[q] = c.y;
-            }
+            for (int q = 0; q < 4; ++q) key[q] = q0 + q * 16 + l16 < cnt_r ? keys[q0 + q * 16 + l16] : 0ull;
 #pragma unroll 4
-            for (int i = 0; i < total; ++i) {
-                const int2 c = list[i];
-                const float w = __int_as_float(c.x);
+            for (int i = 0; i < cnt_r; ++i) {
+                const unsigned long long w = keys[i];
 #pragma unroll
-                for (int q = 0; q < 2; ++q) rank[q] += w > v[q] || (w == v[q] && c.y < id[q]);
+                for (int q = 0; q < 4; ++q) rank[q] += w > key[q];
             }
 #pragma unroll
-            for (int q = 0; q < 2; ++q)
-                if (q0 + q * 32 + lane < total && rank[q] < a.k) {
-                    a.out_ids[o + rank[q]] = id[q];
-                    a.out_logp[o + rank[q]] = v[q];
+            for (int q = 0; q < 4; ++q)
+                if (q0 + q * 16 + l16 < cnt_r && rank[q] < a.k) {
+                    const uint32_t mono = (uint32_t)(key[q] >> 32);
+                    a.out_ids[o + rank[q]] = (int)(0xffffffffu - (uint32_t)key[q]);
+                    a.out_logp[o + rank[q]] = __uint_as_float(mono ^ (mono >> 31 ? 0x80000000u : 0xffffffffu));
                 }
         }
     }
@@ -405,7 +449,7 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
     // ---- the exact way: each half's best KM candidates by (logp desc, id asc); the two halves merged into
     // the row's slice list, pushed to the CTA that owns the row; the owner merges the 8 slice lists ----
     if (any) {
-        const int slot = (rt % HT_ROWS_PER_OWNER) * HT_SLICES + j;
+        const int owner = rt / HT_ROWS_PER_OWNER, slot = (rt % HT_ROWS_PER_OWNER) * HT_SLICES + j;
         float* hv_s = reinterpret_cast<float*>(smem + HT_HALF_LISTS);  // [2][128][KM] values, then ids
         int* hi_s = reinterpret_cast<int*>(smem + HT_HALF_LISTS) + 2 * HT_M * KM;
         float val[KM];
@@ -565,12 +609,16 @@ cudaError_t launch_heads_tc(const HeadsTc& g0, cudaStream_t s, bool pdl) {
         kern = reinterpret_cast<const void*>(heads_tc_kernel<16>);
     else
         kern = reinterpret_cast<const void*>(heads_tc_kernel<32>);
-    cudaError_t e = ensure_kernel_smem(kern, HT_SMEM);
+    // Clusters of 8 at one CTA per SM: 15 fit this GPU at once; beyond, two CTAs per SM with half the ring
+    // each
+    a.stages = (a.m + HT_M - 1) / HT_M * a.n <= 15 ? HT_MAX_STAGES : HT_STAGES;
+    const size_t smem = a.stages * HT_STAGE + 1024;
+    cudaError_t e = ensure_kernel_smem(kern, HT_MAX_STAGES * HT_STAGE + 1024);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(HT_SLICES, a.n, (a.m + HT_M - 1) / HT_M);
     cfg.blockDim = dim3(HT_THREADS);
-    cfg.dynamicSmemBytes = HT_SMEM;
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

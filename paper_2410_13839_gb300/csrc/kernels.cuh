@@ -374,13 +374,14 @@ struct HeadsTcArgs {
     int32_t* out_ids; float* out_logp;   // [m][n][k]
     float* out_lse;               // [m][n] or null
     float* out_logits; int ldl;   // [m][ldl], head i at column i * V, or null
+    int stages;                   // set by launch_heads_tc: ring stages
     float z;                      // set by launch_heads_tc: candidates are logp >= mean + z sd of the row (pruning)
     int* err;
     unsigned long long* trace;
 };
 struct HeadsTc {
     CUtensorMap w128, w144;       // head weight rows [n_max * V][d]: boxes of 64 x 128 and 64 x 144 rows
-    CUtensorMap a_hi, a_lo;       // LN_f rows: boxes of 64 x a_rows rows
+    CUtensorMap a_hi, a_lo;       // LN_f rows: boxes of 64 x a_rows rows (a_rows = 128: of 64 x 16, copied to a cluster)
     HeadsTcArgs args;
 };
 bool heads_tc_supported(int V, int k);
