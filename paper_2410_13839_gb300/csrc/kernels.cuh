@@ -20,10 +20,12 @@ constexpr int MAX_ROWS = 8;      // rows per weight-streaming pass (B * n_heads 
 constexpr int PREFILL_ROWS = 128; // prompt positions of a decode step's prefill lane
 // Most prompt positions of one prefill pass (28 KB of buffers each at d = 1024).  A pass of a few
 // hundred rows is bound by its chain of dependent launches, like a decode step (0.55 ms for 128 rows,
-// 0.9 ms for 384), and a short last pass costs nearly as much as a long one.  Prefill of 32 / 128
-// serving prompts (12.8k / 48.6k positions): 7.6 / 29.3 ms in passes of 16384, 9.7 / 34.2 in
-// passes of 4096, 29.2 / 68.9 in passes of 384 / 1152; one 289-position prompt: 0.79 ms in one pass, 1.7 ms in three.
-constexpr int PREFILL_PASS_ROWS = 16384;
+// 0.9 ms for 384), and a short last pass costs nearly as much as a long one.  A multiple of 32 rows per
+// SM makes whole waves of the pair GEMM's 256 x 256 tiles (d = 1024 on 152 SMs: 19 row tiles times 12,
+// 16, 4 and 4 weight tiles over 76 pairs).  Prefill of 32 / 128 serving prompts (12.8k / 48.6k
+// positions): 7.7 / 28.4 ms at 96 rows per SM (14592), 7.6 / 29.3 in passes of 16384, 9.7 / 34.2 of 4096,
+// 29.2 / 68.9 of 384 / 1152; one 289-position prompt: 0.75 ms in one pass, 1.7 in three of 128.
+constexpr int PREFILL_PASS_ROWS_PER_SM = 96;
 constexpr int MAX_TOPK = 32;     // one warp lane per candidate
 constexpr int MAX_NHEADS = 8;    // prediction heads
 constexpr int MAX_VOCAB = 1056;  // 33 logits per lane in the top-k warp

@@ -8,7 +8,8 @@
 //                 (LN_f + n x V logits) and one select kernel (log-softmax,
 //                 top-k, Viterbi, acceptance, slot bookkeeping);
 //   prefill      = the same layer stack over the prompt: bf16 models in passes of
-//                 up to PREFILL_PASS_ROWS positions, fp32 models 8 rows at a time.
+//                 up to PREFILL_PASS_ROWS_PER_SM positions per SM, fp32 models 8
+//                 rows at a time.
 // Within a pass the kernels are chained with programmatic dependent launch;
 // each (n_heads, top_k) decode step is captured once into a CUDA graph.
 #include <cuda_runtime.h>
@@ -540,13 +541,13 @@ int launch_step_pass(mtp_ctx* c, int rows, int rpg, int seq_base, cudaStream_t s
 
 // Rows of the batched buffers: a decode step's (every slot's fed rows plus a prefill lane of up
 // to PREFILL_ROWS prompt rows), and for bf16 models a whole prefill pass: as many prompt rows as
-// the slots can hold, up to PREFILL_PASS_ROWS.
+// the slots can hold, up to PREFILL_PASS_ROWS_PER_SM per SM (whole groups of 8).
 int batched_rows(const mtp_ctx* c) {
     const mtp_config& cf = c->cfg;
     const long long step = (long long)cf.max_batch * cf.n_heads_max + PREFILL_ROWS;
     if (c->wbytes != 2) return (int)step;
     const long long prompts = ((long long)cf.max_batch * cf.max_ctx + 7) / 8 * 8;
-    return (int)std::max(step, std::min<long long>(prompts, PREFILL_PASS_ROWS));
+    return (int)std::max(step, std::min<long long>(prompts, PREFILL_PASS_ROWS_PER_SM * c->num_sms / 8 * 8));
 }
 
 // Buffers and tensor maps of the batched path (bf16 weights only).

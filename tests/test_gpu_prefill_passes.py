@@ -1,7 +1,7 @@
 """Prefill passes (Sec. III-A: the prompt runs through the blocks as one sequence)
 against the oracle at the sizes where a pass can go wrong: fewer rows than an
 attention group, the edges of the 128-row tiles, and prompts or batches of
-prompts just below, at and past the rows one pass holds (16384)."""
+prompts just below, at and past the rows one pass holds (96 per SM: 14592)."""
 import copy
 
 import numpy as np
@@ -35,8 +35,8 @@ def test_one_prompt(length):
 @pytest.mark.parametrize("lengths,passes", [
     ([5, 130, 61], 1),
     ([700, 1300, 900, 1100, 500, 33], 1),
-    ([1024] * 15 + [1016, 8], 1),         # exactly one pass of 16384 rows
-    ([1024] * 15 + [1016, 9], 2),         # one prompt row left for the second pass
+    ([1024] * 14 + [248, 8], 1),          # exactly one pass of 14592 rows
+    ([1024] * 14 + [248, 9], 2),          # one prompt row left for the second pass
     ([900, 333] * 14, 2),                 # a prompt cut by the end of the pass
 ])
 def test_admitted_prompts(lengths, passes):
