@@ -6,14 +6,19 @@
 // w: bf16 weights, K-major ([N_w][K]); a_hi + a_lo: the fp32 activations as
 // two bf16 parts, K-major ([M][K]).  The weights are the MMA's M = 128 side
 // (one 128-row tile per CTA) and the activation rows its N side (NT per
-// tile), so a handful of fed rows still fills the tensor core; both parts of
-// the activations go through the same accumulator (two MMAs per k-step),
-// which keeps the product to fp32 accuracy.
+// tile), so a handful of fed rows still fills the tensor core.  The two parts
+// of the activations lie one behind the other and are one operand of 2 NT
+// columns, whose two halves of the accumulator are added when it is read: an
+// MMA of N = 128 takes as long as one of N = 256 (W1 of 512 rows with two MMAs
+// per k-step, one per part: 13.2 us; with one: 11.3; d = 1024, q|k|v, W_o, W1
+// and W2 of 128 rows: 9.5 us on average, now 8.4).  Each accumulator truncates
+// half as often, too: K = 4096 is off by 4.4e-6 of the result's scale, by
+// 9.2e-6 with both parts in one accumulator.
 //
 // Per CTA: one elected thread streams 64-wide k-chunks of the weight tile
 // and of both activation parts into a 4-stage shared-memory ring with TMA
 // (128-byte swizzled tiles), a second elected thread issues tcgen05.mma
-// into a TMEM accumulator (128 lanes x NT fp32 columns) and releases each
+// into a TMEM accumulator (128 lanes x 2 NT fp32 columns) and releases each
 // stage with tcgen05.commit.  Eight warps read the accumulator back with
 // tcgen05.ld and finish it from the registers (tc_epilogue.cuh): warps w and
 // w + 4 share TMEM lanes 32 (w % 4) .., i.e. weight rows, and take half of the
@@ -73,9 +78,9 @@ __device__ __forceinline__ uint32_t mapa_rank(uint32_t saddr, int rank) {
 }
 
 // Instruction descriptor of kind::f16: fp32 accumulator, bf16 A and B, both
-// K-major, M = 128, N = nt.
-__host__ __device__ constexpr uint32_t tc_idesc(int nt) {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(nt >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
+// K-major, M = 128, N = n.
+__host__ __device__ constexpr uint32_t tc_idesc(int n) {
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(TC_M >> 4) << 24);
 }
 
 template <int NT, int EPI, bool CLUSTER>
@@ -84,7 +89,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
                    const __grid_constant__ CUtensorMap tal, const TcGemmArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     constexpr uint32_t A_BYTES = NT * TC_K * 2, STAGE = TC_W_BYTES + 2 * A_BYTES;
-    constexpr uint32_t TMEM_COLS = NT < 32 ? 32 : NT;
+    constexpr uint32_t TMEM_COLS = 2 * NT;  // the products with the hi parts, then with the lo parts
     constexpr int TC_STAGES = tc_stages(NT);
     __shared__ uint64_t full[TC_MAX_STAGES], empty[TC_MAX_STAGES], done, red_bar;
     __shared__ uint32_t tmem_base;
@@ -164,20 +169,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             tma_load_2d(st + TC_W_BYTES + A_BYTES, &tal, kx, arow, &full[s]);
         }
     } else if (tid == 32) {  // MMA issuer
-        constexpr uint32_t IDESC = tc_idesc(NT);
+        constexpr uint32_t IDESC = tc_idesc(2 * NT);  // the stage's hi and lo rows are one operand
         int c = 0;
         for (; c < chunks; ++c) {
             const int s = c % TC_STAGES;
             if (!mbar_wait(&full[s], (uint32_t)(c / TC_STAGES) & 1, a.err)) break;
             tc_fence_after();
             const uint32_t wb = smem_addr(smem + (size_t)s * STAGE);
-            const uint32_t hb = wb + TC_W_BYTES, lb = hb + A_BYTES;
+            const uint32_t ab = wb + TC_W_BYTES;
 #pragma unroll
-            for (int kk = 0; kk < TC_K / 16; ++kk) {
-                const uint64_t dw = sw128_desc(wb + kk * 32);
-                tc_mma(tmem, dw, sw128_desc(hb + kk * 32), IDESC, (c | kk) != 0);
-                tc_mma(tmem, dw, sw128_desc(lb + kk * 32), IDESC, 1u);
-            }
+            for (int kk = 0; kk < TC_K / 16; ++kk)
+                tc_mma(tmem, sw128_desc(wb + kk * 32), sw128_desc(ab + kk * 32), IDESC, (c | kk) != 0);
             tc_commit(&empty[s]);  // stage s is free once these MMAs have read it
         }
         if (c < chunks) s_ok = 0;
@@ -233,15 +235,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         if (tid == 0) mbar_arrive_expect_tx(&red_bar, part_bytes * (uint32_t)(Sc - 1));
         __syncthreads();
         cluster_arrive_release();  // this CTA's ring is free and its barrier armed
-        float v[4][N];
+        float v[4][N], w[4][N];
         // unit u: rows r0(u) .. + N of share p(u)
         auto share = [&](int u) { return Sc == 4 ? u : u >> 1; };
         auto first = [&](int u) { return half * (R / 2) + (Sc == 4 ? 0 : (u & 1) * N); };
 #pragma unroll
-        for (int u = 0; u < 4; ++u) tmem_ld_issue<N>(acc + (uint32_t)(share(u) * R + first(u)), v[u]);
+        for (int u = 0; u < 4; ++u) {
+            tmem_ld_issue<N>(acc + (uint32_t)(share(u) * R + first(u)), v[u]);
+            tmem_ld_issue<N>(acc + (uint32_t)(NT + share(u) * R + first(u)), w[u]);
+        }
         tmem_ld_wait();
 #pragma unroll
-        for (int u = 0; u < 4; ++u) tmem_ld_done(v[u]);
+        for (int u = 0; u < 4; ++u) {
+            tmem_ld_done(v[u]);
+            tmem_ld_done(w[u]);
+#pragma unroll
+            for (int e = 0; e < N; ++e) v[u][e] += w[u][e];
+        }
         if (good) {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -295,8 +305,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         // the tile's first split adds the bias (heads: rows past n_valid have none)
         const float bias = a.bias && split == 0 && (!a.n_valid || f < a.n_valid) ? __ldg(a.bias + f) : 0.f;
         for (int j0 = half * (NT / 2); j0 < (half + 1) * (NT / 2) && j0 < rows; j0 += N) {
-            float v[N];
-            tmem_ld<N>(acc + (uint32_t)j0, v);
+            float v[N], w[N];
+            tmem_ld_issue<N>(acc + (uint32_t)j0, v);
+            tmem_ld_issue<N>(acc + (uint32_t)(NT + j0), w);
+            tmem_ld_wait();
+            tmem_ld_done(v);
+            tmem_ld_done(w);
+#pragma unroll
+            for (int e = 0; e < N; ++e) v[e] += w[e];
             tc_epilogue<EPI, true>(a, v, arow + j0, j0, rows - j0, f, bias, s_rowbase, s_rowt);
         }
         trace_mark(a.trace, 5);  // thread 0's stores issued

@@ -310,10 +310,11 @@ cudaError_t launch_epi(const TcGemm& g, int pairs, cudaStream_t s, bool pdl) {
 
 }  // namespace
 
-// Both kernels take about 0.66 us per 64-wide k-chunk and wave of tiles, this one 7.5 us around that
-// (filling the ring, the last tile's epilogue) and tc_gemm.cu 2.7 us: in chunks, 11 and 4.  Measured at
-// K = 1024, us by waves: here 18.1 / 29.0 / 40.2 / 49.5 for 1-4 waves of 256 x 256 tiles, tc_gemm.cu
-// 13.3 / 22.9 / 34.5 / 45.0 for 1-4 waves of 128 x 128.  So one wave there stays there.
+// This kernel takes about 0.66 us per 64-wide k-chunk and wave of tiles and 7 us around that (filling the
+// ring, the last tile's epilogue), tc_gemm.cu 0.6 and under 2: in chunks, 11 and less than 4.  Measured at
+// K = 1024, us by waves: here 17.5 / 28.3 / 39.2 / 49.5 for 1-4 waves of 256 x 256 tiles, tc_gemm.cu
+// 11.2 / 20.8 / 30.0 / 39.7 for 1-4 waves of 128 x 128, of which there are twice as many where no tile is
+// ragged.  So one wave there stays there, and two do where two are needed here.
 bool tc_gemm_pair_fits(int n_w, int m, int k_chunks, int splits, int num_sms) {
     if (n_w % (2 * TP_F) || m <= TP_N / 2) return false;
     const int tiles = n_w / (2 * TP_F) * ((m + TP_N - 1) / TP_N), pairs = std::max(1, num_sms / 2);
