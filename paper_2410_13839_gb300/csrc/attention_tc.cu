@@ -262,30 +262,32 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
             s_issued = ok;
         }
         for (int2 t = first; ok && t.x < nseg; ++i) {
+            const int keys = seg_kmax[t.x] - t.y * PA_KEYS;  // of the item that some row of the tile sees
             t = next_item(t);
-            // S has been read into registers: the next item's overwrites it
-            ok = wait(&s_read, (uint32_t)i & 1);
-            if (!ok) break;
-            if (t.x < nseg) {
-                issue_s(i + 1);
-                if (!ok) break;
-                ++s_issued;
-            }
             const uint32_t vb = smem_addr(sm + OFF_KV + (uint32_t)(2 * (i & 1) + 1) * PA_TILE);
 #pragma unroll
             for (int half = 0; half < 2; ++half) {
+                if (half) {  // S is in the rows' registers: the next item's overwrites it
+                    ok = wait(&s_read, (uint32_t)i & 1);
+                    if (!ok) break;
+                    if (t.x < nseg) {
+                        issue_s(i + 1);
+                        if (!ok) break;
+                        ++s_issued;
+                    }
+                }
                 ok = wait(&p_full[half], (uint32_t)i & 1);
                 if (!ok) break;
                 tc_fence_after();
-                if (lane == 0) {
+                if (lane == 0 && half * PA_HALF < keys) {
 #pragma unroll
                     for (int kk = 0; kk < PA_HALF / 16; ++kk) {
                         const uint64_t bv = sw128_mn_desc(vb + (half * (PA_HALF / 16) + kk) * 2048);
                         tc_mma_ta(tmem + TM_O, tmem + TM_P + kk * 8, bv, IDESC_O, (i | half | kk) != 0);
                         tc_mma_ta(tmem + TM_O, tmem + TM_PLO + kk * 8, bv, IDESC_O, 1u);
                     }
-                    tc_commit(&pv_done[half]);
                 }
+                if (lane == 0) tc_commit(&pv_done[half]);
                 __syncwarp();
                 ++pv_issued;
             }
@@ -344,44 +346,59 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
                 break;
             }
             tc_fence_after();
-            float sv[PA_KEYS];
-#pragma unroll
-            for (int c0 = 0; c0 < PA_KEYS; c0 += 32) {
-                float v[32];
-                tmem_ld32(base + TM_S + c0, v);
-#pragma unroll
-                for (int e = 0; e < 32; ++e) sv[c0 + e] = v[e];
-            }
-            if (!__all_sync(FULL_MASK, lim >= PA_KEYS - 1)) {
-#pragma unroll
-                for (int c = 0; c < PA_KEYS; ++c) sv[c] = c <= lim ? sv[c] : -INFINITY;
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&s_read);
-            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-#pragma unroll
-            for (int c = 0; c < PA_KEYS; ++c) mx[c & 3] = fmaxf(mx[c & 3], sv[c]);
-            const float top = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * LOG2E;
-            // a row's first keys set its reference; later a maximum RESCALE above moves it
-            const bool fresh = m_run == -INFINITY;
-            const bool move = !fresh && top > m_run + RESCALE;
-            const float corr = move ? ex2(m_run - top) : 1.f;
-            if (fresh || move) m_run = top;
-            const float ref = m_run == -INFINITY ? 0.f : m_run;  // a row that has seen no key: every weight 0
-            l_run *= corr;
-            float sum[4] = {0.f, 0.f, 0.f, 0.f};
+            // two halves of 64 keys, each with its own look at the reference; a half of which no row of the
+            // warp sees a key (another run's rows, keys past every row) has weight zero without any work
             bool done = true;
-#pragma unroll
+#pragma unroll 1
             for (int half = 0; half < 2; ++half) {
+                const int hl = lim - half * PA_HALF;  // columns 0 .. hl of this half
+                const bool need = __any_sync(FULL_MASK, hl >= 0) != 0;
                 uint32_t hi[PA_HALF / 2], lo[PA_HALF / 2];
+                float corr = 1.f;
+                bool move = false;
+                if (need) {
+                    float sv[PA_HALF];
+                    tmem_ld_issue<32>(base + TM_S + half * PA_HALF, *reinterpret_cast<float(*)[32]>(&sv[0]));
+                    tmem_ld_issue<32>(base + TM_S + half * PA_HALF + 32, *reinterpret_cast<float(*)[32]>(&sv[32]));
+                    tmem_ld_wait();
+                    tmem_ld_done(*reinterpret_cast<float(*)[32]>(&sv[0]));
+                    tmem_ld_done(*reinterpret_cast<float(*)[32]>(&sv[32]));
+                    if (half) {
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&s_read);
+                    }
+                    if (!__all_sync(FULL_MASK, hl >= PA_HALF - 1)) {
 #pragma unroll
-                for (int e = 0; e < PA_HALF / 2; ++e) {
-                    const float p0 = ex2(fmaf(sv[half * PA_HALF + 2 * e], LOG2E, -ref));
-                    const float p1 = ex2(fmaf(sv[half * PA_HALF + 2 * e + 1], LOG2E, -ref));
-                    sum[(2 * e) & 3] += p0;
-                    sum[(2 * e + 1) & 3] += p1;
-                    split_pair(p0, p1, hi[e], lo[e]);
+                        for (int c = 0; c < PA_HALF; ++c) sv[c] = c <= hl ? sv[c] : -INFINITY;
+                    }
+                    float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                    for (int c = 0; c < PA_HALF; ++c) mx[c & 3] = fmaxf(mx[c & 3], sv[c]);
+                    const float top = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * LOG2E;
+                    // a row's first keys set its reference; later a maximum RESCALE above moves it
+                    const bool fresh = m_run == -INFINITY;
+                    move = !fresh && top > m_run + RESCALE;
+                    if (move) corr = ex2(m_run - top);
+                    if (fresh || move) m_run = top;
+                    const float ref = m_run == -INFINITY ? 0.f : m_run;  // a row that has seen no key: every weight 0
+                    float sum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int e = 0; e < PA_HALF / 2; ++e) {
+                        const float p0 = ex2(fmaf(sv[2 * e], LOG2E, -ref));
+                        const float p1 = ex2(fmaf(sv[2 * e + 1], LOG2E, -ref));
+                        sum[(2 * e) & 3] += p0;
+                        sum[(2 * e + 1) & 3] += p1;
+                        split_pair(p0, p1, hi[e], lo[e]);
+                    }
+                    l_run = fmaf(l_run, corr, (sum[0] + sum[1]) + (sum[2] + sum[3]));
+                } else {
+                    if (half) {
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(&s_read);
+                    }
+#pragma unroll
+                    for (int e = 0; e < PA_HALF / 2; ++e) hi[e] = lo[e] = 0u;
                 }
                 // the previous half's weights have been read (and O is complete up to them)
                 if (half || items > 0)
@@ -389,7 +406,7 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
                                                                         (uint32_t)(half ? items : items - 1) & 1, a.err));
                 if (!done) break;
                 tc_fence_after();
-                if (half == 0 && __any_sync(FULL_MASK, move)) {
+                if (__any_sync(FULL_MASK, move)) {
 #pragma unroll
                     for (int c0 = 0; c0 < HEAD_DIM; c0 += 16) {
                         float v[16];
@@ -415,7 +432,6 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
                 fine = false;
                 break;
             }
-            l_run += (sum[0] + sum[1]) + (sum[2] + sum[3]);
         }
     }
     // ---- this row's unnormalised output (registers) ----
