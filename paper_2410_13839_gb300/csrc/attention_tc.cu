@@ -145,6 +145,17 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
     pdl_wait();
     trace_wait(a.trace);
 
+    // Q of this head, 16 lanes per row: on its way while the rows' runs are found
+    constexpr int PER = 32 * (HEAD_DIM / 4) / 32;
+    float4 x[PER];
+    if (tid < PA_ROWS) {
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {  // (rows past the pass read its last one)
+            const int r = min(row0 + warp * 32 + u * 2 + (lane >> 4), a.rows - 1);
+            x[u] = *reinterpret_cast<const float4*>(a.q + (size_t)r * a.ldq + h * HEAD_DIM + (lane & 15) * 4);
+        }
+    }
+
     // ---- the tile's rows and their runs ----
     int my_seq = -1, my_pos = -1;
     if (tid < PA_ROWS) {
@@ -158,8 +169,9 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
     }
     __syncthreads();
     bool head = false;
-    unsigned heads = 0;
+    unsigned heads = 0, live = 0;  // the warp's rows that start a run, and those of a sequence
     if (tid < PA_ROWS) {
+        live = __ballot_sync(FULL_MASK, my_seq >= 0);
         head = my_seq >= 0 && (tid == 0 || s_seq[tid - 1] != my_seq);
         heads = __ballot_sync(FULL_MASK, head);
         if (lane == 0) s_heads[warp] = __popc(heads);
@@ -311,20 +323,11 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
         __syncwarp();
     } else {  // ---- one row per thread: Q, then softmax ----
         {
-            // Q of this head: rows pre-scaled by 1/sqrt(64), bf16 hi | lo, swizzled; 16 lanes per row, every
-            // load issued before any is used
-            constexpr int PER = PA_ROWS * (HEAD_DIM / 4) / PA_ROWS;
-            float4 x[PER];
+            // Q: rows pre-scaled by 1/sqrt(64), zero without a sequence, bf16 hi | lo, swizzled
 #pragma unroll
             for (int u = 0; u < PER; ++u) {
-                const int q = (tid >> 4) + u * (PA_ROWS / 16), c4 = tid & 15;
-                x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (s_seq[q] >= 0)
-                    x[u] = *reinterpret_cast<const float4*>(a.q + (size_t)(row0 + q) * a.ldq + h * HEAD_DIM + c4 * 4);
-            }
-#pragma unroll
-            for (int u = 0; u < PER; ++u) {
-                const int q = (tid >> 4) + u * (PA_ROWS / 16), c4 = tid & 15;
+                const int q = warp * 32 + u * 2 + (lane >> 4), c4 = lane & 15;
+                if (!(live >> (q & 31) & 1)) x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
                 uint2 hi, lo;
                 split_pair(x[u].x * 0.125f, x[u].y * 0.125f, hi.x, lo.x);
                 split_pair(x[u].z * 0.125f, x[u].w * 0.125f, hi.y, lo.y);
@@ -466,21 +469,42 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
             ost[tid * 16 + (c ^ (tid & 15))] =
                 make_float4(v[4 * c] * scale, v[4 * c + 1] * scale, v[4 * c + 2] * scale, v[4 * c + 3] * scale);
     };
-    auto write_rows = [&]() {  // every warp writes the rows its own threads staged
+    auto write_rows = [&]() {  // every warp writes the rows its own threads staged, 8 lanes and dims each
         __syncwarp();
+        float4 y[16];
 #pragma unroll
-        for (int u = 0; u < 16; ++u) {
-            const int q = warp * 32 + u * 2 + (lane >> 4), c4 = lane & 15, rq = row0 + q;
-            if (rq >= a.rows) continue;
-            const bool on = s_seq[q] >= 0;
-            const float4 y = on ? ost[q * 16 + (c4 ^ (q & 15))] : make_float4(0.f, 0.f, 0.f, 0.f);
-            if (a.out && on) *reinterpret_cast<float4*>(a.out + (size_t)rq * a.ldo + h * HEAD_DIM + c4 * 4) = y;
-            if (a.out_hi) {
-                uint2 hi, lo;
-                split_pair(y.x, y.y, hi.x, lo.x);
-                split_pair(y.z, y.w, hi.y, lo.y);
-                *reinterpret_cast<uint2*>(a.out_hi + (size_t)rq * a.ldb + h * HEAD_DIM + c4 * 4) = hi;
-                *reinterpret_cast<uint2*>(a.out_lo + (size_t)rq * a.ldb + h * HEAD_DIM + c4 * 4) = lo;
+        for (int u = 0; u < 8; ++u) {
+            const int q = warp * 32 + u * 4 + (lane >> 3);
+            const bool on = live >> (q & 31) & 1;
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int c4 = 2 * (lane & 7) + e;
+                y[2 * u + e] = ost[q * 16 + (c4 ^ (q & 15))];
+                if (!on) y[2 * u + e] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+        const int c = h * HEAD_DIM + (lane & 7) * 8, q0 = warp * 32 + (lane >> 3);
+        if (a.out) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u)
+                if (live >> ((q0 + u * 4) & 31) & 1) {
+                    float4* o = reinterpret_cast<float4*>(a.out + (size_t)(row0 + q0 + u * 4) * a.ldo + c);
+                    o[0] = y[2 * u];
+                    o[1] = y[2 * u + 1];
+                }
+        }
+        if (a.out_hi) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (row0 + q0 + u * 4 >= a.rows) continue;
+                uint4 hi, lo;
+                split_pair(y[2 * u].x, y[2 * u].y, hi.x, lo.x);
+                split_pair(y[2 * u].z, y[2 * u].w, hi.y, lo.y);
+                split_pair(y[2 * u + 1].x, y[2 * u + 1].y, hi.z, lo.z);
+                split_pair(y[2 * u + 1].z, y[2 * u + 1].w, hi.w, lo.w);
+                const size_t at = (size_t)(row0 + q0 + u * 4) * a.ldb + c;
+                *reinterpret_cast<uint4*>(a.out_hi + at) = hi;
+                *reinterpret_cast<uint4*>(a.out_lo + at) = lo;
             }
         }
     };
