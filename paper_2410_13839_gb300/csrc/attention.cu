@@ -237,12 +237,13 @@ __global__ void __launch_bounds__(ATT_THREADS, 4)
     __syncthreads();
 
     // ---- copies: warp 0 walks the stream ahead of the tiles ----
-    int pg = 0, pb = 0, pnb = 0, pseq = -1, ppages = 0, pold = 0, staged = 0;  // group, its next batch, ...
+    int pg = 0, pb = 0, pnb = 0, pseq = -1, pkeys = 0, ppages = 0, pold = 0, staged = 0;  // group, its next batch, ...
     auto next_group = [&]() {  // the next group with keys, from pg on
         for (;; ++pg) {
             const Group x = group_of(pg);
             pnb = batches(x);
             pseq = x.seq;
+            pkeys = x.keys;
             ppages = (x.keys + P - 1) / P;
             pold = a.plan == PLAN_DEVICE ? (x.keys - x.rows) / P : ppages;  // pages of earlier steps' keys only
             if (pnb > 0) return;
@@ -253,10 +254,12 @@ __global__ void __launch_bounds__(ATT_THREADS, 4)
         const bool mine = lane < ppb && p < ppages;
         const int phys = mine ? a.block_table[(size_t)pseq * a.bt_stride + p] : -1;
         if (mine && phys < 0 && a.err) atomicOr(a.err, ERR_BOUNDS);  // unreserved page: report, never read
-        const unsigned have = __ballot_sync(FULL_MASK, phys >= 0);
-        const uint32_t blk = (uint32_t)P * HEAD_DIM * 2;
+        // of the group's last page only the 16-key tiles that hold a key (tensor copies: whole pages)
+        const int rows = PLAIN ? P : min(P, (pkeys - p * P + 15) & ~15);
+        const uint32_t blk = phys >= 0 ? (uint32_t)rows * HEAD_DIM * 2 : 0u;
+        const uint32_t bytes = 2 * __reduce_add_sync(FULL_MASK, blk);
         fence_proxy_async();  // the slot was last read by this CTA's threads
-        if (lane == 0) mbar_arrive_expect_tx(&bar[slot], 2 * blk * __popc(have));
+        if (lane == 0) mbar_arrive_expect_tx(&bar[slot], bytes);
         __syncwarp();
         if (phys >= 0) {
             __nv_bfloat16* kd = Ks + ((size_t)slot * KB + lane * P) * HEAD_DIM;
@@ -379,7 +382,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 4)
         const int cend = min(gnb, cb + n - i);
         for (; cb < cend; ++cb, ++i) {
             const int slot = i % ATT_STAGES, key0 = cb * KB;
-            const int nk = min(ppb, gpages - cb * ppb) * P;
+            const int nk = min(min(ppb, gpages - cb * ppb) * P, (x.keys - key0 + 15) & ~15);
             ok = mbar_wait(&bar[slot], (uint32_t)(i / ATT_STAGES) & 1, a.err) && ok;
             const uint32_t kb = smem_addr(Ks + (size_t)slot * KB * HEAD_DIM);
             const uint32_t vb = smem_addr(Vs + (size_t)slot * KB * HEAD_DIM);
