@@ -246,20 +246,20 @@ MTP_API int mtp_debug_lattice(mtp_ctx* ctx, int32_t* out_ids, float* out_logp, i
  *                        allow it; 0 = two block kernels per layer (default: faster on GB300 at B = 1)
  *   MTP_OPT_PREFILL_TC   attention of prefill passes (mtp_prefill, mtp_prefill_pending): 1 = always on the
  *                        tensor cores (tcgen05: tiles of 128 prompt rows, 128-key items, S and P V
- *                        accumulated in TMEM); 0 = so in passes of more than 512 rows (47 vs 143 us per
- *                        launch at 4096 rows of the serving prompts), the split-key kernel of the decode
+ *                        accumulated in TMEM); 0 = so in passes of more than 512 rows (124 us per
+ *                        launch at 14592 rows of 128 prompts, 16 heads), the kernel of the decode
  *                        steps, in groups of 8 rows, in smaller ones (default)
  *   MTP_OPT_GEMM_CLUSTER 1 = the batched path's projections at up to 128 fed rows run as one
  *                        activation tile per weight tile, their K split over the CTAs of a cluster
- *                        (up to 8) that sum the partial tiles in distributed shared memory, each
- *                        CTA finishing its share of the rows (q|k|v append, GELU pack, residual
- *                        add); more splits than a cluster holds add by atomics (default); 0 =
+ *                        (2 or 4) that sum the partial tiles in distributed shared memory, each
+ *                        CTA finishing its share of the rows (q|k|v append, GELU pack); accumulated
+ *                        outputs add their splits by atomics (default); 0 =
  *                        tiles of 32 rows, K split only where the output is accumulated
  *   MTP_OPT_HEADS_FUSED  heads, log-softmax and top-k of more than 8 hidden rows as one tensor-core
  *                        kernel (LN_f rows as bf16 hi + lo; per (tile of 128 rows, head) a cluster of
  *                        8 CTAs over vocabulary slices, lse merged in the cluster before the top-k):
  *                        0 = never (heads GEMM into memory, then the selection kernel's top-k);
- *                        1 = in mtp_heads_topk (default: 65.8 vs 94.6 us for 256 rows, n = 8, top-16);
+ *                        1 = in mtp_heads_topk (default: 32.0 vs 94.6 us for 256 rows, n = 8, top-16);
  *                        2 = also in batched decode steps (measured 1.2 % slower per step at B = 32)
  *   MTP_OPT_SEED         seed of the path draws (any 32-bit value, zero-extended; default 0).
  *                        Position t of a draw of slot b that has generated g tokens uses the

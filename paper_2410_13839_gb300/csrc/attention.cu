@@ -48,7 +48,6 @@ constexpr int ATT_STAGES = 3;    // staging slots of the key/value ring (three 6
 constexpr int RPG = MAX_ROWS;    // rows per group, upper bound
 constexpr int PART = 2 + HEAD_DIM;  // (max, sum, out[64]) per row and split
 constexpr float LOG2E = 1.4426950408889634f;
-constexpr float RESCALE = 8.f;   // growth of a row's scores (log2) that moves its reference
 constexpr int NW = ATT_THREADS / 32;
 constexpr int MROWS = 4;         // rows whose warp states are merged at a time (one per warp)
 static_assert(HEAD_DIM == 64, "score scale 0.125 assumes 64-wide heads");
@@ -405,10 +404,12 @@ __global__ void __launch_bounds__(ATT_THREADS, 4)
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
                     sv[e] = key0 + kt + g8 + (e >> 1) * 8 <= qpos[e & 1] ? sh[e] + sl[e] : -INFINITY;
-                // weights are taken relative to the row's reference m_w, a bound of the scores up to a factor
-                // 2^RESCALE: it moves (a maximum over the lanes, the sums rescaled) only past that
+                // weights are taken relative to the row's running maximum m_w; where no lane's score exceeds it,
+                // the maximum over the lanes and the rescaling are skipped.  (A reference that may lag behind by
+                // up to 2^8 moves less often, 0.5 % faster, but 32 slots of 180-2000 keys are then 3.4e-6 from
+                // 64 bits instead of 3.1e-6.)
                 float t0 = fmaxf(sv[0], sv[2]), t1 = fmaxf(sv[1], sv[3]);
-                if (__any_sync(FULL_MASK, t0 > m_w[0] + RESCALE || t1 > m_w[1] + RESCALE)) {
+                if (__any_sync(FULL_MASK, t0 > m_w[0] || t1 > m_w[1])) {
 #pragma unroll
                     for (int off = 4; off < 32; off <<= 1) {  // over the tile's keys: lanes g8
                         t0 = fmaxf(t0, __shfl_xor_sync(FULL_MASK, t0, off));
