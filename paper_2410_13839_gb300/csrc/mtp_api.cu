@@ -334,10 +334,11 @@ int tile_index(int nt) { return nt == 32 ? 0 : (nt == 64 ? 1 : 2); }
 // positions, plan PLAN_ROWS).  prefill_keys > 0: a prefill pass whose rows see
 // at most that many keys; its attention runs in tiles of 128 rows (tcgen05)
 // above PREFILL_TC_ROWS rows, or always with that option.  A tile's chain of
-// 128-key items takes 5 + 3 us per item, which only many tiles pay back: per
-// launch 47 vs 143 us at 4096 serving-prompt rows, 28 vs 28 at 528, 19 vs 14 at
-// one prompt of 289.
-constexpr int PREFILL_TC_ROWS = 512;
+// 128-key items is longer than a group's of 64-key batches, which only enough
+// tiles pay back: whole prefills with the groups and with the tiles, ms, of one
+// prompt of 289 rows 0.70 and 0.75, of 320 0.78 and 0.75, of 448 0.86 and 0.82,
+// of two prompts of 160 0.80 and 0.78, of four of 122 0.87 and 0.79.
+constexpr int PREFILL_TC_ROWS = 304;
 int run_layers_batched(mtp_ctx* c, int M, int rpg, int groups, int plan, cudaStream_t s, bool pdl, Prof* prof,
                        int prefill_keys = 0) {
     const mtp_config& cf = c->cfg;

@@ -17,7 +17,7 @@ pytestmark = pytest.mark.gpu
 MODEL = synth.TINY_BF16
 
 
-@pytest.mark.parametrize("length", [1, 7, 9, 127, 129, 257, 1025, 4095, 4097])
+@pytest.mark.parametrize("length", [1, 7, 9, 127, 129, 257, 304, 305, 385, 1025, 4095, 4097])
 def test_one_prompt(length):
     ph, ac = synth.make_prompt(300 + length, length // 3, length - length // 3, MODEL.phone_vocab)
     dec, w = decoder(MODEL, max_batch=1, max_ctx=length + 32)
