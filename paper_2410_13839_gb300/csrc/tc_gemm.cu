@@ -19,11 +19,11 @@
 // and of both activation parts into a 4-stage shared-memory ring with TMA
 // (128-byte swizzled tiles), a second elected thread issues tcgen05.mma
 // into a TMEM accumulator (128 lanes x 2 NT fp32 columns) and releases each
-// stage with tcgen05.commit.  Eight warps read the accumulator back with
-// tcgen05.ld and finish it from the registers (tc_epilogue.cuh): warps w and
-// w + 4 share TMEM lanes 32 (w % 4) .., i.e. weight rows, and take half of the
-// columns each.  Staging the tile in shared memory first, to write float4
-// pieces of rows, took 0.65 us more and left the stores as long (512 rows,
+// stage with tcgen05.commit.  8 or 16 warps read the accumulator back with
+// tcgen05.ld and finish it from the registers (tc_epilogue.cuh): warps w, w + 4,
+// .. share TMEM lanes 32 (w % 4) .., i.e. weight rows, and divide the columns.
+// Staging the tile in shared memory first, to write float4 pieces of rows,
+// took 0.65 us more and left the stores as long (512 rows,
 // d = 1024: W2 12.0 -> 10.2 us); where K splits meet in a cluster it is the
 // layout of the exchange (q|k|v and W1 of 128 rows: 8.0 -> 7.3 us).  Grid:
 // (N_w / 128 weight tiles, K splits, activation tiles).  The weight copies of
@@ -50,9 +50,13 @@ constexpr int TC_K = 64;       // k per stage: one 128-byte swizzle row of bf16
 // ring stages per activation tile size: about 190 KB of copies in flight per CTA
 __host__ __device__ constexpr int tc_stages(int nt) { return nt <= 32 ? 8 : (nt <= 64 ? 6 : 4); }
 constexpr int TC_MAX_STAGES = 8;
-// 8 warps: two elected lanes run the ring; the epilogue is instruction-latency bound (one warp per
-// scheduler hid nothing)
-constexpr int TC_THREADS = 256;
+// 8 or 16 warps: two elected lanes run the ring; the epilogue is instruction-latency bound (one warp per
+// scheduler hid nothing).  16 where a thread of 8 would finish 64 rows with arithmetic or read-modify-write
+// (d = 1024, 512 rows: q|k|v 10.1 -> 9.1 us, W1 10.2 -> 9.3, W_o 4.9 -> 4.5, W2 8.4 -> 7.9); plain stores
+// gain nothing (W1 11.3 vs 11.7 us), nor do the halved tiles of a cluster.
+__host__ __device__ constexpr int tc_threads(int nt, int epi, bool cluster) {
+    return nt == 128 && epi != TC_STORE && !cluster ? 512 : 256;
+}
 constexpr uint32_t TC_W_BYTES = TC_M * TC_K * 2;
 
 // ---- PTX wrappers (tcgen05, TMA) ----
@@ -84,13 +88,13 @@ __host__ __device__ constexpr uint32_t tc_idesc(int n) {
 }
 
 template <int NT, int EPI, bool CLUSTER>
-__global__ void __launch_bounds__(TC_THREADS, 1)
+__global__ void __launch_bounds__(tc_threads(NT, EPI, CLUSTER), 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tw, const __grid_constant__ CUtensorMap tah,
                    const __grid_constant__ CUtensorMap tal, const TcGemmArgs a) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     constexpr uint32_t A_BYTES = NT * TC_K * 2, STAGE = TC_W_BYTES + 2 * A_BYTES;
     constexpr uint32_t TMEM_COLS = 2 * NT;  // the products with the hi parts, then with the lo parts
-    constexpr int TC_STAGES = tc_stages(NT);
+    constexpr int TC_STAGES = tc_stages(NT), THREADS = tc_threads(NT, EPI, CLUSTER), PARTS = THREADS / 128;
     __shared__ uint64_t full[TC_MAX_STAGES], empty[TC_MAX_STAGES], done, red_bar;
     __shared__ uint32_t tmem_base;
     __shared__ int s_ok;
@@ -186,7 +190,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         tc_commit(&done);  // every MMA issued above has completed
     } else if (warp >= 2 && (EPI == TC_QKV || EPI == TC_GELU_PACK)) {
         // per-row facts of the epilogue, gathered by the two idle warps while the ring runs
-        for (int j = tid - 64; j < NT; j += TC_THREADS - 64) {
+        for (int j = tid - 64; j < NT; j += THREADS - 64) {
             const int n = arow + j;
             const int seq = n < a.m ? a.row_seq[n] : -1;
             long long base = -1;
@@ -213,7 +217,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
     tc_fence_after();
     trace_mark(a.trace, 0);  // accumulator complete
     const bool good = fin && s_ok;
-    const int quarter = warp & 3, half = warp >> 2;  // the TMEM lanes (weight rows) this warp may read
+    const int quarter = warp & 3, part = warp >> 2;  // the TMEM lanes (weight rows) this warp may read, its columns
     const int f = tile * TC_M + quarter * 32 + lane;
     const uint32_t acc = tmem + ((uint32_t)(quarter * 32) << 16);
     const int rows = min(NT, a.m - arow);  // activation rows of the tile
@@ -238,7 +242,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         float v[4][N], w[4][N];
         // unit u: rows r0(u) .. + N of share p(u)
         auto share = [&](int u) { return Sc == 4 ? u : u >> 1; };
-        auto first = [&](int u) { return half * (R / 2) + (Sc == 4 ? 0 : (u & 1) * N); };
+        auto first = [&](int u) { return part * (R / 2) + (Sc == 4 ? 0 : (u & 1) * N); };
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             tmem_ld_issue<N>(acc + (uint32_t)(share(u) * R + first(u)), v[u]);
@@ -278,7 +282,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
         trace_mark(a.trace, 3);  // the peers' partial rows received
         if (good && got) {
             const float bias = a.bias ? __ldg(a.bias + f) : 0.f;
-            for (int r0 = half * (R / 2); r0 < (half + 1) * (R / 2); r0 += N) {
+            for (int r0 = part * (R / 2); r0 < (part + 1) * (R / 2); r0 += N) {
                 float y[N];
 #pragma unroll
                 for (int e = 0; e < N; ++e) y[e] = 0.f;
@@ -301,10 +305,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1)
             trace_mark(a.trace, 5);  // thread 0's stores issued
         }
     } else if (good) {
-        constexpr int N = NT / 2 < 32 ? NT / 2 : 32;
+        constexpr int COLS = NT / PARTS, N = COLS < 32 ? COLS : 32;
         // the tile's first split adds the bias (heads: rows past n_valid have none)
         const float bias = a.bias && split == 0 && (!a.n_valid || f < a.n_valid) ? __ldg(a.bias + f) : 0.f;
-        for (int j0 = half * (NT / 2); j0 < (half + 1) * (NT / 2) && j0 < rows; j0 += N) {
+        for (int j0 = part * COLS; j0 < (part + 1) * COLS && j0 < rows; j0 += N) {
             float v[N], w[N];
             tmem_ld_issue<N>(acc + (uint32_t)j0, v);
             tmem_ld_issue<N>(acc + (uint32_t)(NT + j0), w);
@@ -350,13 +354,13 @@ size_t tc_smem() {
 }
 
 template <int NT, typename K>
-cudaError_t launch_kern(K kern, const TcGemm& g, cudaStream_t s, bool pdl) {
+cudaError_t launch_kern(K kern, int threads, const TcGemm& g, cudaStream_t s, bool pdl) {
     const size_t smem = tc_smem<NT>();
     cudaError_t e = ensure_kernel_smem(reinterpret_cast<const void*>(kern), smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(g.n_w / TC_M, g.splits, (g.args.m + NT - 1) / NT);
-    cfg.blockDim = dim3(TC_THREADS);
+    cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
@@ -378,14 +382,14 @@ template <int NT>
 cudaError_t launch_nt(const TcGemm& g, cudaStream_t s, bool pdl) {
     const bool cluster = g.args.cluster_reduce > 1;
     switch (g.args.epilogue) {
-        case TC_STORE: return launch_kern<NT>(tc_gemm_kernel<NT, TC_STORE, false>, g, s, pdl);
-        case TC_ACCUM: return launch_kern<NT>(tc_gemm_kernel<NT, TC_ACCUM, false>, g, s, pdl);
+        case TC_STORE: return launch_kern<NT>(tc_gemm_kernel<NT, TC_STORE, false>, tc_threads(NT, TC_STORE, false), g, s, pdl);
+        case TC_ACCUM: return launch_kern<NT>(tc_gemm_kernel<NT, TC_ACCUM, false>, tc_threads(NT, TC_ACCUM, false), g, s, pdl);
         case TC_QKV:
-            if (cluster) return launch_kern<NT>(tc_gemm_kernel<NT, TC_QKV, true>, g, s, pdl);
-            return launch_kern<NT>(tc_gemm_kernel<NT, TC_QKV, false>, g, s, pdl);
+            if (cluster) return launch_kern<NT>(tc_gemm_kernel<NT, TC_QKV, true>, tc_threads(NT, TC_QKV, true), g, s, pdl);
+            return launch_kern<NT>(tc_gemm_kernel<NT, TC_QKV, false>, tc_threads(NT, TC_QKV, false), g, s, pdl);
         case TC_GELU_PACK:
-            if (cluster) return launch_kern<NT>(tc_gemm_kernel<NT, TC_GELU_PACK, true>, g, s, pdl);
-            return launch_kern<NT>(tc_gemm_kernel<NT, TC_GELU_PACK, false>, g, s, pdl);
+            if (cluster) return launch_kern<NT>(tc_gemm_kernel<NT, TC_GELU_PACK, true>, tc_threads(NT, TC_GELU_PACK, true), g, s, pdl);
+            return launch_kern<NT>(tc_gemm_kernel<NT, TC_GELU_PACK, false>, tc_threads(NT, TC_GELU_PACK, false), g, s, pdl);
         default: return cudaErrorInvalidValue;
     }
 }
