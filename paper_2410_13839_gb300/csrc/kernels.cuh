@@ -299,13 +299,10 @@ cudaError_t launch_save_last(const float* x, const int* row_seq, const int* row_
                              unsigned long long* trace, cudaStream_t s, bool pdl);
 
 // ------------------------------------------------------- batched path ----
-enum PackMode : int { PACK_LN = 0, PACK_COPY = 1, PACK_GELU = 2 };
-struct PackArgs {
-    int mode;                     // PackMode
+struct PackArgs {  // LayerNorm rows as bf16 hi + lo parts
     const float* x; int ldx;      // input rows [m][ldx], k columns used
     int x_bf16;                   // x holds bf16 rows (8-byte aligned; every-row variant, row_seq null)
-    float* zero_after;            // PACK_GELU: rows zeroed after reading (may be x), or null
-    const float* gamma; const float* beta; float eps;   // PACK_LN
+    const float* gamma; const float* beta; float eps;
     const int* row_seq;           // rows with row_seq < 0 are packed as zeros (null: every row is packed,
                                   // and zero_buf [zero_n] is zeroed first)
     __nv_bfloat16* hi; __nv_bfloat16* lo;  // [m][k] bf16 parts: hi + lo = the fp32 row

@@ -359,11 +359,11 @@ int run_layers_batched(mtp_ctx* c, int M, int rpg, int groups, int plan, cudaStr
         const Layer& L = c->layers[l];
         const mtp_ctx::LayerMaps& W = c->lmaps[l];
         const long long layer_off = (long long)l * 2 * H * P * HEAD_DIM;
-        auto pack = [&](int mode, const float* x, int k, const float* g, const float* bta, float* zero,
-                        __nv_bfloat16* hi, __nv_bfloat16* lo) -> int {
+        auto pack = [&](const float* x, int k, const float* g, const float* bta, __nv_bfloat16* hi,
+                        __nv_bfloat16* lo) -> int {
             PackArgs pa;
             std::memset(&pa, 0, sizeof(pa));
-            pa.mode = mode; pa.x = x; pa.ldx = k; pa.zero_after = zero; pa.gamma = g; pa.beta = bta;
+            pa.x = x; pa.ldx = k; pa.gamma = g; pa.beta = bta;
             pa.eps = cf.ln_eps; pa.row_seq = c->d_row_seq; pa.hi = hi; pa.lo = lo; pa.k = k; pa.m = M;
             pa.trace = tslot(c, MTP_K_PACK);
             LAUNCH(MTP_K_PACK, launch_pack_rows(pa, s, pdl));
@@ -402,7 +402,7 @@ int run_layers_batched(mtp_ctx* c, int M, int rpg, int groups, int plan, cudaStr
             return MTP_OK;
         };
         // LN1 -> q|k|v: queries out, keys and values appended to the cache
-        MTP_TRY(pack(PACK_LN, c->d_bx, d, L.ln1_g, L.ln1_b, nullptr, c->d_ahi, c->d_alo));
+        MTP_TRY(pack(c->d_bx, d, L.ln1_g, L.ln1_b, c->d_ahi, c->d_alo));
         MTP_TRY(gemm(W.wqkv, 3 * d, d, false, TC_QKV, c->d_bq, d, L.bqkv, 0));
         // attention of every group's fed rows over its cached keys
         AttnArgs at;
@@ -436,7 +436,7 @@ int run_layers_batched(mtp_ctx* c, int M, int rpg, int groups, int plan, cudaStr
         // x += attention W_o^T + b_o (the per-head W_o blocks are the k-chunks)
         MTP_TRY(gemm(W.wo, d, d, false, TC_ACCUM, c->d_bx, d, L.bo, d));
         // x += GELU(LN2(x) W1^T + b1) W2^T + b2 (W1's epilogue writes the GELU rows as bf16 hi + lo)
-        MTP_TRY(pack(PACK_LN, c->d_bx, d, L.ln2_g, L.ln2_b, nullptr, c->d_ahi, c->d_alo));
+        MTP_TRY(pack(c->d_bx, d, L.ln2_g, L.ln2_b, c->d_ahi, c->d_alo));
         MTP_TRY(gemm(W.w1, F, d, false, TC_GELU_PACK, nullptr, F, L.b1, 0));
         MTP_TRY(gemm(W.w2, d, F, true, TC_ACCUM, c->d_bx, d, L.b2, 0));
     }
@@ -631,7 +631,7 @@ int launch_heads_batched(mtp_ctx* c, const void* x, bool x_bf16, int B, int n, f
     const int d = cf.d_model, V = cf.codec_vocab;
     PackArgs pa;
     std::memset(&pa, 0, sizeof(pa));
-    pa.mode = PACK_LN; pa.x = static_cast<const float*>(x); pa.x_bf16 = x_bf16; pa.ldx = d;
+    pa.x = static_cast<const float*>(x); pa.x_bf16 = x_bf16; pa.ldx = d;
     pa.gamma = c->lnf_g; pa.beta = c->lnf_b;
     pa.eps = cf.ln_eps; pa.row_seq = nullptr; pa.hi = c->d_ahi; pa.lo = c->d_alo; pa.k = d; pa.m = B;
     pa.zero_buf = logits; pa.zero_n = (long long)B * n * V;
@@ -671,7 +671,7 @@ int launch_heads_fused(mtp_ctx* c, const void* x, bool x_bf16, int B, int n, int
     const int d = cf.d_model, V = cf.codec_vocab;
     PackArgs pa;
     std::memset(&pa, 0, sizeof(pa));
-    pa.mode = PACK_LN; pa.x = static_cast<const float*>(x); pa.x_bf16 = x_bf16; pa.ldx = d;
+    pa.x = static_cast<const float*>(x); pa.x_bf16 = x_bf16; pa.ldx = d;
     pa.gamma = c->lnf_g; pa.beta = c->lnf_b;
     pa.eps = cf.ln_eps; pa.row_seq = nullptr; pa.hi = c->d_ahi; pa.lo = c->d_alo; pa.k = d; pa.m = B;
     pa.trace = tslot(c, MTP_K_PACK);
