@@ -9,10 +9,8 @@
 //
 //   D = (Z_hi + Z_lo) W_slice^T      tcgen05.mma, M = 128 rows (TMEM lanes),
 //                                    N = 128 or 144 vocabulary columns, K = d
-//                                    in 64-wide chunks through a 2-stage TMA
-//                                    ring (128-byte swizzled tiles); the rows of
-//                                    a whole tile are the same in the 8 CTAs, so
-//                                    each copies an eighth of them to all
+//                                    in 64-wide chunks through a TMA ring of two
+//                                    or four stages (128-byte swizzled tiles)
 //   phase 1   thread = (row, half of the columns), one pass: max, sum of exp,
 //             sum and sum of squares of the logits (logit = D + b, read back
 //             from TMEM), the two halves combined in shared memory; the 8
@@ -89,23 +87,6 @@ __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, i
         : "memory");
 }
 
-// The same box into every CTA of the cluster, at this offset, each completing on its own barrier.
-__device__ __forceinline__ void tma_load_2d_all(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1, {%2, "
-        "%3}], [%4], %5;" ::"r"(smem_addr(dst)),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(smem_addr(bar)), "h"((uint16_t)0xff)
-        : "memory");
-}
-// Arrive on `bar` in every CTA of the cluster once the MMAs issued so far are done.
-__device__ __forceinline__ void tc_commit_all(uint64_t* bar) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-            smem_addr(bar)),
-        "h"((uint16_t)0xff)
-        : "memory");
-}
-
 __device__ __forceinline__ int ld_dsmem_i32(uint32_t addr) {
     int v;
     asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
@@ -149,7 +130,6 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
     heads_tc_kernel(const __grid_constant__ CUtensorMap tw128, const __grid_constant__ CUtensorMap tw144,
                     const __grid_constant__ CUtensorMap tah, const __grid_constant__ CUtensorMap tal,
                     const HeadsTcArgs a) {
-    const bool all = a.a_rows == HT_M;  // whole tiles: each CTA copies its 16 rows of a stage to all eight
     extern __shared__ __align__(1024) unsigned char ht_raw[];
     __shared__ uint64_t full[HT_MAX_STAGES], empty[HT_MAX_STAGES], done;
     __shared__ uint32_t tmem_base;
@@ -180,7 +160,7 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
     if (tid == 32) {
         for (int s = 0; s < HT_MAX_STAGES; ++s) {
             mbar_init(&full[s], 1);
-            mbar_init(&empty[s], all ? HT_SLICES : 1);  // every CTA that a stage's copies go to has read it
+            mbar_init(&empty[s], 1);
         }
         mbar_init(&done, 1);
         fence_barrier_init();
@@ -189,10 +169,6 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
     for (int c = tid; c < HT_NMAX; c += HT_THREADS) s_bias[c] = c < cnt ? a.bias[wrow + c] : 0.f;
     tc_fence_before();
     __syncthreads();
-    if (all) {  // the peers' barriers are initialised before anything completes on them
-        cluster_arrive_release();
-        cluster_wait();
-    }
     tc_fence_after();
     const uint32_t tmem = tmem_base;
 
@@ -221,14 +197,8 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
                 mbar_arrive_expect_tx(&full[s], stage_bytes);
                 tma_load_2d(st + 2 * HT_A_BYTES, wide ? &tw144 : &tw128, c * HT_K, wrow, &full[s]);
             }
-            if (all) {
-                constexpr int R = HT_M / HT_SLICES;
-                tma_load_2d_all(st + j * R * HT_K * 2, &tah, c * HT_K, arow + j * R, &full[s]);
-                tma_load_2d_all(st + HT_A_BYTES + j * R * HT_K * 2, &tal, c * HT_K, arow + j * R, &full[s]);
-            } else {
-                tma_load_2d(st, &tah, c * HT_K, arow, &full[s]);
-                tma_load_2d(st + HT_A_BYTES, &tal, c * HT_K, arow, &full[s]);
-            }
+            tma_load_2d(st, &tah, c * HT_K, arow, &full[s]);
+            tma_load_2d(st + HT_A_BYTES, &tal, c * HT_K, arow, &full[s]);
         }
     } else if (tid == 32) {  // MMA issuer
         const uint32_t idesc = f16_idesc(HT_M, N, false);
@@ -244,10 +214,7 @@ __global__ void __cluster_dims__(HT_SLICES, 1, 1) __launch_bounds__(HT_THREADS, 
                 tc_mma(tmem, sw128_desc(hb + kk * 32), dw, idesc, (c | kk) != 0);
                 tc_mma(tmem, sw128_desc(lb + kk * 32), dw, idesc, 1u);
             }
-            if (all)
-                tc_commit_all(&empty[s]);
-            else
-                tc_commit(&empty[s]);
+            tc_commit(&empty[s]);
         }
         if (c < chunks) s_ok = 0;
         tc_commit(&done);

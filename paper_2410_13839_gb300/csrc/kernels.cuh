@@ -380,7 +380,7 @@ struct HeadsTcArgs {
 };
 struct HeadsTc {
     CUtensorMap w128, w144;       // head weight rows [n_max * V][d]: boxes of 64 x 128 and 64 x 144 rows
-    CUtensorMap a_hi, a_lo;       // LN_f rows: boxes of 64 x a_rows rows (a_rows = 128: of 64 x 16, copied to a cluster)
+    CUtensorMap a_hi, a_lo;       // LN_f rows: boxes of 64 x a_rows rows
     HeadsTcArgs args;
 };
 bool heads_tc_supported(int V, int k);

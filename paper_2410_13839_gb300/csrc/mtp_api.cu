@@ -148,7 +148,6 @@ struct mtp_ctx {
     CUtensorMap heads_map144;  // the same rows in boxes of 144 (the fused heads' last vocabulary slice)
     bool heads_tc_ok = false;  // the fused heads kernel serves this model (tensor maps, vocabulary size)
     CUtensorMap amap_hi[3], amap_lo[3], umap_hi[3], umap_lo[3];  // activation tiles of 32, 64, 128 rows
-    CUtensorMap amap16_hi, amap16_lo;  // a CTA's share of a 128-row tile of the fused heads
     float* d_pe = nullptr;
     // KV cache
     uint16_t* d_kv = nullptr;
@@ -592,8 +591,6 @@ int setup_batched(mtp_ctx* c) {
         bad |= tc_encode_2d(&c->umap_hi[t], c->d_uhi, (uint64_t)F, M, (uint32_t)nts[t], false);
         bad |= tc_encode_2d(&c->umap_lo[t], c->d_ulo, (uint64_t)F, M, (uint32_t)nts[t], false);
     }
-    bad |= tc_encode_2d(&c->amap16_hi, c->d_ahi, (uint64_t)d, M, 16, false);
-    bad |= tc_encode_2d(&c->amap16_lo, c->d_alo, (uint64_t)d, M, 16, false);
     bad |= tc_encode_2d(&c->heads_map, c->w_heads, (uint64_t)d, (uint64_t)cf.n_heads_max * cf.codec_vocab, 128,
                         false);
     c->heads_tc_ok = tc_encode_2d(&c->heads_map144, c->w_heads, (uint64_t)d,
@@ -680,8 +677,7 @@ int launch_heads_fused(mtp_ctx* c, const void* x, bool x_bf16, int B, int n, int
     std::memset(&g, 0, sizeof(g));
     g.w128 = c->heads_map; g.w144 = c->heads_map144;
     const int ar = tc_tile_rows(B);  // 32, 64 or 128 activation rows per stage
-    g.a_hi = ar == 128 ? c->amap16_hi : c->amap_hi[tile_index(ar)];
-    g.a_lo = ar == 128 ? c->amap16_lo : c->amap_lo[tile_index(ar)];
+    g.a_hi = c->amap_hi[tile_index(ar)]; g.a_lo = c->amap_lo[tile_index(ar)];
     HeadsTcArgs& ha = g.args;
     ha.bias = c->b_heads; ha.m = B; ha.n = n; ha.V = V; ha.k = k; ha.k_chunks = d / 64; ha.a_rows = ar;
     ha.out_ids = ids; ha.out_logp = logp; ha.out_lse = lse; ha.out_logits = logits; ha.ldl = n * V;

@@ -713,7 +713,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1) step_ke
     // cluster exchanges (transaction barriers: one local arrival + the bytes the peers push):
     // q|k|v rows, attention partials, FFN partial outputs
     __shared__ uint64_t xq_bar, xa_bar, xf_bar;
-    __shared__ uint64_t xr_bar;  // the phase's input rows, multicast into every CTA of the cluster
+    __shared__ uint64_t xr_bar;  // the phase's input rows
     __shared__ int s_seq[MAX_ROWS], s_pos[MAX_ROWS], s_tok[MAX_ROWS];
     __shared__ int s_gseq[MAX_ROWS], s_gold[MAX_ROWS], s_gnew[MAX_ROWS];
     __shared__ float ln_part[2 * NWARPS][MT];
@@ -744,7 +744,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1) step_ke
     const uint32_t xa_bytes = (uint32_t)CL * MT * PARTW * 4;
     const uint32_t xf_bytes = (uint32_t)f_senders * MT * orows * 4;
     const uint32_t xr_bytes = (uint32_t)MT * d * 4;
-    const int xr_total = (att ? a.L - 1 : 0) + (fcl ? a.L : 0);  // multicast row copies this CTA receives
+    const int xr_total = (att ? a.L - 1 : 0) + (fcl ? a.L : 0);  // row copies of this CTA
 
     if (tid == 0) {
         for (int s = 0; s < a.ring_stages; ++s) {
@@ -872,19 +872,15 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1) step_ke
         consumer_sync();
         trace_mark(a.trace, 0);
 
-        // The rows a phase starts from ([MT][d] fp32) come from global memory once per cluster:
-        // rank 0 copies them with one multicast bulk copy into the x area of all four CTAs (a
-        // quarter of the L2 requests of every CTA loading them), each waiting on its xr_bar.
+        // The rows a phase starts from ([MT][d] fp32) come from global memory with one bulk copy per CTA
+        // into its x area, completing on xr_bar.
         int xr_left = xr_total;
         auto issue_rows = [&](const float* src) {
-            if (rank == 0 && tid == 0) {
-                // the rows were written by other CTAs (generic proxy) and are read by the copy engine
-                asm volatile("fence.proxy.async.global;" ::: "memory");
-                asm volatile(
-                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster "
-                    "[%0], [%1], %2, [%3], %4;" ::"r"(smem_addr(xs)),
-                    "l"(src), "r"(xr_bytes), "r"(smem_addr(&xr_bar)), "h"((uint16_t)((1u << CL) - 1))
-                    : "memory");
+            if (tid == 0) {
+                // the rows were written by other CTAs and the x area last used by this one's threads
+                // (generic proxy); both are now the copy engine's
+                asm volatile("fence.proxy.async;" ::: "memory");
+                bulk_copy_g2s(xs, src, xr_bytes, &xr_bar);
             }
         };
         auto wait_rows = [&]() -> bool {
@@ -920,7 +916,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1) step_ke
             store_rows_split<MT>(xr, d, xb);
             consumer_sync();
         };
-        // rows [MT][d] fp32 in shared memory (the cluster's multicast copy) -> registers
+        // rows [MT][d] fp32 in shared memory -> registers
         auto load_resid = [&](RowRegs<MT>& xr, const float* x) {
 #pragma unroll
             for (int m = 0; m < MT; ++m) {
@@ -962,7 +958,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1) step_ke
                 } else {
                     ok = consumer_all(wait_rows());
                     if (!ok) break;
-                    load_resid(xr, xs);  // x(l), multicast into this CTA's x area
+                    load_resid(xr, xs);  // x(l)
                 }
 #pragma unroll
                 for (int k = 0; k < RES_N; ++k) {
@@ -1199,7 +1195,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(THREADS, 1) step_ke
             if (2 * l + 2 <= 2 * a.L - 1) zero_part(tbuf(2 * l + 2));
             if (l == a.L - 1) pdl_launch_dependents();
             if (fcl) {
-                ok = consumer_all(wait_rows());  // x_mid(l), multicast into this CTA's x area
+                ok = consumer_all(wait_rows());  // x_mid(l)
                 if (!ok) break;
                 float4 resv[RES_PER];  // residual cluster: x_mid + b2 of the columns this CTA reduces
 #pragma unroll
