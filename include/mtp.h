@@ -388,8 +388,11 @@ MTP_API int mtp_heads_topk(mtp_ctx* ctx, int batch, const void* hidden, int hidd
  *   row_pos    int32 [rows]: position; the row sees keys 0..row_pos
  *   block_table int32 [slots][bt_stride]: page of each page_size span
  *   out        float [rows][n_heads*64]
- *   workspace  device scratch of mtp_attention_workspace_bytes(...) bytes;
- *              its counters must be zero on the first call and are left zero.
+ *   workspace  device scratch of mtp_attention_workspace_bytes(...) bytes.  It starts with
+ *              merge counters, which must be zero on the first call and are left zero.
+ *              Their place is the same for all calls: one buffer zeroed once serves calls
+ *              of any sizes, of mtp_attention and mtp_attention_tc alike, one after the
+ *              other on a stream.
  *   max_keys   upper bound of (row_pos + 1) over all rows; sets the split count
  * Keys/values for positions 0..max row_pos of each group must be present.
  * Errors: MTP_ERR_INVALID, MTP_ERR_CUDA. */
@@ -417,7 +420,7 @@ MTP_API int mtp_attention(const mtp_attention_args* args, void* workspace, size_
  * cache layout: 16-byte chunk c of row t of a page at chunk position
  * c ^ (t mod 8).  Other arguments and layouts as mtp_attention; row_seq < 0 rows
  * are left untouched.  workspace: mtp_attention_tc_workspace_bytes(args) bytes,
- * counters zero on the first call and left zero.
+ * 16-byte aligned; counters as mtp_attention's.
  * Errors: MTP_ERR_INVALID (sizes, null pointers, workspace too small, q not
  * 16-byte aligned), MTP_ERR_CUDA. */
 MTP_API size_t mtp_attention_tc_workspace_bytes(const mtp_attention_args* args);

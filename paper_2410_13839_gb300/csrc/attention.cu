@@ -26,9 +26,9 @@
 // to fp32 accuracy, and its online-softmax state in registers; the warps'
 // states are merged in shared memory at the end of the group.  A group that
 // several CTAs share leaves partial results (max, sum, unnormalised output) in
-// the workspace, and the CTA that finishes last (an atomic counter per group
-// and head, reset by that CTA) merges them in stream order, so no second kernel
-// is needed.
+// the workspace, and the CTA that finishes last (an atomic counter of the
+// group's first CTA and head, reset by that CTA) merges them in stream order, so
+// no second kernel is needed.
 //
 // Under programmatic dependent launch the plan and the first batches that hold
 // only keys cached by earlier steps are fetched before griddepcontrol.wait.
@@ -332,6 +332,8 @@ __global__ void __launch_bounds__(ATT_THREADS, 4)
     // block and queries c2, c2 + 1 in O^T.
     const int g8 = lane >> 2, c2 = (lane & 3) * 2;
     // partials: a CTA shares at most its first group (slot 0) and its last (slot 1: begun here)
+    // (a CTA is the first of one shared group at most: its counter is that group's)
+    auto count_of = [&](int c_first) { return a.ws_count + (size_t)h * J + c_first; };
     auto part_of = [&](int cta, int c_first) {
         return a.ws_part + (((size_t)(h * J + cta) * 2 + (cta == c_first ? 1 : 0)) * RPG) * PART;
     };
@@ -526,7 +528,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 4)
     trace_mark(a.trace, 2);  // partials written
     if (tid < 2) {
         const int* sh = s_share[tid];
-        s_last[tid] = ok && sh[2] > 0 ? atomicAdd(a.ws_count + (size_t)sh[0] * H + h, 1) == sh[2] - 1 : 0;
+        s_last[tid] = ok && sh[2] > 0 ? atomicAdd(count_of(sh[1]), 1) == sh[2] - 1 : 0;
     }
     __syncthreads();
 #pragma unroll 1
@@ -569,7 +571,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 4)
             }
             put(sg, row_j, y0 / L, y1 / L);
         }
-        if (tid == 0) a.ws_count[(size_t)sg * H + h] = 0;
+        if (tid == 0) *count_of(c_first) = 0;
     }
     if (!ok && warp == 0) {  // error word set; let copies in flight land before leaving
         for (int i = max(0, staged - ATT_STAGES); i < staged; ++i)

@@ -79,7 +79,7 @@ struct AttnArgs {
     float* out; int ldo;                       // fp32 output rows, or null
     __nv_bfloat16* out_hi; __nv_bfloat16* out_lo; int ldb;  // or null: output rows as bf16 hi + lo (the
                                                // W_o GEMM's operand; rows of no sequence written as zeros)
-    float* ws_part; int* ws_count;             // split partials and per-(group, head) counters
+    float* ws_part; int* ws_count;             // split partials and merge counters (attn_counters), zero between launches
     int rows_per_group, n_heads, page_size;
     int groups, ctas;                          // attn_kernel: groups of rows, CTAs per head that share them out
     int whole;                                 // attn_kernel: or a CTA per group and head (no partials)
@@ -96,6 +96,9 @@ constexpr int ATTN_CTAS_PER_SM = 4;  // attn_kernel: 128 threads x at most 128 r
 int attn_ctas_for(int groups, int n_heads, int page_size, int max_keys, int num_sms);
 bool attn_whole_groups(int groups, int n_heads, int page_size, int max_keys, int num_sms);  // AttnArgs::whole
 size_t attn_workspace_floats(int n_heads, int ctas);
+// merge counters of any launch of either attention kernel: attn_kernel has one per CTA of a wave,
+// attention_tc one per (tile, head) where it splits keys, which needs fewer of them than SMs
+inline size_t attn_counters(int num_sms) { return (size_t)ATTN_CTAS_PER_SM * num_sms; }
 size_t attn_smem_bytes(int page_size);
 cudaError_t launch_attention(const AttnArgs& a, cudaStream_t s, bool pdl);   // the cache's swizzled pages
 cudaError_t launch_attention_plain(const AttnArgs& a, cudaStream_t s);       // plain pages, PLAN_ROWS
@@ -395,19 +398,19 @@ cudaError_t ensure_kernel_smem(const void* kernel, size_t bytes, bool max_shared
 
 // The stand-alone attention operator (mtp_attention*): its arguments checked
 // and its workspace laid out once, for every entry point that runs it.  The
-// workspace holds the split partials (part_bytes, a multiple of 256) and then
-// the per-(group, head) merge counters (count_bytes), which must be zero when
-// a launch starts and are left zero by it.
+// workspace starts with the merge counters (count_bytes, a multiple of 256),
+// which must be zero when a launch starts and are left zero by it; the partials
+// (part_bytes) follow.
 struct AttnStandalonePlan {
     int groups, splits;  // splits: CTAs per head (mtp_attention*), key splits (mtp_attention_tc)
     bool whole;          // mtp_attention*: a CTA per group and head instead
-    size_t part_bytes, count_bytes, need;
+    size_t part_bytes, count_bytes, need;  // count_bytes: the same for every call on a device
     size_t least;        // bytes a call is accepted with (need: what it runs fastest with)
 };
 // MTP_OK or MTP_ERR_INVALID / MTP_ERR_CUDA (message set); with check_pointers
 // the device pointers must be non-null too.
 int attention_standalone_plan(const struct ::mtp_attention_args* a, bool check_pointers, AttnStandalonePlan* p);
-// Enqueue the kernel on `stream` with the `bytes` (>= p.least) of `workspace`: partials, then counters.
+// Enqueue the kernel on `stream` with the `bytes` (>= p.least) of `workspace`.
 int attention_standalone_launch(const struct ::mtp_attention_args* a, const AttnStandalonePlan& p, void* workspace,
                                 size_t bytes, cudaStream_t stream);
 

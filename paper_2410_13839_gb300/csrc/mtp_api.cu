@@ -568,11 +568,10 @@ int setup_batched(mtp_ctx* c) {
     c->d_uhi = reinterpret_cast<__nv_bfloat16*>(uhi);
     c->d_ulo = reinterpret_cast<__nv_bfloat16*>(ulo);
     {  // attention workspace: one wave's partials, and those of a tensor-core prefill pass of few tiles
-        const int groups = std::max(cf.max_batch + PREFILL_ROWS, (c->bm_max + 7) / 8);  // lane: groups of one row
         c->battn_ctas = std::max(1, ATTN_CTAS_PER_SM * c->num_sms / H);
         c->battn_ws_floats = std::max(attn_workspace_floats(H, c->battn_ctas), attn_tc_workspace_floats(4, H, 2));
         MTP_TRY(c->alloc(&c->d_bws, c->battn_ws_floats));
-        MTP_TRY(c->alloc(&c->d_bwc, (size_t)groups * H));
+        MTP_TRY(c->alloc(&c->d_bwc, attn_counters(c->num_sms)));
     }
     c->lmaps.resize(cf.layers);
     int bad = 0;
@@ -1174,13 +1173,13 @@ int mtp::attention_standalone_plan(const mtp_attention_args* a, bool check_point
     p->whole = attn_whole_groups(p->groups, a->n_heads, a->page_size, a->max_keys, sms);
     p->splits = p->whole ? 1 : attn_ctas_for(p->groups, a->n_heads, a->page_size, a->max_keys, sms);
     p->part_bytes = align256(attn_workspace_floats(a->n_heads, p->splits) * sizeof(float));
-    p->count_bytes = align256((size_t)p->groups * a->n_heads * sizeof(int));
+    p->count_bytes = align256(attn_counters(sms) * sizeof(int));
     // a call is accepted with the partials of `parts` key splits of every group, as the operator has always
     // asked for; it runs with as many CTAs per head as the workspace has room for
     const int max_pages = (a->max_keys + a->page_size - 1) / a->page_size;
     const int parts = std::max(1, std::min({sms / std::max(1, p->groups * a->n_heads), max_pages, 32}));
     p->least = align256((size_t)p->groups * a->n_heads * parts * MAX_ROWS * (2 + HEAD_DIM) * sizeof(float)) +
-               p->count_bytes;
+               align256((size_t)p->groups * a->n_heads * sizeof(int));
     p->need = std::max(p->part_bytes + p->count_bytes, p->least);
     return MTP_OK;
 }
@@ -1197,13 +1196,15 @@ int mtp::attention_standalone_launch(const mtp_attention_args* a, const AttnStan
     at.block_table = a->block_table; at.bt_stride = a->bt_stride;
     at.row_seq = a->row_seq; at.row_pos = a->row_pos;
     at.out = a->out; at.ldo = d;
-    at.ws_count = static_cast<int*>(workspace);  // counters, then partials
+    // counters, then partials: no call's partials lie where another's counters are, so one zeroed buffer
+    // serves calls of all sizes and both operators
+    at.ws_count = static_cast<int*>(workspace);
     at.ws_part = reinterpret_cast<float*>(static_cast<char*>(workspace) + p.count_bytes);
     at.rows_per_group = a->rows_per_group; at.n_heads = a->n_heads; at.page_size = a->page_size;
     at.groups = p.groups; at.rows = a->rows;
-    const size_t room = (bytes - p.count_bytes) / sizeof(float);
+    const size_t room = bytes > p.count_bytes ? (bytes - p.count_bytes) / sizeof(float) : 0;
     for (at.ctas = p.splits; at.ctas > 1 && attn_workspace_floats(a->n_heads, at.ctas) > room;) --at.ctas;
-    at.whole = p.whole;
+    at.whole = p.whole || (at.ctas < p.splits && at.ctas < p.groups);  // (a CTA per group needs no room)
     at.plan = PLAN_ROWS;
     at.err = nullptr;
     CUDA_TRY(launch_attention_plain(at, stream));
@@ -1873,8 +1874,10 @@ int attention_tc_plan(const mtp_attention_args* a, bool check_pointers, AttnStan
     p->groups = attn_tc_tiles(a->rows);
     p->splits = attn_tc_splits_for(p->groups, a->n_heads, a->max_keys, sms);
     p->part_bytes = align256(attn_tc_workspace_floats(p->groups, a->n_heads, p->splits) * sizeof(float));
-    p->count_bytes = align256((size_t)p->groups * a->n_heads * sizeof(int));
-    p->need = p->least = p->part_bytes + p->count_bytes;
+    p->count_bytes = align256(attn_counters(sms) * sizeof(int));
+    p->need = p->part_bytes + p->count_bytes;
+    p->least = p->part_bytes + align256((size_t)p->groups * a->n_heads * sizeof(int));  // as the operator has always asked
+    p->need = std::max(p->need, p->least);
     return MTP_OK;
 }
 }  // namespace
@@ -1895,7 +1898,7 @@ MTP_API int mtp_attention_tc(const mtp_attention_args* a, void* workspace, size_
     AttnStandalonePlan p;
     MTP_TRY(attention_tc_plan(a, true, &p));
     if (!workspace) return fail(MTP_ERR_INVALID, "attention_tc: null workspace");
-    if (workspace_bytes < p.need)
+    if (workspace_bytes < p.least)
         return fail(MTP_ERR_INVALID, "attention_tc: workspace %zu bytes, need %zu", workspace_bytes, p.need);
     AttnArgs at;
     std::memset(&at, 0, sizeof(at));
@@ -1907,10 +1910,13 @@ MTP_API int mtp_attention_tc(const mtp_attention_args* a, void* workspace, size_
     at.block_table = a->block_table; at.bt_stride = a->bt_stride;
     at.row_seq = a->row_seq; at.row_pos = a->row_pos;
     at.out = a->out; at.ldo = d;
-    at.ws_part = static_cast<float*>(workspace);
-    at.ws_count = reinterpret_cast<int*>(static_cast<char*>(workspace) + p.part_bytes);
+    at.ws_count = static_cast<int*>(workspace);  // counters, then partials, as mtp_attention
+    at.ws_part = reinterpret_cast<float*>(static_cast<char*>(workspace) + p.count_bytes);
     at.rows = a->rows; at.n_heads = a->n_heads; at.page_size = a->page_size;
-    at.n_splits = p.splits; at.plan = PLAN_ROWS;
+    const size_t room = workspace_bytes > p.count_bytes ? (workspace_bytes - p.count_bytes) / sizeof(float) : 0;
+    at.n_splits = p.splits;
+    while (at.n_splits > 1 && attn_tc_workspace_floats(p.groups, a->n_heads, at.n_splits) > room) --at.n_splits;
+    at.plan = PLAN_ROWS;
     at.err = nullptr;
     CUDA_TRY(launch_attention_tc(at, static_cast<cudaStream_t>(cuda_stream), false));
     return MTP_OK;
