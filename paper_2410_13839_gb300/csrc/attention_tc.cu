@@ -17,18 +17,26 @@
 //                                segment's rows and keys <= the row's position;
 //                                written to TMEM as bf16 hi + lo, 64 keys at a time
 //   O += (P_hi + P_lo) V         two MMAs per 16 keys with P read from TMEM,
-//                                128 x 64 fp32 accumulated in TMEM (V read as
-//                                an MN-major operand)
+//                                128 x 64 fp32 in TMEM per 64 keys (V read as an
+//                                MN-major operand), added up in registers
 //
-// m is a row's running maximum; where no row of a warp has a new one, O is left
-// alone, otherwise the warp rescales it.  (A reference that may lag behind by up
-// to 2^8 costs no less time but 2.80e-6 instead of 2.73e-6 from 64 bits.)
+// m is a row's running maximum; where no row of a warp has a new one, nothing is
+// rescaled.  (A reference that may lag behind by up to 2^8 costs no less time but
+// 2.80e-6 instead of 2.73e-6 from 64 bits.)
 //
-// What bounds it: the softmax's instructions, about 10 per score with one warp
-// per scheduler and CTA.  S is read into registers at once, so the next item's
-// S = Q K^T runs under this one's softmax, P V of each half under the other
-// half's, and two CTAs share an SM (97 KB of shared memory, 256 TMEM columns
-// each).
+// O is accumulated in TMEM over 64 keys only; the row threads add these products
+// up in registers, in fp32, and rescale them there.  The tensor core truncates its
+// accumulator at every MMA, so a sum over all of a row's keys drifts: with values
+// of mean 1, rows of one prompt of 2000 keys are 3.5e-7 from 64 bits, and 1.4e-6
+// with one accumulation per row (4.2e-7 with one per 128 keys; mean 0: 2.84e-6,
+// 2.92e-6 and 2.87e-6).  It costs no time: the rescaling in TMEM, which reads and
+// writes O, was needed for most halves, and goes.
+//
+// What bounds it: the softmax's instructions, about 8 per score with one warp per
+// scheduler and CTA (fp32 additions and multiplications two at a time).  S is
+// read into registers at once, so the next item's S = Q K^T runs under this one's
+// softmax, P V of each half under the other half's, and two CTAs share an SM (97
+// KB of shared memory, 256 TMEM columns each).
 // Q and P enter as bf16 hi + lo pairs (hi + lo = x to about 2^-16 relative),
 // so the products keep fp32 accuracy; the keys and values are the cache's bf16.
 // One elected thread of the fifth warp issues the copies and the MMAs; the
@@ -66,6 +74,23 @@ __device__ __forceinline__ float ex2(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
+// Two fp32 operations in one instruction, each rounded on its own.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n\t.reg .b64 a, b, c, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tmov.b64 c, {%6, %7};\n\t"
+        "fma.rn.f32x2 d, a, b, c;\n\tmov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+        "add.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
 // D = A B (+ D) with A (bf16, K-major) read from TMEM: lane = row, two K elements per column
 __device__ __forceinline__ void tc_mma_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc,
                                           uint32_t acc) {
@@ -89,7 +114,8 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 __device__ __forceinline__ void split_pair(float x0, float x1, uint32_t& hi, uint32_t& lo) {
     const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
     hi = *reinterpret_cast<const uint32_t*>(&h);
-    const __nv_bfloat162 l = __floats2bfloat162_rn(x0 - bf16_lo(hi), x1 - bf16_hi(hi));
+    const float2 r = add2(make_float2(x0, x1), make_float2(-bf16_lo(hi), -bf16_hi(hi)));
+    const __nv_bfloat162 l = __floats2bfloat162_rn(r.x, r.y);
     lo = *reinterpret_cast<const uint32_t*>(&l);
 }
 
@@ -202,6 +228,24 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
     const int2 first = skip_empty(make_int2(0, sp));
 
     float m_run = -INFINITY, l_run = 0.f;  // m_run in log2 units
+    float o[HEAD_DIM];  // this row's unnormalised output, without the last half's product
+#pragma unroll
+    for (int c = 0; c < HEAD_DIM; ++c) o[c] = 0.f;
+    // adds the last half's product (complete) to it
+    auto add_product = [&]() {
+#pragma unroll
+        for (int c0 = 0; c0 < HEAD_DIM; c0 += 16) {
+            float v[16];
+            tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + TM_O + c0, v);
+#pragma unroll
+            for (int e = 0; e < 16; e += 2) {
+                const float2 y = add2(make_float2(o[c0 + e], o[c0 + e + 1]), make_float2(v[e], v[e + 1]));
+                o[c0 + e] = y.x;
+                o[c0 + e + 1] = y.y;
+            }
+        }
+    };
+    bool seen = false;  // a row of the warp sees keys of the last half
     int items = 0;
     bool fine = true;
     if (warp == 4) {  // ---- the issuing warp: copies (a lane per page) and MMAs (lane 0) ----
@@ -294,7 +338,7 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
 #pragma unroll
                     for (int kk = 0; kk < PA_HALF / 16; ++kk) {
                         const uint64_t bv = sw128_mn_desc(vb + (half * (PA_HALF / 16) + kk) * 2048);
-                        tc_mma_ta(tmem + TM_O, tmem + TM_P + kk * 8, bv, IDESC_O, (i | half | kk) != 0);
+                        tc_mma_ta(tmem + TM_O, tmem + TM_P + kk * 8, bv, IDESC_O, kk != 0);
                         tc_mma_ta(tmem + TM_O, tmem + TM_PLO + kk * 8, bv, IDESC_O, 1u);
                     }
                 }
@@ -384,16 +428,16 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
                     if (move) corr = ex2(m_run - top);
                     if (fresh || move) m_run = top;
                     const float ref = m_run == -INFINITY ? 0.f : m_run;  // a row that has seen no key: every weight 0
-                    float sum[4] = {0.f, 0.f, 0.f, 0.f};
+                    float2 sum[2] = {{0.f, 0.f}, {0.f, 0.f}};
 #pragma unroll
                     for (int e = 0; e < PA_HALF / 2; ++e) {
-                        const float p0 = ex2(fmaf(sv[2 * e], LOG2E, -ref));
-                        const float p1 = ex2(fmaf(sv[2 * e + 1], LOG2E, -ref));
-                        sum[(2 * e) & 3] += p0;
-                        sum[(2 * e + 1) & 3] += p1;
-                        split_pair(p0, p1, hi[e], lo[e]);
+                        const float2 x = fma2(make_float2(sv[2 * e], sv[2 * e + 1]), make_float2(LOG2E, LOG2E),
+                                              make_float2(-ref, -ref));
+                        const float2 p = make_float2(ex2(x.x), ex2(x.y));
+                        sum[e & 1] = add2(sum[e & 1], p);
+                        split_pair(p.x, p.y, hi[e], lo[e]);
                     }
-                    l_run = fmaf(l_run, corr, (sum[0] + sum[1]) + (sum[2] + sum[3]));
+                    l_run = fmaf(l_run, corr, (sum[0].x + sum[0].y) + (sum[1].x + sum[1].y));
                 } else {
                     if (half) {
                         __syncwarp();
@@ -402,23 +446,18 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
 #pragma unroll
                     for (int e = 0; e < PA_HALF / 2; ++e) hi[e] = lo[e] = 0u;
                 }
-                // the previous half's weights have been read (and O is complete up to them)
+                // the previous half's weights have been read, and its product is complete
                 if (half || items > 0)
                     done = __all_sync(FULL_MASK, lane != 0 || mbar_wait(&pv_done[half ^ 1],
                                                                         (uint32_t)(half ? items : items - 1) & 1, a.err));
                 if (!done) break;
                 tc_fence_after();
+                if (seen) add_product();  // the next product overwrites it
                 if (__any_sync(FULL_MASK, move)) {
 #pragma unroll
-                    for (int c0 = 0; c0 < HEAD_DIM; c0 += 16) {
-                        float v[16];
-                        uint32_t r[16];
-                        tmem_ld16(base + TM_O + c0, v);
-#pragma unroll
-                        for (int e = 0; e < 16; ++e) r[e] = __float_as_uint(v[e] * corr);
-                        tmem_st16(base + TM_O + c0, r);
-                    }
+                    for (int c = 0; c < HEAD_DIM; ++c) o[c] *= corr;
                 }
+                seen = need;
 #pragma unroll
                 for (int q = 0; q < PA_HALF / 2; q += 16) {
                     tmem_st16(base + TM_P + q, *reinterpret_cast<const uint32_t(*)[16]>(&hi[q]));
@@ -436,20 +475,10 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
             }
         }
     }
-    // ---- this row's unnormalised output (registers) ----
-    float o[HEAD_DIM];
-#pragma unroll
-    for (int c = 0; c < HEAD_DIM; ++c) o[c] = 0.f;
     if (tid < PA_ROWS && items > 0 && fine) {
         if (__all_sync(FULL_MASK, lane != 0 || mbar_wait(&pv_done[1], (uint32_t)(items - 1) & 1, a.err))) {
             tc_fence_after();
-#pragma unroll
-            for (int c0 = 0; c0 < HEAD_DIM; c0 += 32) {
-                float v[32];
-                tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + TM_O + c0, v);
-#pragma unroll
-                for (int e = 0; e < 32; ++e) o[c0 + e] = v[e];
-            }
+            if (seen) add_product();
         } else {
             s_abort = 1;
         }
