@@ -43,6 +43,7 @@
 // four other warps own one row each per thread.  Splits leave (maximum, sum,
 // unnormalised output) per row in the workspace and the CTA that finishes
 // last merges them (an atomic counter per tile and head, reset by that CTA).
+#include <float.h>
 #include <math.h>
 
 #include <algorithm>
@@ -87,6 +88,14 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
     float2 d;
     asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
         "add.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    float2 d;
+    asm("{\n\t.reg .b64 a, b, d;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+        "mul.rn.f32x2 d, a, b;\n\tmov.b64 {%0, %1}, d;\n\t}"
         : "=f"(d.x), "=f"(d.y)
         : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
     return d;
@@ -491,11 +500,21 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
     // ---- results: rows of this tile, through shared memory (Q's space is free), 16 lanes per row ----
     const int r = row0 + tid;
     float4* ost = reinterpret_cast<float4*>(sm + OFF_Q);  // [128][16], chunk c of row q at c ^ (q & 15)
-    auto stage_row = [&](const float* v, float scale) {
+    // v / sum: the product with the reciprocal, corrected by its remainder (q + r (v - q sum); 64 divisions
+    // are 2 us of instructions that every tile fetches and runs once).  An infinite q has no remainder: any
+    // finite value leaves it as it is.
+    auto stage_row = [&](const float* v, float sum) {
+        const float r = 1.f / sum;
+        auto quotients = [&](const float* x) {
+            const float2 y = make_float2(x[0], x[1]), r2 = make_float2(r, r);
+            const float2 q = mul2(y, r2), rem = fma2(q, make_float2(-sum, -sum), y);
+            return fma2(make_float2(fmaxf(rem.x, -FLT_MAX), fmaxf(rem.y, -FLT_MAX)), r2, q);
+        };
 #pragma unroll
-        for (int c = 0; c < HEAD_DIM / 4; ++c)
-            ost[tid * 16 + (c ^ (tid & 15))] =
-                make_float4(v[4 * c] * scale, v[4 * c + 1] * scale, v[4 * c + 2] * scale, v[4 * c + 3] * scale);
+        for (int c = 0; c < HEAD_DIM / 4; ++c) {
+            const float2 a0 = quotients(v + 4 * c), a1 = quotients(v + 4 * c + 2);
+            ost[tid * 16 + (c ^ (tid & 15))] = make_float4(a0.x, a0.y, a1.x, a1.y);
+        }
     };
     auto write_rows = [&]() {  // every warp writes the rows its own threads staged, 8 lanes and dims each
         __syncwarp();
@@ -539,7 +558,7 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
     const bool active = tid < PA_ROWS && r < a.rows && my_seq >= 0;
     if (S == 1) {
         if (tid >= PA_ROWS) return;
-        if (active) stage_row(o, 1.f / l_run);
+        if (active) stage_row(o, l_run);
         write_rows();
         return;
     }
@@ -583,7 +602,7 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
                 o[c + 3] = fmaf(w, v.w, o[c + 3]);
             }
         }
-        stage_row(o, 1.f / L);
+        stage_row(o, L);
     }
     write_rows();
 }

@@ -45,3 +45,33 @@ def test_prompt_sums_do_not_drift():
     """Values of mean 1: an accumulation only grows, and the tensor core truncates it at every MMA, by less than
     2^-23.  64 keys are eight MMAs; what lies behind them is added in fp32."""
     assert _error(True, 4, 2000, 1900, 1.0, 8) <= 8 * 2.0 ** -23
+
+
+@pytest.mark.parametrize("tc", [False, True])
+@pytest.mark.parametrize("keys,rows", [(100, 100), (1100, 64)])
+def test_equal_weights_give_the_rounded_mean(tc, keys, rows):
+    """Queries of zero weight every key alike, whole values make the sums exact: what is left is one division,
+    which is rounded once."""
+    torch = pytest.importorskip("torch")
+    mtp = lib_module()
+    heads, pages = 2, -(-keys // P)
+    gen = torch.Generator(device="cuda").manual_seed(keys)
+    kv = torch.randn(pages, 2, heads, P, HD, device="cuda", generator=gen).bfloat16()
+    kv[:, 1] = torch.randint(-128, 129, (pages, heads, P, HD), device="cuda", generator=gen).bfloat16()
+    pool = kv
+    if tc:  # the cache's row layout: chunk c of row t at chunk c ^ (t mod 8)
+        t, c = torch.arange(P, device="cuda")[:, None], torch.arange(8, device="cuda")[None, :]
+        pool = kv.view(pages, 2, heads, P, 8, 8)[..., t, c ^ (t & 7), :].flatten(-2).contiguous()
+    q = torch.zeros(rows, heads * HD, device="cuda")
+    ints = lambda x: torch.tensor(x, dtype=torch.int32, device="cuda")  # noqa: E731
+    table, seq, pos = ints([list(range(pages))]), ints([0] * rows), ints(list(range(keys - rows, keys)))
+    out = torch.zeros(rows, heads * HD, device="cuda")
+    args = mtp.attention_args(rows=rows, rows_per_group=min(8, rows), n_heads=heads, page_size=P, layers=1, layer=0,
+                              bt_stride=pages, max_keys=keys, q=q, kv_pool=pool, block_table=table, row_seq=seq,
+                              row_pos=pos, out=out)
+    nbytes = (mtp.mtp_attention_tc_workspace_bytes if tc else mtp.mtp_attention_workspace_bytes)(args)
+    ws = torch.zeros(max(16, nbytes), dtype=torch.uint8, device="cuda")
+    (mtp.mtp_attention_tc if tc else mtp.mtp_attention)(args, ws, nbytes, torch.cuda.current_stream())
+    sums = kv[:, 1].double().permute(1, 0, 2, 3).flatten(1, 2).cumsum(1)[:, keys - rows:keys]
+    want = (sums / (pos.double() + 1)[None, :, None]).float().transpose(0, 1).flatten(1)
+    assert torch.equal(out, want)
