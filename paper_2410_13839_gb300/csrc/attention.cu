@@ -363,7 +363,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 4)
                 for (int hh = 0; hh < 2; ++hh)
                     v[ks][hh] = make_float2(qr[ks * 16 + hh * 8], qr[ks * 16 + hh * 8 + 1]);
             act = __ballot_sync(FULL_MASK, row_pos >= 0);
-            const float scale = in && (act >> g8 & 1) ? 0.125f * LOG2E : 0.f;  // 1/sqrt(64); scores in log2 units
+            const float scale = in && (act >> g8 & 1) ? 0.125f : 0.f;  // 1/sqrt(64): bf16-valued queries stay exact
 #pragma unroll
             for (int j = 0; j < 2; ++j) qpos[j] = __shfl_sync(FULL_MASK, row_pos, c2 + j);
 #pragma unroll
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 4)
                     split2(scale != 0.f ? v[ks][hh].x * scale : 0.f, scale != 0.f ? v[ks][hh].y * scale : 0.f,
                            qhi[ks][hh], qlo[ks][hh]);
         }
-        float m_w[2] = {-INFINITY, -INFINITY}, l_w[2] = {0.f, 0.f};
+        float m_w[2] = {-INFINITY, -INFINITY} /* log2 units */, l_w[2] = {0.f, 0.f};
         float o[4][4];  // O^T block dp: dims dp * 16 + g8 (0, 1) and + 8 (2, 3), queries c2 + (i & 1)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 4)
                 // the maximum over the lanes and the rescaling are skipped.  (A reference that may lag behind by
                 // up to 2^8 moves less often, 0.5 % faster, but 32 slots of 180-2000 keys are then 3.4e-6 from
                 // 64 bits instead of 3.1e-6.)
-                float t0 = fmaxf(sv[0], sv[2]), t1 = fmaxf(sv[1], sv[3]);
+                float t0 = fmaxf(sv[0], sv[2]) * LOG2E, t1 = fmaxf(sv[1], sv[3]) * LOG2E;
                 if (__any_sync(FULL_MASK, t0 > m_w[0] || t1 > m_w[1])) {
 #pragma unroll
                     for (int off = 4; off < 32; off <<= 1) {  // over the tile's keys: lanes g8
@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(ATT_THREADS, 4)
                 }
                 float pv[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) pv[e] = sv[e] == -INFINITY ? 0.f : ex2(sv[e] - m_w[e & 1]);
+                for (int e = 0; e < 4; ++e) pv[e] = sv[e] == -INFINITY ? 0.f : ex2(fmaf(sv[e], LOG2E, -m_w[e & 1]));
                 l_w[0] += pv[0] + pv[2];
                 l_w[1] += pv[1] + pv[3];
                 // P^T as the B operand (keys x queries): this lane holds rows g8 (keys) and columns c2

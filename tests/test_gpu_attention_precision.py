@@ -49,20 +49,26 @@ def test_prompt_sums_do_not_drift():
 
 @pytest.mark.parametrize("tc", [False, True])
 @pytest.mark.parametrize("keys,rows", [(100, 100), (1100, 64)])
-def test_equal_weights_give_the_rounded_mean(tc, keys, rows):
-    """Queries of zero weight every key alike, whole values make the sums exact: what is left is one division,
-    which is rounded once."""
+@pytest.mark.parametrize("queries", ["zero", "cancelling"])
+def test_equal_weights_give_the_rounded_mean(tc, keys, rows, queries):
+    """Where every score is zero the weights are equal, and whole values make the sums exact: what is left is one
+    division, which is rounded once.  Queries (3, 5) against keys (5 t, -3 t) are zero only if the scaled queries
+    are exact, as bf16-valued ones are when scaled by 1/8."""
     torch = pytest.importorskip("torch")
     mtp = lib_module()
     heads, pages = 2, -(-keys // P)
     gen = torch.Generator(device="cuda").manual_seed(keys)
     kv = torch.randn(pages, 2, heads, P, HD, device="cuda", generator=gen).bfloat16()
     kv[:, 1] = torch.randint(-128, 129, (pages, heads, P, HD), device="cuda", generator=gen).bfloat16()
+    q = torch.zeros(rows, heads * HD, device="cuda")
+    if queries == "cancelling":
+        q[:, 0::2], q[:, 1::2] = 3.0, 5.0
+        t = torch.randint(-25, 26, (pages, heads, P, HD // 2), device="cuda", generator=gen)
+        kv[:, 0, ..., 0::2], kv[:, 0, ..., 1::2] = (5 * t).bfloat16(), (-3 * t).bfloat16()
     pool = kv
     if tc:  # the cache's row layout: chunk c of row t at chunk c ^ (t mod 8)
         t, c = torch.arange(P, device="cuda")[:, None], torch.arange(8, device="cuda")[None, :]
         pool = kv.view(pages, 2, heads, P, 8, 8)[..., t, c ^ (t & 7), :].flatten(-2).contiguous()
-    q = torch.zeros(rows, heads * HD, device="cuda")
     ints = lambda x: torch.tensor(x, dtype=torch.int32, device="cuda")  # noqa: E731
     table, seq, pos = ints([list(range(pages))]), ints([0] * rows), ints(list(range(keys - rows, keys)))
     out = torch.zeros(rows, heads * HD, device="cuda")
