@@ -600,12 +600,25 @@ cudaError_t launch_viterbi_kp(const ViterbiArgs& a, cudaStream_t s) {
 
 }  // namespace
 
+// Under programmatic launch the blocks are placed while the kernel before them still holds its SMs' shared
+// memory, and then pack onto the few SMs that have room: 8 rows of 8 heads, top-32, behind a head product of
+// 200 KB a CTA took 84 us a call in mtp_heads_topk, 45 without programmatic launch.  A request of more than half
+// an SM's shared memory puts one block on an SM: 42 us (4 heads, top-4: 14.9 either way, 16.9 without).  More
+// blocks than SMs share them anyway.
+constexpr int SELECT_SPREAD = 128;  // most blocks that are spread: no sm_103a part has fewer SMs
+constexpr size_t SELECT_SPREAD_SMEM = 128 * 1024;
+
 cudaError_t launch_select(const SelectArgs& a, int batch, bool do_accept, cudaStream_t s, bool pdl) {
     if (a.n < 1 || a.n > MAX_NHEADS || a.k < 1 || a.k > MAX_TOPK || a.V > MAX_VOCAB || a.k > a.V)
         return cudaErrorInvalidValue;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(batch);
     cfg.blockDim = dim3(256);
+    if (pdl && batch > 1 && batch <= SELECT_SPREAD) {
+        const cudaError_t e = ensure_kernel_smem(reinterpret_cast<const void*>(select_kernel), SELECT_SPREAD_SMEM);
+        if (e != cudaSuccess) return e;
+        cfg.dynamicSmemBytes = SELECT_SPREAD_SMEM;
+    }
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
