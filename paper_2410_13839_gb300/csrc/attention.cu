@@ -171,8 +171,9 @@ __global__ void __launch_bounds__(ATT_THREADS, 4)
     }
 
     // ---- this CTA's share of the head's stream of batches ----
-    const bool few = a.groups <= ATT_THREADS && !a.whole;
-    auto group_of = [&](int g) { return few ? s_group[g] : load_group(a, g); };
+    // the groups' facts in shared memory: of all of them, or (whole) of this CTA's
+    const bool few = a.groups <= ATT_THREADS || a.whole;
+    auto group_of = [&](int g) { return few ? s_group[a.whole ? 0 : g] : load_group(a, g); };
     auto batches = [&](const Group& x) { return (x.keys + KB - 1) / KB; };
     // inclusive sum of v over the block's threads before and including this one; total: of all
     auto block_scan = [&](int v, int& total) {
@@ -195,8 +196,10 @@ __global__ void __launch_bounds__(ATT_THREADS, 4)
     int T, J, x0, x1;  // batches of the head, CTAs that take part (each has a batch), this CTA's range
     if (a.whole) {  // group jc, all of it
         T = J = x0 = 0;
-        x1 = batches(load_group(a, jc));
+        const Group x = load_group(a, jc);
+        x1 = batches(x);
         if (tid == 0) {
+            s_group[0] = x;
             s_g0 = jc;
             s_off = 0;
         }
@@ -592,17 +595,24 @@ size_t attn_smem_bytes(int page_size) {
 int attn_ctas_per_sm(int page_size) { return page_size > 64 ? ATTN_CTAS_PER_SM / 2 : ATTN_CTAS_PER_SM; }
 
 int attn_ctas_for(int groups, int n_heads, int page_size, int max_keys, int num_sms) {
-    // one wave of resident CTAs while they have batches; of a long context's batches at least two each
-    // (sharing a group costs its CTAs a partial each and a merge)
-    const int nb = (max_keys + half_keys(page_size) - 1) / half_keys(page_size);  // batches per group
-    const long long want = (long long)groups * (nb >= 8 ? nb / 2 : nb);
+    // one wave of resident CTAs while they have batches: a batch each (5 slots of 100-600 keys, 8 heads: 10.5 us,
+    // 12.7 with two), of contexts over 1024 keys more, since every CTA of a group leaves partials that its last
+    // one merges (1 slot of 2000 keys, 16 heads: 20.8, 14.6 and 12.6 us with 32, 16 and 8 CTAs a head; with few
+    // heads the merges do not meet in time: 2 slots, 1 head: 12.5, 11.0 and 12.5)
+    const int kb = half_keys(page_size), nb = (max_keys + kb - 1) / kb;  // keys of a batch, batches per group
+    const int each = max_keys <= 1024 ? 1 : (n_heads <= 4 ? 128 : 256) / kb;
+    const long long want = (long long)groups * ((nb + each - 1) / each);
     return (int)max(1ll, min(want, (long long)max(1, attn_ctas_per_sm(page_size) * num_sms / n_heads)));
 }
 
 bool attn_whole_groups(int groups, int n_heads, int page_size, int max_keys, int num_sms) {
-    // contexts of a batch or two that fill the GPU: a plan and a merge would cost more than they share out
-    // (20 slots of 33-99 keys, 16 heads: 8.5 vs 10.4 us)
-    return max_keys <= 2 * half_keys(page_size) && (long long)groups * n_heads >= num_sms;
+    // contexts of a batch or two: a plan and a merge would cost more than they share out (1 slot of 33 keys: 6.6 vs
+    // 8.4 us; 20 slots of 33-99 keys, 16 heads: 8.5 vs 10.4).  Longer ones where the groups are most of a wave, and
+    // no more: 20 slots of 200-400 keys, 8 heads: 12.6 vs 18.9 us, 10 slots of 300-600, 12 heads: 12.6 vs 14.6 (with
+    // 8 heads, 80 groups, 14.5 vs 12.5; 32 slots of 180-2000 keys, 8 heads: 28.4 vs 20.7).
+    const long long ctas = (long long)groups * n_heads;
+    return max_keys <= 2 * half_keys(page_size) ||
+           (max_keys <= 640 && 4 * ctas >= 3ll * num_sms && ctas <= (long long)attn_ctas_per_sm(page_size) * num_sms);
 }
 
 template <bool PLAIN>
