@@ -5,9 +5,9 @@
 //
 // Grid (split, head, tile).  A tile is 128 rows of the pass, the MMA's M side
 // and the 128 TMEM lanes; its rows may belong to several slots (a prefill pass
-// packs the prompts of many slots).  Each run of consecutive rows of one slot
-// is a segment; the segment's keys 0 .. (its largest position) are cut into
-// items of 128 keys, and split s takes items s, s + S, ... of every segment.
+// packs the prompts of many slots), in any order.  The tile's rows of one slot are
+// a segment; the segment's keys 0 .. (its largest position) are cut into items of
+// 128 keys, and split s takes items s, s + S, ... of every segment.
 // Per item, with the cached keys and values of the item's pages copied by
 // cp.async.bulk into a two-stage ring (the cache stores chunk c of key row t
 // at c ^ (t & 7): exactly the 128-byte-swizzled tile the MMA reads):
@@ -132,13 +132,56 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
+struct TileRows {
+    int seq[PA_ROWS];                  // the rows' slots
+    int slot[PA_ROWS], kmax[PA_ROWS];  // segments: the tile's rows of one slot, the keys they see
+    int count[PA_ROWS / 32];           // run starts per warp
+    int number[PA_ROWS];               // a slot's first run -> its segment
+};
+
+// Runs 0 .. nseg - 1 joined to a segment per slot, in order of the slots' first runs; leaves the number of
+// segments in rows.count[0] and every row's in rows.seq (my_seg: the run of this thread's row, < 0: none).  The
+// whole block calls it.  (Not inlined, and nothing returned in registers: inlined it costs the softmax 8 %.)
+__device__ __noinline__ void join_runs(TileRows& rows, int nseg, int my_seg) {
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, runs = nseg;
+    int slot = -1, kmax = 0, first = 0;
+    if (tid < runs) {
+        slot = rows.slot[tid];
+        kmax = rows.kmax[tid];
+        while (rows.slot[first] != slot) ++first;
+    }
+    const bool own = tid < runs && first == tid;
+    const unsigned owners = __ballot_sync(FULL_MASK, own);
+    if (tid < PA_ROWS) {
+        rows.seq[tid] = first;  // a run's first run of the same slot
+        if (lane == 0) rows.count[warp] = __popc(owners);
+    }
+    __syncthreads();
+    int number = __popc(owners & ((1u << lane) - 1));
+    nseg = 0;
+    for (int w = 0; w < PA_ROWS / 32; ++w) {
+        if (w == warp) number += nseg;
+        nseg += rows.count[w];
+    }
+    if (own) {
+        rows.number[tid] = number;
+        rows.slot[number] = slot;
+    }
+    if (tid < PA_ROWS) rows.kmax[tid] = 0;
+    __syncthreads();
+    if (tid < runs) atomicMax(&rows.kmax[rows.number[first]], kmax);
+    if (my_seg >= 0) my_seg = rows.number[rows.seq[my_seg]];
+    __syncthreads();
+    if (tid < PA_ROWS) rows.seq[tid] = my_seg;
+    if (tid == 0) rows.count[0] = nseg;
+    __syncthreads();
+}
+
 __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a) {
     extern __shared__ __align__(1024) unsigned char pa_raw[];
     __shared__ uint64_t kv_full[2], s_full, s_read, p_full[2], pv_done[2];  // p, pv: the item's halves
     __shared__ uint32_t tmem_base;
-    __shared__ int s_seq[PA_ROWS];
-    __shared__ int seg_slot[PA_ROWS], seg_kmax[PA_ROWS];  // runs of consecutive rows of one slot
-    __shared__ int s_heads[PA_ROWS / 32];                 // run starts per warp
+    __shared__ TileRows rows;
     __shared__ int s_abort, s_last;
     unsigned char* sm = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(pa_raw) + 1023) & ~(uintptr_t)1023);
     TraceEnd trace_guard(a.trace);
@@ -198,33 +241,40 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
             my_seq = a.row_seq[r];
             my_pos = a.row_pos[r];
         }
-        s_seq[tid] = my_seq;
-        seg_kmax[tid] = 0;
+        rows.seq[tid] = my_seq;
+        rows.kmax[tid] = 0;
     }
     __syncthreads();
     bool head = false;
     unsigned heads = 0, live = 0;  // the warp's rows that start a run, and those of a sequence
     if (tid < PA_ROWS) {
         live = __ballot_sync(FULL_MASK, my_seq >= 0);
-        head = my_seq >= 0 && (tid == 0 || s_seq[tid - 1] != my_seq);
+        head = my_seq >= 0 && (tid == 0 || rows.seq[tid - 1] != my_seq);
         heads = __ballot_sync(FULL_MASK, head);
-        if (lane == 0) s_heads[warp] = __popc(heads);
+        if (lane == 0) rows.count[warp] = __popc(heads);
     }
     __syncthreads();
     int nseg = 0, my_seg = -1;
 #pragma unroll
     for (int w = 0; w < PA_ROWS / 32; ++w) {
         if (w == warp) my_seg = nseg + __popc(heads & (0xffffffffu >> (31 - lane))) - 1;  // run of this row
-        nseg += s_heads[w];
+        nseg += rows.count[w];
     }
     if (tid < PA_ROWS && my_seq >= 0) {
-        if (head) seg_slot[my_seg] = my_seq;
-        atomicMax(&seg_kmax[my_seg], my_pos + 1);
+        if (head) rows.slot[my_seg] = my_seq;
+        atomicMax(&rows.kmax[my_seg], my_pos + 1);
     }
     __syncthreads();
+    // a slot whose rows lie in several runs is one segment (runs of ascending slots, as packed prompts are, need
+    // no look)
+    if (nseg > 1 && __syncthreads_or(tid > 0 && tid < nseg && rows.slot[tid] <= rows.slot[tid - 1])) {
+        join_runs(rows, nseg, my_seg);
+        nseg = rows.count[0];
+        if (tid < PA_ROWS) my_seg = rows.seq[tid];
+    }
     // this split's items in order: segment g, key tiles j = sp, sp + S, ... below the segment's end
     auto skip_empty = [&](int2 t) {
-        while (t.x < nseg && t.y * PA_KEYS >= seg_kmax[t.x]) {
+        while (t.x < nseg && t.y * PA_KEYS >= rows.kmax[t.x]) {
             ++t.x;
             t.y = sp;
         }
@@ -266,8 +316,8 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
         auto item_page = [&](int2 t) {
             if (t.x >= nseg) return -2;
             const int p = t.y * (PA_KEYS / P) + lane;
-            if (lane >= PA_KEYS / P || p * P >= seg_kmax[t.x]) return -2;
-            return p < a.bt_stride ? max(-1, a.block_table[(size_t)seg_slot[t.x] * a.bt_stride + p]) : -1;
+            if (lane >= PA_KEYS / P || p * P >= rows.kmax[t.x]) return -2;
+            return p < a.bt_stride ? max(-1, a.block_table[(size_t)rows.slot[t.x] * a.bt_stride + p]) : -1;
         };
         // copies of item i into stage i & 1
         auto stage_item = [&](int i, int page) {
@@ -326,7 +376,7 @@ __global__ void __launch_bounds__(PA_THREADS, 2) attn_tc_kernel(const AttnArgs a
             s_issued = ok;
         }
         for (int2 t = first; ok && t.x < nseg; ++i) {
-            const int keys = seg_kmax[t.x] - t.y * PA_KEYS;  // of the item that some row of the tile sees
+            const int keys = rows.kmax[t.x] - t.y * PA_KEYS;  // of the item that some row of the tile sees
             t = next_item(t);
             const uint32_t vb = smem_addr(sm + OFF_KV + (uint32_t)(2 * (i & 1) + 1) * PA_TILE);
 #pragma unroll
