@@ -244,11 +244,10 @@ MTP_API int mtp_debug_lattice(mtp_ctx* ctx, int32_t* out_ids, float* out_logp, i
  *                        and cached keys streamed into shared-memory rings ahead of use, bounded grid
  *                        barriers between the attention and MLP phases), where the model and GPU
  *                        allow it; 0 = two block kernels per layer (default: faster on GB300 at B = 1)
- *   MTP_OPT_PREFILL_TC   attention of prefill passes (mtp_prefill, mtp_prefill_pending): 1 = always on the
- *                        tensor cores (tcgen05: tiles of 128 prompt rows, 128-key items, S and P V
- *                        accumulated in TMEM); 0 = so in passes of more than 304 rows (124 us per
- *                        launch at 14592 rows of 128 prompts, 16 heads), the kernel of the decode
- *                        steps, in groups of 8 rows, in smaller ones (default)
+ *   MTP_OPT_PREFILL_TC   attention of prefill passes (mtp_prefill, mtp_prefill_pending): 1 = always in
+ *                        tcgen05 tiles (128 prompt rows, 128-key items, S and P V accumulated in
+ *                        TMEM); 0 = always by the kernel of the decode steps, in groups of 8 rows;
+ *                        2 = tiles in passes of more than 304 rows, groups in smaller ones (default)
  *   MTP_OPT_GEMM_CLUSTER 1 = the batched path's projections at up to 128 fed rows run as one
  *                        activation tile per weight tile, their K split over the CTAs of a cluster
  *                        (2 or 4) that sum the partial tiles in distributed shared memory, each

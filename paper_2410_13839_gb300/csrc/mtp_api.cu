@@ -116,7 +116,7 @@ struct mtp_ctx {
     int device = 0, num_sms = 0, wbytes = 2;
     int mlp_clusters = 1;  // MLP clusters co-resident in one wave
     bool use_graphs = true, use_pdl = true, use_l2_prefetch = false;
-    bool use_attn_tc = false;  // prefill passes of any size: tcgen05 attention (option; else by the pass's rows)
+    int attn_tc = 2;  // prefill passes' attention in tcgen05 tiles: 0 never, 1 always, 2 by the pass's rows
     int use_heads_tc = 1;  // fused heads kernel: 0 never, 1 stand-alone heads calls, 2 also batched decode steps
     bool gemm_cluster = true;  // batched projections: one 128-row activation tile, K splits summed in clusters
     std::vector<void*> allocs;
@@ -332,7 +332,7 @@ int tile_index(int nt) { return nt == 32 ? 0 : (nt == 64 ? 1 : 2); }
 // slot b's fed rows b*n.., plan PLAN_DEVICE; prefill: 8 consecutive prompt
 // positions, plan PLAN_ROWS).  prefill_keys > 0: a prefill pass whose rows see
 // at most that many keys; its attention runs in tiles of 128 rows (tcgen05)
-// above PREFILL_TC_ROWS rows, or always with that option.  A tile's chain of
+// above PREFILL_TC_ROWS rows, or always or never by option.  A tile's chain of
 // 128-key items is longer than a group's of 64-key batches, which only enough
 // tiles pay back: whole prefills with the groups and with the tiles, ms, of one
 // prompt of 289 rows 0.70 and 0.75, of 320 0.78 and 0.75, of 448 0.86 and 0.82,
@@ -421,7 +421,7 @@ int run_layers_batched(mtp_ctx* c, int M, int rpg, int groups, int plan, cudaStr
         at.whole = prefill_keys > 0 || attn_whole_groups(groups, H, P, cf.max_ctx, c->num_sms);
         at.plan = plan; at.seq_len = c->d_len; at.seq_new = c->d_npend; at.active = c->d_active; at.done = c->d_done;
         at.err = c->d_err;
-        if (prefill_keys > 0 && (c->use_attn_tc || M > PREFILL_TC_ROWS) && plan == PLAN_ROWS) {
+        if (prefill_keys > 0 && plan == PLAN_ROWS && (c->attn_tc == 1 || (c->attn_tc == 2 && M > PREFILL_TC_ROWS))) {
             // tiles of 128 rows; splits as many as the batched attention workspace holds (S = 1 uses none)
             const int tiles = attn_tc_tiles(M);
             at.n_splits = std::max(1, std::min(attn_tc_splits_for(tiles, H, prefill_keys, c->num_sms),
@@ -1339,7 +1339,7 @@ MTP_API int mtp_set_option(mtp_ctx* c, int option, int value) {
         changed = c->use_persistent != (value != 0);
         c->use_persistent = value != 0;
     } else if (option == MTP_OPT_PREFILL_TC) {
-        c->use_attn_tc = value != 0;  // prefill passes are not captured
+        c->attn_tc = value == 0 || value == 2 ? value : 1;  // prefill passes are not captured
     } else if (option == MTP_OPT_GEMM_CLUSTER) {
         changed = c->gemm_cluster != (value != 0);
         c->gemm_cluster = value != 0;
@@ -1388,7 +1388,7 @@ MTP_API int mtp_get_option(mtp_ctx* c, int option, int32_t* value) {
         case MTP_OPT_SAMPLING: *value = c->sampling; break;
         case MTP_OPT_SEED: *value = (int32_t)c->sample_seed; break;
         case MTP_OPT_PERSISTENT: *value = c->use_persistent && c->sk_ok; break;
-        case MTP_OPT_PREFILL_TC: *value = c->use_attn_tc; break;
+        case MTP_OPT_PREFILL_TC: *value = c->attn_tc; break;
         case MTP_OPT_HEADS_FUSED: *value = c->heads_tc_ok && c->batched_ok ? c->use_heads_tc : 0; break;
         case MTP_OPT_GEMM_CLUSTER: *value = c->gemm_cluster; break;
         default: return fail(MTP_ERR_INVALID, "unknown option %d", option);
