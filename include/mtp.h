@@ -247,7 +247,9 @@ MTP_API int mtp_debug_lattice(mtp_ctx* ctx, int32_t* out_ids, float* out_logp, i
  *   MTP_OPT_PREFILL_TC   attention of prefill passes (mtp_prefill, mtp_prefill_pending): 1 = always in
  *                        tcgen05 tiles (128 prompt rows, 128-key items, S and P V accumulated in
  *                        TMEM); 0 = always by the kernel of the decode steps, in groups of 8 rows;
- *                        2 = tiles in passes of more than 304 rows, groups in smaller ones (default)
+ *                        2 = tiles where the groups are more than a wave of CTAs: 304 rows of one
+ *                        prompt with 16 attention heads, 1216 with 4, twice that where prompts are
+ *                        shorter than a tile (default)
  *   MTP_OPT_GEMM_CLUSTER 1 = the batched path's projections at up to 128 fed rows run as one
  *                        activation tile per weight tile, their K split over the CTAs of a cluster
  *                        (2 or 4) that sum the partial tiles in distributed shared memory, each

@@ -92,6 +92,7 @@ struct AttnArgs {
 };
 
 constexpr int ATTN_CTAS_PER_SM = 4;  // attn_kernel: 128 threads x at most 128 registers, ~54 KB of shared memory
+int attn_ctas_per_sm(int page_size);  // resident CTAs of attn_kernel
 // CTAs per head of a launch (AttnArgs::ctas), and the floats of its partials (ws_part)
 int attn_ctas_for(int groups, int n_heads, int page_size, int max_keys, int num_sms);
 bool attn_whole_groups(int groups, int n_heads, int page_size, int max_keys, int num_sms);  // AttnArgs::whole

@@ -326,20 +326,27 @@ int gemm_splits(const mtp_ctx* c, int n_w, int k, int ntiles) {
 
 int tile_index(int nt) { return nt == 32 ? 0 : (nt == 64 ? 1 : 2); }
 
+// Prefill attention in tiles of 128 rows, or in groups of 8.  A tile's chain of 128-key items is longer than a
+// group's of 64-key batches, which pays back once the groups are more than a wave of CTAs, twice that where a slot
+// has fewer rows than a tile (tiles of two slots go through both slots' keys).  Prefill of three layers in groups
+// and in tiles, us, one prompt, 16 heads: 304 rows 196 and 206, 512 rows 233 and 222; 12 heads: 400 rows 187 and
+// 199, 512 rows 208 and 201; 8 heads: 512 rows 174 and 185, 700 rows 201 and 201; 4 heads: 1000 rows 191 and 227,
+// 2000 rows 275 and 283.  16 heads, 4 prompts of 90 rows 306 and 348, 8 of 60 397 and 443, 16 of 100 853 and 789.
+bool prefill_in_tiles(const mtp_ctx* c, int rows, int slots) {
+    if (c->attn_tc != 2) return c->attn_tc == 1;
+    const long long wave = 8ll * attn_ctas_per_sm(c->cfg.page_size) * c->num_sms;  // rows x heads in groups of 8
+    return (long long)rows * c->cfg.n_attn_heads > (rows < 128 * slots ? 2 * wave : wave);
+}
+
 // The block stack over the M rows the embedding put in d_bx, as tensor-core
 // projections plus row-wise kernels; the final hidden rows stay in d_bx.
 // Attention groups: `groups` runs of rpg rows, each of one slot (decode:
 // slot b's fed rows b*n.., plan PLAN_DEVICE; prefill: 8 consecutive prompt
 // positions, plan PLAN_ROWS).  prefill_keys > 0: a prefill pass whose rows see
-// at most that many keys; its attention runs in tiles of 128 rows (tcgen05)
-// above PREFILL_TC_ROWS rows, or always or never by option.  A tile's chain of
-// 128-key items is longer than a group's of 64-key batches, which only enough
-// tiles pay back: whole prefills with the groups and with the tiles, ms, of one
-// prompt of 289 rows 0.70 and 0.75, of 320 0.78 and 0.75, of 448 0.86 and 0.82,
-// of two prompts of 160 0.80 and 0.78, of four of 122 0.87 and 0.79.
-constexpr int PREFILL_TC_ROWS = 304;
+// at most that many keys, of prefill_slots slots; its attention runs in tiles of
+// 128 rows (tcgen05) or in the groups, see prefill_in_tiles.
 int run_layers_batched(mtp_ctx* c, int M, int rpg, int groups, int plan, cudaStream_t s, bool pdl, Prof* prof,
-                       int prefill_keys = 0) {
+                       int prefill_keys = 0, int prefill_slots = 1) {
     const mtp_config& cf = c->cfg;
     const int d = cf.d_model, F = cf.d_ffn, H = cf.n_attn_heads, P = cf.page_size;
     // activation tiles: a weight tile is streamed once per activation tile.  32-row
@@ -416,12 +423,12 @@ int run_layers_batched(mtp_ctx* c, int M, int rpg, int groups, int plan, cudaStr
         at.rows_per_group = rpg; at.n_heads = H; at.page_size = P;
         at.groups = groups; at.rows = M;
         at.ctas = std::min(attn_ctas_for(groups, H, P, cf.max_ctx, c->num_sms), c->battn_ctas);
-        // prefill passes (up to PREFILL_TC_ROWS rows): 8 positions see few keys more than the 8 before them, a
+        // prefill passes in groups: 8 positions see few keys more than the 8 before them, a
         // CTA each (one prompt of 289: 14 vs 18.5 us per launch)
         at.whole = prefill_keys > 0 || attn_whole_groups(groups, H, P, cf.max_ctx, c->num_sms);
         at.plan = plan; at.seq_len = c->d_len; at.seq_new = c->d_npend; at.active = c->d_active; at.done = c->d_done;
         at.err = c->d_err;
-        if (prefill_keys > 0 && plan == PLAN_ROWS && (c->attn_tc == 1 || (c->attn_tc == 2 && M > PREFILL_TC_ROWS))) {
+        if (prefill_keys > 0 && plan == PLAN_ROWS && prefill_in_tiles(c, M, prefill_slots)) {
             // tiles of 128 rows; splits as many as the batched attention workspace holds (S = 1 uses none)
             const int tiles = attn_tc_tiles(M);
             at.n_splits = std::max(1, std::min(attn_tc_splits_for(tiles, H, prefill_keys, c->num_sms),
@@ -1524,10 +1531,15 @@ MTP_API int mtp_prefill_pending(mtp_ctx* c) {
     int passes = 0;
     while (lane_pending(c)) {
         long long want = 0;  // rows the admitted slots still need (whole groups): a pass has no empty tail
-        for (int left : c->h_prompt_left) want += left > 0 ? (left + 7) / 8 * 8 : 0;
+        int slots = 0;       // about as many as have rows in this pass
+        for (int left : c->h_prompt_left)
+            if (left > 0 && want < cap) {
+                want += (left + 7) / 8 * 8;
+                ++slots;
+            }
         const int P = (int)std::min<long long>(cap, want);
         MTP_TRY(enqueue_lane_plan(c, 0, P, 8, s, c->use_pdl, nullptr));
-        MTP_TRY(run_layers_batched(c, P, 8, P / 8, PLAN_ROWS, s, c->use_pdl, nullptr, cf.max_ctx));
+        MTP_TRY(run_layers_batched(c, P, 8, P / 8, PLAN_ROWS, s, c->use_pdl, nullptr, cf.max_ctx, slots));
         Prof* prof = nullptr;
         LAUNCH(MTP_K_SAVE, launch_save_last(c->d_bx, c->d_row_seq, c->d_row_last, c->d_h_last, cf.d_model, P, nullptr, s,
                                             c->use_pdl));
