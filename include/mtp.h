@@ -111,7 +111,10 @@ typedef struct mtp_ctx mtp_ctx;
  * (the AR decoder theta_AR of Eq. 1) with the n MTP heads of Sec. III-B and
  * the transition matrix Q of Sec. III-C: validates config and blob, copies
  * the weights to the device (the caller keeps the blob), allocates the KV
- * page pool and all step buffers.  `cuda_stream` is a cudaStream_t
+ * page pool and all step buffers, and for bf16 models buffers of prefill passes
+ * of up to 96 rows per SM and no more than max_batch * max_ctx (28 KB a row at
+ * d_model 1024, d_ffn 4096; never more than a quarter of the memory that is
+ * free by then: passes are shorter instead).  `cuda_stream` is a cudaStream_t
  * (NULL = legacy default stream) used by every later call on the context.
  * Errors: MTP_ERR_INVALID (config), MTP_ERR_WEIGHTS (blob), MTP_ERR_CUDA. */
 MTP_API int mtp_create(const mtp_config* config, const void* weights_blob, size_t blob_bytes,

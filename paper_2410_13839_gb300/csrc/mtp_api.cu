@@ -128,7 +128,7 @@ struct mtp_ctx {
     // batched path (bf16 weights; more fed rows than one fused pass takes): tensor-core
     // projections over all rows of a step, row-wise glue kernels, split-KV attention
     bool use_batched = true, batched_ok = false;
-    int bm_max = 0;  // rows of the batched buffers (batched_rows)
+    int bm_max = 0;  // rows of the batched buffers (batched_rows, or fewer where memory is short)
     uint16_t* d_w2p = nullptr;  // W2 [layers][d][F] as stored in the blob (the fused kernels keep it transposed)
     float *d_bx = nullptr, *d_bq = nullptr;
     float* d_bws = nullptr;  // attention split partials
@@ -549,19 +549,31 @@ int launch_step_pass(mtp_ctx* c, int rows, int rpg, int seq_base, cudaStream_t s
 // Rows of the batched buffers: a decode step's (every slot's fed rows plus a prefill lane of up
 // to PREFILL_ROWS prompt rows), and for bf16 models a whole prefill pass: as many prompt rows as
 // the slots can hold, up to PREFILL_PASS_ROWS_PER_SM per SM (whole groups of 8).
+int step_rows(const mtp_ctx* c) { return c->cfg.max_batch * c->cfg.n_heads_max + PREFILL_ROWS; }
 int batched_rows(const mtp_ctx* c) {
     const mtp_config& cf = c->cfg;
-    const long long step = (long long)cf.max_batch * cf.n_heads_max + PREFILL_ROWS;
-    if (c->wbytes != 2) return (int)step;
+    if (c->wbytes != 2) return step_rows(c);
     const long long prompts = ((long long)cf.max_batch * cf.max_ctx + 7) / 8 * 8;
-    return (int)std::max(step, std::min<long long>(prompts, PREFILL_PASS_ROWS_PER_SM * c->num_sms / 8 * 8));
+    return (int)std::max<long long>(step_rows(c), std::min<long long>(prompts, PREFILL_PASS_ROWS_PER_SM * c->num_sms / 8 * 8));
 }
 
 // Buffers and tensor maps of the batched path (bf16 weights only).
 int setup_batched(mtp_ctx* c) {
     const mtp_config& cf = c->cfg;
-    const int d = cf.d_model, F = cf.d_ffn, H = cf.n_attn_heads, P = cf.page_size;
+    const int d = cf.d_model, F = cf.d_ffn, H = cf.n_attn_heads;
     if (c->wbytes != 2 || !c->d_w2p) return MTP_OK;
+    {  // attention workspace: one wave's partials, and those of a tensor-core prefill pass of few tiles
+        c->battn_ctas = std::max(1, ATTN_CTAS_PER_SM * c->num_sms / H);
+        c->battn_ws_floats = std::max(attn_workspace_floats(H, c->battn_ctas), attn_tc_workspace_floats(4, H, 2));
+        MTP_TRY(c->alloc(&c->d_bws, c->battn_ws_floats));
+        MTP_TRY(c->alloc(&c->d_bwc, attn_counters(c->num_sms)));
+    }
+    // longer prefill passes are for speed only (28 KB a row at d = 1024, 400 MB at most): they take a quarter of
+    // the memory that is left, and a device that is nearly full gets shorter ones
+    size_t left = 0, total = 0;
+    CUDA_TRY(cudaMemGetInfo(&left, &total));
+    const size_t row_bytes = (size_t)d * 2 * sizeof(float) + (size_t)(d + F) * 2 * sizeof(uint16_t);
+    c->bm_max = std::max(step_rows(c), (int)std::min<size_t>((size_t)c->bm_max, left / 4 / row_bytes / 8 * 8));
     const size_t M = (size_t)c->bm_max;
     MTP_TRY(c->alloc(&c->d_bx, M * d));
     MTP_TRY(c->alloc(&c->d_bq, M * d));
@@ -574,12 +586,6 @@ int setup_batched(mtp_ctx* c) {
     c->d_alo = reinterpret_cast<__nv_bfloat16*>(alo);
     c->d_uhi = reinterpret_cast<__nv_bfloat16*>(uhi);
     c->d_ulo = reinterpret_cast<__nv_bfloat16*>(ulo);
-    {  // attention workspace: one wave's partials, and those of a tensor-core prefill pass of few tiles
-        c->battn_ctas = std::max(1, ATTN_CTAS_PER_SM * c->num_sms / H);
-        c->battn_ws_floats = std::max(attn_workspace_floats(H, c->battn_ctas), attn_tc_workspace_floats(4, H, 2));
-        MTP_TRY(c->alloc(&c->d_bws, c->battn_ws_floats));
-        MTP_TRY(c->alloc(&c->d_bwc, attn_counters(c->num_sms)));
-    }
     c->lmaps.resize(cf.layers);
     int bad = 0;
     for (int l = 0; l < cf.layers; ++l) {
