@@ -46,6 +46,9 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
+#include <mutex>
+#include <utility>
 
 #include "common.cuh"
 #include "kernels.cuh"
@@ -557,6 +560,37 @@ float normal_upper_quantile(double p) {
     return (float)(0.5 * (lo + hi));
 }
 
+// Clusters that are resident at once with the long ring, one CTA per SM (15 on a GB300 of 152 SMs: clusters stay
+// within a GPC), asked once per kernel and device.
+static cudaError_t heads_tc_clusters(const void* kern, int* fit) {
+    static std::mutex mu;
+    static std::map<std::pair<const void*, int>, int> known;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mu);
+    auto it = known.find({kern, dev});
+    if (it == known.end()) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(HT_SLICES);
+        cfg.blockDim = dim3(HT_THREADS);
+        cfg.dynamicSmemBytes = HT_MAX_STAGES * HT_STAGE + 1024;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = HT_SLICES;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
+        if (e != cudaSuccess) return e;
+        it = known.emplace(std::make_pair(kern, dev), n).first;
+    }
+    *fit = it->second;
+    return cudaSuccess;
+}
+
 cudaError_t launch_heads_tc(const HeadsTc& g0, cudaStream_t s, bool pdl) {
     HeadsTc g = g0;
     HeadsTcArgs& a = g.args;
@@ -576,12 +610,14 @@ cudaError_t launch_heads_tc(const HeadsTc& g0, cudaStream_t s, bool pdl) {
         kern = reinterpret_cast<const void*>(heads_tc_kernel<16>);
     else
         kern = reinterpret_cast<const void*>(heads_tc_kernel<32>);
-    // Clusters of 8 at one CTA per SM: 15 fit this GPU at once; beyond, two CTAs per SM with half the ring
-    // each
-    a.stages = (a.m + HT_M - 1) / HT_M * a.n <= 15 ? HT_MAX_STAGES : HT_STAGES;
-    const size_t smem = a.stages * HT_STAGE + 1024;
     cudaError_t e = ensure_kernel_smem(kern, HT_MAX_STAGES * HT_STAGE + 1024);
     if (e != cudaSuccess) return e;
+    // as many clusters as fit the GPU at one CTA per SM take the long ring; more share the SMs, two CTAs with half
+    // the ring each
+    int fit = 0;
+    if ((e = heads_tc_clusters(kern, &fit)) != cudaSuccess) return e;
+    a.stages = (a.m + HT_M - 1) / HT_M * a.n <= fit ? HT_MAX_STAGES : HT_STAGES;
+    const size_t smem = a.stages * HT_STAGE + 1024;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(HT_SLICES, a.n, (a.m + HT_M - 1) / HT_M);
     cfg.blockDim = dim3(HT_THREADS);
