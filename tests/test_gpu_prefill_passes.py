@@ -1,7 +1,7 @@
 """Prefill passes (Sec. III-A: the prompt runs through the blocks as one sequence)
 against the oracle at the sizes where a pass can go wrong: fewer rows than an
 attention group, the edges of the 128-row tiles, and prompts or batches of
-prompts just below, at and past the rows one pass holds (96 per SM: 14592)."""
+prompts just below, at and past the rows one pass holds (96 per SM)."""
 import copy
 
 import numpy as np
@@ -32,15 +32,23 @@ def test_one_prompt(length):
         dec.close()
 
 
-@pytest.mark.parametrize("lengths,passes", [
-    ([5, 130, 61], 1),
-    ([700, 1300, 900, 1100, 500, 33], 1),
-    ([1024] * 14 + [248, 8], 1),          # exactly one pass of 14592 rows
-    ([1024] * 14 + [248, 9], 2),          # one prompt row left for the second pass
-    ([900, 333] * 14, 2),                 # a prompt cut by the end of the pass
+def _lengths(kind, rows):
+    """Prompt lengths around the `rows` rows of a pass (a multiple of 8; prompts take whole groups of 8)."""
+    if kind in ("one pass", "a row more"):   # full, and one prompt row left for the second pass
+        rest = rows % 1024 or 1024
+        return [1024] * ((rows - rest) // 1024) + [rest - 8, 8 if kind == "one pass" else 9]
+    if kind == "cut":                        # a prompt cut by the end of the pass
+        return [900, 333] * (rows // (904 + 336) + 3)
+    return kind
+
+
+@pytest.mark.parametrize("kind,passes", [
+    ([5, 130, 61], 1), ([700, 1300, 900, 1100, 500, 33], 1), ("one pass", 1), ("a row more", 2), ("cut", 2),
 ])
-def test_admitted_prompts(lengths, passes):
+def test_admitted_prompts(kind, passes):
+    torch = pytest.importorskip("torch")
     mtp = lib_module()
+    lengths = _lengths(kind, 96 * torch.cuda.get_device_properties(0).multi_processor_count)
     prompts = [synth.make_prompt(320 + b, t // 4, t - t // 4, MODEL.phone_vocab) for b, t in enumerate(lengths)]
     dec, w = decoder(MODEL, max_batch=len(lengths), max_ctx=max(lengths) + 32)
     try:

@@ -62,14 +62,25 @@ def test_tc_gemm_rejects_bad_shapes():
 PAIR_CASES = [  # many rows: 256 x 256 tiles of CTA pairs, where they are enough to fill the GPU
     (4096, 1024, 640, 1, 0),      # ragged last activation tile (half a tile)
     (3072, 1024, 1025, 1, 0),     # one row in the last tile
-    (1024, 1024, 2500, 4, 1),     # accumulate; ragged
+    (1024, 1024, 2500, 1, 1),     # accumulate; ragged
+    (1024, 4096, 2500, 4, 1),     # accumulate; ragged; the split K of the other kernel in one
     (1024, 4096, 4096, 8, 1),     # the largest row count, long K
-    (2560, 64, 2048, 1, 0),       # one k-chunk per tile
+    (9216, 64, 4096, 1, 0),       # one k-chunk per tile
     (4096, 192, 4000, 1, 0),      # fewer chunks than ring stages, several tiles per pair
-    (768, 256, 4096, 1, 0),       # the tiny model's q|k|v
+    (2048, 256, 4096, 1, 0),      # as many chunks as ring stages
 ]
+
+
+def _takes_pairs(n_w, k, m, splits, sms):
+    """The rule by which a product goes to the CTA pairs, restated: chunks of K per wave of tiles."""
+    chunks, up = k // 64, lambda a, b: -(-a // b)
+    here = up(n_w // 256 * up(m, 256), sms // 2) * chunks + 11
+    there = up(n_w // 128 * up(m, 128) * splits, sms) * (chunks // splits) + 4
+    return n_w % 256 == 0 and m > 128 and here < there
 
 
 @pytest.mark.parametrize("n_w,k,m,splits,accumulate", PAIR_CASES)
 def test_pair_gemm_matches_fp64_product(n_w, k, m, splits, accumulate):
+    torch = pytest.importorskip("torch")
+    assert _takes_pairs(n_w, k, m, splits, torch.cuda.get_device_properties(0).multi_processor_count)
     test_tc_gemm_matches_fp32_product(n_w, k, m, splits, accumulate)
