@@ -17,7 +17,7 @@
 // tiles: q|k|v 40 vs 74 us (1.29 PFLOP/s of MMA), W1 with GELU 59 vs 101,
 // W_o 22 vs 24, W2 52 vs 81.
 //
-// Per CTA, 12 or 20 warps: warp 0 copies (one lane, TMA into a four-stage ring; both
+// Per CTA, 20 warps: warp 0 copies (one lane, TMA into a four-stage ring; both
 // CTAs' copies complete on the leader's barrier), warp 1 of the leader issues
 // the MMAs (one lane), warps 4 and up read the accumulator back and write it out
 // (TMEM lane = weight row f, so a warp's store of one activation row is 32
@@ -122,8 +122,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
                         const __grid_constant__ CUtensorMap tal, const TcGemmArgs a, const int tiles_f,
                         const int tiles_n) {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ uint64_t full[TP_STAGES], empty[TP_STAGES], acc_full[2], acc_empty[2];
+    __shared__ uint64_t full[TP_STAGES], empty[TP_STAGES], acc_full[2], acc_empty[2], drained;
     __shared__ uint32_t tmem_base;
+    __shared__ int s_staged, s_failed;  // stages filled; a wait ran out
     __shared__ long long s_rowbase[2][TP_N];  // TC_QKV: element offset of the row's key row in its page
                                               // (-1: unreserved page, -2: row of no sequence)
     __shared__ int s_rowt[2][TP_N];           // TC_QKV: key row within the page; TC_GELU_PACK: row of a sequence
@@ -148,7 +149,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], 2 * TP_EPI_WARPS);  // the epilogue warps of both CTAs
         }
+        mbar_init(&drained, 1);
         fence_barrier_init();
+        s_staged = s_failed = 0;
     }
     tc_fence_before();
     __syncthreads();
@@ -194,13 +197,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
                 }
                 load_a(tile, c, s);
             }
+        s_staged = it;
+        if (!ok) s_failed = 1;
     } else if (tid == 32 && rank == 0) {  // ---- MMA issuer (the pair's leader) ----
         constexpr uint32_t IDESC = f16_idesc(2 * TP_F, TP_N, false);
         int it = 0;
         bool ok = true;
         for (int t = 0; t < work && ok; ++t) {
             const int b = t & 1, c0 = t % segs * TP_SEG, c1 = min(chunks, c0 + TP_SEG);
-            if (t >= 2 && !mbar_wait_cluster(&acc_empty[b], (uint32_t)(t / 2 - 1) & 1, a.err)) break;
+            if (t >= 2 && !mbar_wait_cluster(&acc_empty[b], (uint32_t)(t / 2 - 1) & 1, a.err)) {
+                ok = false;
+                break;
+            }
             tc_fence_after();
             const uint32_t acc = tmem + (uint32_t)b * TP_N;
             for (int c = c0; c < c1; ++c, ++it) {
@@ -221,6 +229,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
                 tc_commit2(&empty[s]);
             }
             if (ok) tc_commit2(&acc_full[b]);
+        }
+        if (!ok) {  // the MMAs that were issued end before TMEM is freed
+            s_failed = 1;
+            tc_commit2(&drained);
+            mbar_wait_cluster(&drained, 0, nullptr);
         }
     } else if (warp >= TP_EPI_WARP) {  // ---- epilogue ----
         const int et = tid - TP_EPI_WARP * 32, quarter = warp & 3, j0 = ((warp - TP_EPI_WARP) >> 2) * TP_COLS;
@@ -254,6 +267,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
             const int got_acc = lane == 0 ? mbar_wait_cluster(&acc_full[b], (uint32_t)(t / 2) & 1, a.err) : 1;
             ok = __all_sync(FULL_MASK, got_acc) != 0;
             if (!ok) {  // the row facts' barrier counts every epilogue warp: keep meeting it
+                s_failed = 1;
                 if (FACTS)
                     for (int rest = i + 1; rest < work / segs; ++rest) epi_barrier();
                 break;
@@ -286,6 +300,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
     // nothing signals a CTA that has left, and TMEM is freed once both are done with it
     tc_fence_before();
     __syncthreads();
+    // where a wait ran out, both CTAs' copies in flight land before the pair leaves (they complete on the leader)
+    if (s_failed && tid == 0 && rank == 0)
+        for (int j = max(0, s_staged - TP_STAGES); j < s_staged; ++j)
+            mbar_wait_cluster(&full[j % TP_STAGES], (uint32_t)(j / TP_STAGES) & 1, nullptr);
     cluster_arrive_release();
     cluster_wait();
     tc_fence_after();
