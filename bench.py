@@ -626,7 +626,7 @@ def run_ours(args):
                  "frac_of_nominal_8tbs": dec_bytes / (decode_ms / 1e3) / 1e9 / 8000.0}
     # decode: the persistent step kernel (or the embedding and 2 block kernels per layer), heads, selection
     per_decode_step = 3 if mtp.mtp_get_option(ctx, 9) else 3 + 2 * L
-    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    sms = torch.cuda.get_device_properties(local).multi_processor_count
     launches_per_step = _prefill_launches(N_PH + N_AC, L, sms) + decode_steps // args.steps * per_decode_step
 
     line = {"metric": METRIC, "value": value, "unit": "codec tokens/s", "n_gpus": world, "steps": args.steps,
