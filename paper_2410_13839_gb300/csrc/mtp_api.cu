@@ -423,9 +423,12 @@ int run_layers_batched(mtp_ctx* c, int M, int rpg, int groups, int plan, cudaStr
         at.rows_per_group = rpg; at.n_heads = H; at.page_size = P;
         at.groups = groups; at.rows = M;
         at.ctas = std::min(attn_ctas_for(groups, H, P, cf.max_ctx, c->num_sms), c->battn_ctas);
-        // prefill passes in groups: 8 positions see few keys more than the 8 before them, a
-        // CTA each (one prompt of 289: 14 vs 18.5 us per launch)
-        at.whole = prefill_keys > 0 || attn_whole_groups(groups, H, P, cf.max_ctx, c->num_sms);
+        // prefill passes in groups: 8 positions see few keys more than the 8 before them, a CTA each (one prompt of
+        // 289: 14 vs 18.5 us per launch).  So do the lane's rows where they are groups of one row, 128 of them beside
+        // the slots' own, and few heads make about a wave (4 heads, 8 to 96 slots: steps of 124 to 144 us instead of
+        // 141 to 153 at 300 keys, 164 instead of 166 at 1500; with 8 heads, 2 slots, 1500 keys 200 instead of 191).
+        at.whole = prefill_keys > 0 || attn_whole_groups(groups, H, P, cf.max_ctx, c->num_sms) ||
+                   (plan == PLAN_ROWS && rpg == 1 && H <= 4);
         at.plan = plan; at.seq_len = c->d_len; at.seq_new = c->d_npend; at.active = c->d_active; at.done = c->d_done;
         at.err = c->d_err;
         if (prefill_keys > 0 && plan == PLAN_ROWS && prefill_in_tiles(c, M, prefill_slots)) {
