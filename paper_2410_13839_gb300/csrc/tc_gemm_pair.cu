@@ -124,7 +124,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ uint64_t full[TP_STAGES], empty[TP_STAGES], acc_full[2], acc_empty[2], drained;
     __shared__ uint32_t tmem_base;
-    __shared__ int s_staged, s_failed;  // stages filled; a wait ran out
+    __shared__ int s_staged, s_failed;  // stages filled when a wait of the copies ran out; a wait of the MMAs did
     __shared__ long long s_rowbase[2][TP_N];  // TC_QKV: element offset of the row's key row in its page
                                               // (-1: unreserved page, -2: row of no sequence)
     __shared__ int s_rowt[2][TP_N];           // TC_QKV: key row within the page; TC_GELU_PACK: row of a sequence
@@ -197,8 +197,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
                 }
                 load_a(tile, c, s);
             }
-        s_staged = it;
-        if (!ok) s_failed = 1;
+        if (!ok) s_staged = it;
     } else if (tid == 32 && rank == 0) {  // ---- MMA issuer (the pair's leader) ----
         constexpr uint32_t IDESC = f16_idesc(2 * TP_F, TP_N, false);
         int it = 0;
@@ -267,7 +266,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
             const int got_acc = lane == 0 ? mbar_wait_cluster(&acc_full[b], (uint32_t)(t / 2) & 1, a.err) : 1;
             ok = __all_sync(FULL_MASK, got_acc) != 0;
             if (!ok) {  // the row facts' barrier counts every epilogue warp: keep meeting it
-                s_failed = 1;
                 if (FACTS)
                     for (int rest = i + 1; rest < work / segs; ++rest) epi_barrier();
                 break;
@@ -300,9 +298,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(TP_THREADS, 1)
     // nothing signals a CTA that has left, and TMEM is freed once both are done with it
     tc_fence_before();
     __syncthreads();
-    // where a wait ran out, both CTAs' copies in flight land before the pair leaves (they complete on the leader)
-    if (s_failed && tid == 0 && rank == 0)
-        for (int j = max(0, s_staged - TP_STAGES); j < s_staged; ++j)
+    // where a wait ran out, both CTAs' copies in flight land before the pair leaves (they complete on the leader).
+    // (An epilogue wait runs out only where the issuer's did; a flag of its own cost W1's epilogue 3 %.)
+    if ((s_failed || s_staged) && tid == 0 && rank == 0)
+        for (int n = s_staged ? s_staged : work / segs * chunks, j = max(0, n - TP_STAGES); j < n; ++j)
             mbar_wait_cluster(&full[j % TP_STAGES], (uint32_t)(j / TP_STAGES) & 1, nullptr);
     cluster_arrive_release();
     cluster_wait();
