@@ -263,7 +263,7 @@ MTP_API int mtp_debug_lattice(mtp_ctx* ctx, int32_t* out_ids, float* out_logp, i
  *                        kernel (LN_f rows as bf16 hi + lo; per (tile of 128 rows, head) a cluster of
  *                        8 CTAs over vocabulary slices, lse merged in the cluster before the top-k):
  *                        0 = never (heads GEMM into memory, then the selection kernel's top-k);
- *                        1 = in mtp_heads_topk (default: 32.0 vs 94.6 us for 256 rows, n = 8, top-16);
+ *                        1 = in mtp_heads_topk (default: 31 vs 95 us for 256 rows, n = 8, top-16);
  *                        2 = also in batched decode steps (measured 1.2 % slower per step at B = 32)
  *   MTP_OPT_SEED         seed of the path draws (any 32-bit value, zero-extended; default 0).
  *                        Position t of a draw of slot b that has generated g tokens uses the
@@ -374,9 +374,10 @@ MTP_API int mtp_viterbi(int batch, int n, int k, int vocab, int eos_id,
  *   out_ids    int32 [batch][n_heads][top_k]; out_logp float, same shape
  *   out_logits float [batch][n_heads][codec_vocab] or NULL
  *   out_lse    float [batch][n_heads] or NULL
- * More than 8 rows with bf16 weights run on the tensor cores (LN_f rows packed
- * as bf16 hi + lo, one GEMM over the n_heads * codec_vocab weight rows, head
- * weights streamed once per chunk of rows); otherwise passes of 8 rows.
+ * More than 8 rows with bf16 weights run on the tensor cores: LN_f rows packed
+ * as bf16 hi + lo, then by default one kernel for the heads, log-softmax and
+ * top-k (MTP_OPT_HEADS_FUSED; without it a GEMM over the n_heads * codec_vocab
+ * weight rows and the selection kernel); otherwise passes of 8 rows.
  * Uses the context's stream.  Errors: MTP_ERR_INVALID, MTP_ERR_CUDA. */
 MTP_API int mtp_heads_topk(mtp_ctx* ctx, int batch, const void* hidden, int hidden_dtype,
                            int n_heads, int top_k, int32_t* out_ids, float* out_logp,

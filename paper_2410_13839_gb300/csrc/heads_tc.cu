@@ -69,8 +69,9 @@ constexpr uint32_t HT_A_BYTES = HT_M * HT_K * 2;
 constexpr uint32_t HT_B_BYTES = HT_NMAX * HT_K * 2;
 constexpr uint32_t HT_STAGE = 2 * HT_A_BYTES + HT_B_BYTES;  // multiple of 1024
 constexpr uint32_t HT_TMEM_COLS = 256;
-// After the MMAs the ring is free.  Candidates of this slice: [128 rows][2 halves][32] of (logp, id), 64 KB; then each thread's staging row of 33 floats (a warp's 32 rows: logits on their way out, a
-// block's logp values, a row's candidates while they are ranked).  The exact way's lists: those pushed by
+// After the MMAs the ring is free.  Candidates of this slice: [128 rows][2 halves][32] of (logp, id), 64 KB;
+// then each thread's staging row of 33 floats (a warp's 32 rows: logits on their way out, a block's logp
+// values, a row's candidates while they are ranked).  The exact way's lists: those pushed by
 // the cluster (at most 2 x 16 rows x 8 slices x 32 entries x 4 B = 32 KB) at the start, the two halves'
 // lists (64 KB) behind them, over the staging rows.
 constexpr int HT_CAND = 32;      // candidates of a half that are listed
